@@ -43,8 +43,13 @@ int esp::choose_splits(const esp_ctx *c, const TileView &v, int n, int prec)
     // wave leaves little idle time (measured best at ~50 CTAs per SM)
     int target = 48 * c->num_sms;
     int s = (target + blocks - 1) / blocks;
+    // at most 64 partial sums per position where the blocks alone fill the GPU;
+    // with few blocks as many as give every SM eight CTAs (1,001 positions
+    // against 894 tiles: 128 CTAs of 64 splits left 24 SMs idle and the others
+    // with one CTA)
+    const int fill = (8 * c->num_sms + blocks - 1) / blocks;
+    s = std::min(s, std::max(64, fill));
     s = std::min(s, std::max(v.n_tiles, 1));
-    s = std::min(s, 64);
     return std::max(s, 1);
 }
 

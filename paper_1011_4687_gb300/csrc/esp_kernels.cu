@@ -6,6 +6,8 @@
 #include "esp_potential.cuh"
 #include "esp_shapes.h"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 namespace esp {
@@ -60,65 +62,55 @@ __device__ __forceinline__ int sort_cell(const double *__restrict__ pos, int i, 
     return key;
 }
 
-// per-block histogram of the cells of positions [b chunk, (b + 1) chunk)
-__global__ void __launch_bounds__(kSortThreads) sort_count_kernel(const double *__restrict__ pos, int n, double cx,
-                                                                  double cy, double cz, int chunk,
-                                                                  int *__restrict__ counts)
+// The cell of every position.  Its own kernel over the whole GPU: at FP64's
+// rate the cells of 65,536 positions take 2 us on 152 SMs and 30 us on the
+// eight of the sort below.
+__global__ void sort_key_kernel(const double *__restrict__ pos, int n, double cx, double cy, double cz,
+                                int *__restrict__ key)
 {
-    __shared__ int h[kSortCells];
-    for (int k = threadIdx.x; k < kSortCells; k += kSortThreads)
-        h[k] = 0;
-    __syncthreads();
-    const int beg = blockIdx.x * chunk, end = min(n, beg + chunk);
-    for (int i = beg + threadIdx.x; i < end; i += kSortThreads)
-        atomicAdd(&h[sort_cell(pos, i, cx, cy, cz)], 1);
-    __syncthreads();
-    for (int k = threadIdx.x; k < kSortCells; k += kSortThreads)
-        counts[(size_t)k * gridDim.x + blockIdx.x] = h[k];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n)
+        key[i] = sort_cell(pos, i, cx, cy, cz);
 }
 
-// exclusive scan of counts[cell][block] (cell-major) in place, one CTA
-__global__ void __launch_bounds__(1024) sort_scan_kernel(int *__restrict__ counts, int m)
+__device__ __forceinline__ int warp_scan(int v, int lane)
 {
-    __shared__ int part[1024];
-    const int t = threadIdx.x, per = (m + 1023) / 1024;
-    const int beg = min(m, t * per), end = min(m, beg + per);
-    int s = 0;
-    for (int i = beg; i < end; ++i)
-        s += counts[i];
-    part[t] = s;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-        const int v = t >= o ? part[t - o] : 0;
-        __syncthreads();
-        part[t] += v;
-        __syncthreads();
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, v, o);
+        v += lane >= o ? x : 0;
     }
-    int run = part[t] - s;
-    for (int i = beg; i < end; ++i) {
-        const int c = counts[i];
-        counts[i] = run;
-        run += c;
-    }
+    return v;
 }
 
-// stable scatter: slot_of[i] and perm[slot] = i
-__global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const double *__restrict__ pos, int n, double cx,
-                                                                    double cy, double cz, int chunk,
-                                                                    const int *__restrict__ offs,
-                                                                    int *__restrict__ slot_of, int *__restrict__ perm)
+// Exclusive scan over the CTA of one value per thread (kSortThreads threads);
+// part holds one int per warp.
+__device__ __forceinline__ int cta_scan(int v, int *part)
 {
-    __shared__ int run[kSortCells];
-    for (int k = threadIdx.x; k < kSortCells; k += kSortThreads)
-        run[k] = offs[(size_t)k * gridDim.x + blockIdx.x];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int inc = warp_scan(v, lane);
+    if (lane == 31)
+        part[warp] = inc;
     __syncthreads();
+    if (warp == 0) {
+        const int p = part[lane];
+        part[lane] = warp_scan(p, lane) - p;
+    }
+    __syncthreads();
+    return part[warp] + inc - v;
+}
+
+// Stable scatter of positions [beg, end) by their cells key_slot[i], which the
+// slots replace; run[c] is the next slot of cell c for this CTA.
+__device__ __forceinline__ void cta_scatter(int *__restrict__ key_slot, int *__restrict__ perm, int beg, int end,
+                                            int *run)
+{
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    const int beg = blockIdx.x * chunk, end = min(n, beg + chunk);
     for (int base = beg; base < end; base += kSortThreads) {
         const int i = base + threadIdx.x;
         const bool valid = i < end;
-        const int key = valid ? sort_cell(pos, i, cx, cy, cz) : -1 - lane; // unique dummy keys
+        const int key = valid ? key_slot[i] : -1 - lane; // unique dummy keys
         const unsigned mask = __match_any_sync(0xffffffffu, key);
         const int rank = __popc(mask & lt);
         for (int w = 0; w < kSortThreads / 32; ++w) { // warps in order: ties keep the input order
@@ -129,12 +121,66 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const double
                 if (leader)
                     run[key] = b0 + __popc(mask);
                 if (valid) {
-                    slot_of[i] = b0 + rank;
+                    key_slot[i] = b0 + rank;
                     perm[b0 + rank] = i;
                 }
             }
             __syncthreads();
         }
+    }
+}
+
+// The order of all positions in one launch: a cluster of kSortCtas CTAs, each
+// with the histogram of its contiguous part of the positions in shared memory;
+// every CTA reads the others' histograms (distributed shared memory) for its
+// own first slot in each cell.  (A histogram pass over up to 256 blocks, a scan
+// of cells x blocks by one CTA and a scatter took 50 us for 10,000 positions
+// and 257 us for 65,536, most of it the scan.)
+__global__ void __cluster_dims__(kSortCtas, 1, 1) __launch_bounds__(kSortThreads)
+    sort_cluster_kernel(int *__restrict__ key_slot, int n, int *__restrict__ perm)
+{
+    __shared__ __align__(16) int hist[kSortCells];
+    __shared__ __align__(16) int run[kSortCells];
+    __shared__ int part[32];
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = int(cl.block_rank()), t = threadIdx.x;
+    const int chunk = (n + kSortCtas - 1) / kSortCtas;
+    const int beg = min(n, rank * chunk), end = min(n, beg + chunk);
+    constexpr int per = kSortCells / kSortThreads;
+    static_assert(per == 4, "one int4 of cells per thread");
+    reinterpret_cast<int4 *>(hist)[t] = make_int4(0, 0, 0, 0);
+    __syncthreads();
+    for (int i = beg + t; i < end; i += kSortThreads)
+        atomicAdd(&hist[key_slot[i]], 1);
+    cl.sync();
+    int4 before = make_int4(0, 0, 0, 0), all = make_int4(0, 0, 0, 0);
+#pragma unroll
+    for (int r = 0; r < kSortCtas; ++r) {
+        const int4 h = reinterpret_cast<const int4 *>(cl.map_shared_rank(hist, r))[t];
+        all.x += h.x, all.y += h.y, all.z += h.z, all.w += h.w;
+        if (r < rank)
+            before.x += h.x, before.y += h.y, before.z += h.z, before.w += h.w;
+    }
+    const int first = cta_scan(all.x + all.y + all.z + all.w, part);
+    int4 o;
+    o.x = first + before.x;
+    o.y = first + all.x + before.y;
+    o.z = first + all.x + all.y + before.z;
+    o.w = first + all.x + all.y + all.z + before.w;
+    reinterpret_cast<int4 *>(run)[t] = o;
+    cl.sync(); // (also: no CTA leaves while another still reads its histogram)
+    cta_scatter(key_slot, perm, beg, end, run);
+}
+
+__global__ void batch_key_kernel(const BatchHeader *__restrict__ hdr, const SysDesc *__restrict__ sys)
+{
+    const int total = hdr->n_pos_total, n_sys = hdr->n_sys;
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < total; g += gridDim.x * blockDim.x) {
+        const SysDesc &d = sys[find_sys(sys, n_sys, g, false)];
+        const int i = g - d.pos_begin;
+        if (d.sorted)
+            d.slot_of[i] = sort_cell(d.pos_in, i, d.qm[0], d.qm[1], d.qm[2]);
     }
 }
 
@@ -174,73 +220,29 @@ __global__ void batch_reduce_kernel(const BatchHeader *__restrict__ hdr, const S
     }
 }
 
-// The spatial order of every sorted system of a batch, one CTA per system
-// (histogram, scan and stable scatter as above, all in shared memory).
-constexpr int kBatchSortThreads = 1024;
-
-__global__ void __launch_bounds__(kBatchSortThreads) batch_sort_kernel(const BatchHeader *__restrict__ hdr,
-                                                                       const SysDesc *__restrict__ sys)
+// The spatial order of every sorted system of a batch, one CTA per system:
+// histogram, scan and stable scatter as above, in its own shared memory.
+__global__ void __launch_bounds__(kSortThreads) batch_sort_kernel(const BatchHeader *__restrict__ hdr,
+                                                                  const SysDesc *__restrict__ sys)
 {
-    __shared__ int h[kSortCells];
-    __shared__ int part[kBatchSortThreads];
+    __shared__ __align__(16) int h[kSortCells];
+    __shared__ int part[32];
     if ((int)blockIdx.x >= hdr->n_sys)
         return;
     const SysDesc &d = sys[blockIdx.x];
     if (!d.sorted)
         return;
     const int n = d.n_pos, t = threadIdx.x;
-    for (int k = t; k < kSortCells; k += kBatchSortThreads)
-        h[k] = 0;
+    reinterpret_cast<int4 *>(h)[t] = make_int4(0, 0, 0, 0);
     __syncthreads();
-    for (int i = t; i < n; i += kBatchSortThreads)
-        atomicAdd(&h[sort_cell(d.pos_in, i, d.qm[0], d.qm[1], d.qm[2])], 1);
+    for (int i = t; i < n; i += kSortThreads)
+        atomicAdd(&h[d.slot_of[i]], 1);
     __syncthreads();
-    // exclusive scan: each thread four consecutive cells, then the threads in order
-    constexpr int per = kSortCells / kBatchSortThreads;
-    int v[per], sum = 0;
-#pragma unroll
-    for (int k = 0; k < per; ++k) {
-        v[k] = h[per * t + k];
-        sum += v[k];
-    }
-    part[t] = sum;
+    const int4 v = reinterpret_cast<const int4 *>(h)[t];
+    const int first = cta_scan(v.x + v.y + v.z + v.w, part);
+    reinterpret_cast<int4 *>(h)[t] = make_int4(first, first + v.x, first + v.x + v.y, first + v.x + v.y + v.z);
     __syncthreads();
-    for (int o = 1; o < kBatchSortThreads; o <<= 1) {
-        const int x = t >= o ? part[t - o] : 0;
-        __syncthreads();
-        part[t] += x;
-        __syncthreads();
-    }
-    int run = part[t] - sum;
-#pragma unroll
-    for (int k = 0; k < per; ++k) {
-        h[per * t + k] = run;
-        run += v[k];
-    }
-    __syncthreads();
-    const int lane = t & 31, warp = t >> 5;
-    const unsigned lt = (1u << lane) - 1u;
-    for (int base = 0; base < n; base += kBatchSortThreads) {
-        const int i = base + t;
-        const bool valid = i < n;
-        const int key = valid ? sort_cell(d.pos_in, i, d.qm[0], d.qm[1], d.qm[2]) : -1 - lane;
-        const unsigned mask = __match_any_sync(0xffffffffu, key);
-        const int rank = __popc(mask & lt);
-        for (int w = 0; w < kBatchSortThreads / 32; ++w) {
-            if (warp == w) {
-                const bool leader = valid && rank == 0;
-                int b0 = leader ? h[key] : 0;
-                b0 = __shfl_sync(0xffffffffu, b0, __ffs(mask) - 1);
-                if (leader)
-                    h[key] = b0 + __popc(mask);
-                if (valid) {
-                    d.slot_of[i] = b0 + rank;
-                    d.perm[b0 + rank] = i;
-                }
-            }
-            __syncthreads();
-        }
-    }
+    cta_scatter(d.slot_of, d.perm, 0, n, h);
 }
 
 // ---------------------------------------------------------------------------
@@ -412,28 +414,62 @@ __global__ void __launch_bounds__(kWideThreads) reduce_wide_kernel(const double 
         V[q] = s_s[0] + s_c[0];
 }
 
-// perm (optional): the input index of staged slot i
-__global__ void reduce_kernel(const double *__restrict__ partial, int n_splits, int n, double *__restrict__ V,
-                              const int *__restrict__ perm)
+// (s, c) += (s2, c2)
+__device__ __forceinline__ void two_sum_join(double &s, double &c, double s2, double c2)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n)
-        return;
-    double s = 0.0, c = 0.0;
-    for (int k = 0; k < n_splits; ++k)
-        two_sum_acc(s, c, partial[(size_t)k * n + i]);
-    V[perm ? perm[i] : i] = s + c;
+    two_sum_acc(s, c, s2);
+    c += c2;
 }
 
+// V of 32 positions per CTA: warp y sums the partials y, y + SLICES, ... of its
+// lanes' positions by TwoSum, then the slices are joined in a fixed order.
+// Bound by the latency of the FP64 additions: one thread per position took 25
+// us for 39 partials of 10,000 positions and 64 us for 57 of 65,536.
+// perm (optional): the input index of staged slot i
+template <int SLICES>
+__global__ void __launch_bounds__(32 * SLICES) reduce_kernel(const double *__restrict__ partial, int n_splits, int n,
+                                                              double *__restrict__ V, const int *__restrict__ perm)
+{
+    __shared__ double s_s[SLICES][32], s_c[SLICES][32];
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + x;
+    double s = 0.0, c = 0.0;
+    if (i < n) {
+#pragma unroll 4
+        for (int k = y; k < n_splits; k += SLICES)
+            two_sum_acc(s, c, partial[(size_t)k * n + i]);
+    }
+    s_s[y][x] = s;
+    s_c[y][x] = c;
+#pragma unroll
+    for (int o = SLICES / 2; o > 0; o >>= 1) {
+        __syncthreads();
+        if (y < o) {
+            two_sum_join(s, c, s_s[y + o][x], s_c[y + o][x]);
+            s_s[y][x] = s;
+            s_c[y][x] = c;
+        }
+    }
+    if (y == 0 && i < n)
+        V[perm ? perm[i] : i] = s + c;
+}
+
+// one warp per walker: its lanes' electrons by TwoSum, then the lanes in a fixed order
 __global__ void walker_kernel(const double *__restrict__ V, int n_walkers, int n_elec, double *__restrict__ E)
 {
-    int w = blockIdx.x * blockDim.x + threadIdx.x;
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (w >= n_walkers)
         return;
     double s = 0.0, c = 0.0;
-    for (int e = 0; e < n_elec; ++e)
+    for (int e = lane; e < n_elec; e += 32)
         two_sum_acc(s, c, -V[(size_t)w * n_elec + e]);
-    E[w] = s + c;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double s2 = __shfl_down_sync(0xffffffffu, s, o), c2 = __shfl_down_sync(0xffffffffu, c, o);
+        two_sum_join(s, c, s2, c2);
+    }
+    if (lane == 0)
+        E[w] = s + c;
 }
 
 } // namespace
@@ -463,26 +499,18 @@ cudaError_t launch_stage(const double *pos_in, int n, const double center[3], do
     return cudaGetLastError();
 }
 
-int sort_blocks(int n) { return std::max(1, std::min(256, (n + 2047) / 2048)); }
-
-size_t sort_scratch_ints(int n) { return (size_t)kSortCells * sort_blocks(n) + 2 * (size_t)n; }
+size_t sort_scratch_ints(int n) { return 2 * (size_t)n; }
 
 cudaError_t launch_sort(const double *pos_in, int n, const double center[3], int *scratch, int **slot_of, int **perm,
                         cudaStream_t s)
 {
-    const int B = sort_blocks(n), chunk = (n + B - 1) / B;
-    int *counts = scratch;
-    *slot_of = scratch + (size_t)kSortCells * B;
-    *perm = *slot_of + n;
-    sort_count_kernel<<<B, kSortThreads, 0, s>>>(pos_in, n, center[0], center[1], center[2], chunk, counts);
+    *slot_of = scratch;
+    *perm = scratch + n;
+    sort_key_kernel<<<(n + 127) / 128, 128, 0, s>>>(pos_in, n, center[0], center[1], center[2], *slot_of);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return e;
-    sort_scan_kernel<<<1, 1024, 0, s>>>(counts, kSortCells * B);
-    if ((e = cudaGetLastError()) != cudaSuccess)
-        return e;
-    sort_scatter_kernel<<<B, kSortThreads, 0, s>>>(pos_in, n, center[0], center[1], center[2], chunk, counts, *slot_of,
-                                                   *perm);
+    sort_cluster_kernel<<<kSortCtas, kSortThreads, 0, s>>>(*slot_of, n, *perm);
     return cudaGetLastError();
 }
 
@@ -512,9 +540,12 @@ cudaError_t launch_batch(int precision, const BatchHeader *hdr, const SysDesc *s
                          int num_sms, int max_pos_total, cudaStream_t s)
 {
     const int sgrid = std::max(1, std::min(4 * num_sms, (max_pos_total + 255) / 256));
-    batch_sort_kernel<<<std::max(1, max_sys), kBatchSortThreads, 0, s>>>(hdr, sys);
+    batch_key_kernel<<<sgrid, 256, 0, s>>>(hdr, sys);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
+        return e;
+    batch_sort_kernel<<<std::max(1, max_sys), kSortThreads, 0, s>>>(hdr, sys);
+    if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
     batch_stage_kernel<<<sgrid, 256, 0, s>>>(hdr, sys);
     e = cudaGetLastError();
@@ -570,7 +601,12 @@ cudaError_t launch_reduce(const double *partial, int n_splits, int n, double *V,
 {
     if (n <= 0)
         return cudaSuccess;
-    reduce_kernel<<<(n + 255) / 256, 256, 0, s>>>(partial, n_splits, n, V, perm);
+    const int grid = (n + 31) / 32;
+    // more slices where the partials are many and the positions few
+    if (n_splits > 64)
+        reduce_kernel<32><<<grid, 32 * 32, 0, s>>>(partial, n_splits, n, V, perm);
+    else
+        reduce_kernel<8><<<grid, 32 * 8, 0, s>>>(partial, n_splits, n, V, perm);
     return cudaGetLastError();
 }
 
@@ -578,7 +614,7 @@ cudaError_t launch_walkers(const double *V, int n_walkers, int n_elec, double *E
 {
     if (n_walkers <= 0)
         return cudaSuccess;
-    walker_kernel<<<(n_walkers + 127) / 128, 128, 0, s>>>(V, n_walkers, n_elec, E);
+    walker_kernel<<<(n_walkers + 3) / 4, 128, 0, s>>>(V, n_walkers, n_elec, E);
     return cudaGetLastError();
 }
 

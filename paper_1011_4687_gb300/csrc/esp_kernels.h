@@ -91,7 +91,8 @@ cudaError_t launch_stage(const double *pos_in, int n, const double center[3], do
 // and *perm[slot] its input index (both inside scratch).
 constexpr int kSortSide = 16;
 constexpr int kSortCells = kSortSide * kSortSide * kSortSide;
-constexpr int kSortThreads = 256;
+constexpr int kSortThreads = 1024;
+constexpr int kSortCtas = 8; // the cluster that orders one call's positions
 constexpr double kSortHalf = 8.0;
 constexpr int kSortMinPositions = 4096; // fewer: the order is not worth its three launches
 size_t sort_scratch_ints(int n);
