@@ -92,7 +92,8 @@ typedef struct {
 typedef enum {
     ESP_FP64 = 0,  /* every step in FP64: reference-accuracy path */
     ESP_FP32C = 1  /* bulk of the pair sum in FP32 with compensated accumulation;
-                      point charges and near (position, tile) blocks in FP64 */
+                      point charges and near (position, tile) blocks in pairs of
+                      FP32 numbers (48 bits) or FP64 */
 } esp_precision;
 
 typedef struct {
@@ -185,7 +186,7 @@ esp_status esp_eval_walkers(esp_ctx *ctx, const double *positions, int64_t n_wal
  *   V_out     [n]    device memory of the context's device, float64
  * Work is enqueued on the context's stream; the call returns without waiting.
  * The scratch (staged positions and per-split partial sums) lives in one
- * file-scope device array of fixed size inside the library, about 7 MiB for
+ * file-scope device array of fixed size inside the library, about 8.5 MiB for
  * ESP_NOALLOC_MAX_POSITIONS positions, which every GPU that loads the library
  * holds until the process exits.  Under CUDA's lazy module loading (the
  * default) the library's device module, and with it this array, is loaded on

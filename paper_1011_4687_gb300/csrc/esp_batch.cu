@@ -93,11 +93,16 @@ esp_status capture_graph(esp_batch *b)
     cudaError_t e2 = e1 == cudaSuccess ? cudaEventRecordWithFlags(b->ev_copied, s, cudaEventRecordExternal) : e1;
     cudaError_t e3 = e2 == cudaSuccess ? cudaMemsetAsync(b->counter.p, 0, sizeof(int), s) : e2;
     const esp_ctx *c0 = b->ctxs[0];
+    const float *boysdd = nullptr; // the same table in every context that has dd records
+    for (const esp_ctx *c : b->ctxs)
+        if (!boysdd)
+            boysdd = static_cast<const float *>(c->boysdd.p);
     cudaError_t e4 = e3 == cudaSuccess
                          ? launch_batch(b->precision, hdr, sys, int(b->ctxs.size()), static_cast<int *>(b->counter.p),
                                         1 << 30,
                                         static_cast<const float *>(c0->boys32.p),
-                                        static_cast<const double *>(c0->boys64.p), b->tile_cap, b->threads, b->ppt,
+                                        static_cast<const double *>(c0->boys64.p),
+                                        boysdd, b->tile_cap, b->threads, b->ppt,
                                         b->num_sms, 1 << 30, s)
                          : e3;
     cudaGraph_t g = nullptr;
@@ -152,7 +157,7 @@ esp_status batch_eval(esp_batch *b, const double *const *positions, const int64_
     // scratch capacity (staged positions + partial sums) per system
     cudaError_t e;
     for (int k = 0; k < ns; ++k) {
-        size_t need = size_t(n[k]) * (3 * sizeof(double) + 6 * sizeof(float)) + 256 +
+        size_t need = size_t(n[k]) * kStagedBytes + 256 +
                       size_t(n[k]) * size_t(splits[size_t(k)]) * sizeof(double) + 2 * size_t(n[k]) * sizeof(int);
         if ((e = b->scratch[size_t(k)].ensure(std::max<size_t>(need, 256))) != cudaSuccess)
             return cuda_fail(e, "allocating batched scratch");
@@ -174,21 +179,14 @@ esp_status batch_eval(esp_batch *b, const double *const *positions, const int64_
         d.tiles = static_cast<const TileMeta *>(c->tiles.p);
         d.rec32 = static_cast<const float *>(c->rec32.p);
         d.rec64 = static_cast<const double *>(c->rec64.p);
+        d.recdd = static_cast<const float *>(c->recdd.p);
+        d.dd_lim = dd_limit(c);
         d.pos_in = positions[k];
         d.V_out = V_out[k];
         const int nk = int(n[k]);
         char *base = static_cast<char *>(b->scratch[size_t(k)].p);
-        d.st.x64 = reinterpret_cast<double *>(base);
-        d.st.y64 = d.st.x64 + nk;
-        d.st.z64 = d.st.y64 + nk;
-        float *f = reinterpret_cast<float *>(d.st.z64 + nk);
-        d.st.xh = f;
-        d.st.yh = f + nk;
-        d.st.zh = f + 2 * nk;
-        d.st.xl = f + 3 * nk;
-        d.st.yl = f + 4 * nk;
-        d.st.zl = f + 5 * nk;
-        size_t off = (size_t(nk) * (3 * sizeof(double) + 6 * sizeof(float)) + 255) / 256 * 256;
+        d.st = staged_at(base, size_t(nk));
+        size_t off = (size_t(nk) * kStagedBytes + 255) / 256 * 256;
         d.partial = reinterpret_cast<double *>(base + off);
         // FP32C systems with many positions are staged in spatial order
         d.sorted = (b->precision == 1 && nk >= kSortMinPositions) ? 1 : 0;
@@ -204,7 +202,7 @@ esp_status batch_eval(esp_batch *b, const double *const *positions, const int64_
         d.blocks = blocks[size_t(k)];
         d.item_begin = item;
         d.pos_begin = pos;
-        d.near_r = float(c->opt.near_radius < 0.0 ? kDefaultNearRadius : c->opt.near_radius);
+        d.near_r = near_radius(c);
         item += d.blocks * d.splits;
         pos += nk;
     }

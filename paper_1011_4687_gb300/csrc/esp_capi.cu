@@ -53,54 +53,87 @@ int esp::choose_splits(const esp_ctx *c, const TileView &v, int n, int prec)
     return std::max(s, 1);
 }
 
-int esp::plan_splits(const esp_ctx *c, const TileView &v, int n, int prec, int max_splits, EvalArgs &a)
+int esp::view_precision(const esp_ctx *c, const TileView &v)
 {
-    const int total = std::max(1, std::min(choose_splits(c, v, n, prec), max_splits));
+    return c->opt.precision == ESP_FP64 || (v.n_tiles > 0 && v.n_tiles == v.n_point_tiles) ? 0 : 1;
+}
+
+int esp::plan_splits(const esp_ctx *c, const TileView &v, int n, int prec, int max_splits, EvalArgs &a, int &dd_splits)
+{
     a.n_tiles = v.n_tiles;
     a.tiles = v.tiles;
+    dd_splits = 0;
+    if (prec == 1 && v.n_dd > 0) // (with few partial sums allowed, at most a quarter of them)
+        dd_splits = std::max(1, std::min(dd_sum_splits(n, v.n_dd, c->num_sms), max_splits / 4));
+    const int total = std::max(1, std::min(choose_splits(c, v, n, prec), max_splits - dd_splits));
     a.n_splits = total;
     single_group(a);
-    if (prec == 0 || c->opt.pair_splits > 0 || v.n_groups <= 1 || v.n_groups > total)
-        return total;
+    // the dd kernel takes the point charges: the groups after theirs
+    const int g0 = prec == 1 && v.n_point_tiles > 0 && v.n_groups > 1 ? 1 : 0;
+    const int ng = v.n_groups - g0;
+    if (prec == 0 || c->opt.pair_splits > 0 || v.n_groups <= 1 || ng > total)
+        return dd_splits + total;
     double work = 0.0;
-    for (int g = 0; g < v.n_groups; ++g)
+    for (int g = g0; g < v.n_groups; ++g)
         work += v.grp_work[g];
     int S[kMaxTileGroups], sum = 0;
-    for (int g = 0; g < v.n_groups; ++g) {
+    for (int g = g0; g < v.n_groups; ++g) {
         const int tiles = v.grp_tile[g + 1] - v.grp_tile[g];
         const int want = int(std::lround(total * v.grp_work[g] / std::max(work, 1e-300)));
         S[g] = std::max(1, std::min(want, tiles));
         sum += S[g];
     }
     while (sum > total) { // give back from the group with the most splits
-        int big = 0;
-        for (int g = 1; g < v.n_groups; ++g)
+        int big = g0;
+        for (int g = g0 + 1; g < v.n_groups; ++g)
             if (S[g] > S[big])
                 big = g;
         --S[big];
         --sum;
     }
-    a.n_groups = v.n_groups;
+    a.n_groups = ng;
     a.grp_split[0] = 0;
-    for (int g = 0; g < v.n_groups; ++g) {
-        a.grp_tile[g] = v.grp_tile[g];
-        a.grp_split[g + 1] = a.grp_split[g] + S[g];
+    for (int g = 0; g < ng; ++g) {
+        a.grp_tile[g] = v.grp_tile[g0 + g];
+        a.grp_split[g + 1] = a.grp_split[g] + S[g0 + g];
     }
-    a.grp_tile[v.n_groups] = v.grp_tile[v.n_groups];
+    a.grp_tile[ng] = v.grp_tile[v.n_groups];
     a.n_splits = sum;
-    return sum;
+    return dd_splits + sum;
+}
+
+cudaError_t esp::launch_planned(const esp_ctx *c, const TileView &v, int prec, EvalArgs a, int dd_splits,
+                                cudaStream_t s)
+{
+    cudaError_t e = cudaSuccess;
+    if (dd_splits > 0 && (e = launch_dd_sum(a, v.dd_list, v.n_dd, dd_splits, s)) != cudaSuccess)
+        return e;
+    a.partial += size_t(dd_splits) * a.n_pos;
+    return launch_potential(prec, a, c->threads[prec], c->ppt[prec], s);
+}
+
+std::vector<int> esp::dd_tile_list(const std::vector<TileMeta> &T, bool near)
+{
+    std::vector<int> list;
+    for (size_t t = 0; t < T.size(); ++t)
+        if (T[t].cls == kClassPoint || (near && !is_point_class(T[t].cls) && T[t].vmax >= kNearVmax))
+            list.push_back(int(t));
+    return list;
 }
 
 void esp::set_tile_groups(const std::vector<TileMeta> &T, TileView &v)
 {
     // FP32 operations per evaluation by L (the kernel's algorithmic count) and
-    // an FP64 point charge, for the split of the work between groups
+    // an FP64 point charge (in pairs of FP32 numbers), for the split of the work between groups
     static const double kCost[kMaxL + 1] = {10.0, 26.0, 52.0, 95.0, 170.0};
-    const double kPointCost = 12.0, kPoint32Cost = 10.0;
+    const double kPointCost = 54.0, kPoint32Cost = 10.0;
     v.n_tiles = int(T.size());
     int64_t n_small = 0, n_all = 0;
     v.n_p32 = 0;
     v.p32_off = 0;
+    v.n_point_tiles = 0;
+    for (const TileMeta &m : T)
+        v.n_point_tiles += m.cls == kClassPoint;
     bool contiguous = true;
     for (const TileMeta &m : T) {
         n_all += m.n;
@@ -150,29 +183,12 @@ esp_status ensure_scratch(esp_ctx *c, int64_t n, int splits, bool host_io, int64
     cudaError_t e;
     if (host_io && (e = c->in.ensure(size_t(n) * 3 * sizeof(double))) != cudaSuccess)
         return cuda_fail(e, "allocating position staging");
-    if ((e = c->stage.ensure(size_t(n) * (3 * sizeof(double) + 6 * sizeof(float)) + 256)) != cudaSuccess)
+    if ((e = c->stage.ensure(size_t(n) * kStagedBytes + 256)) != cudaSuccess)
         return cuda_fail(e, "allocating staged positions");
     if ((e = c->partial.ensure(size_t(n) * splits * sizeof(double))) != cudaSuccess)
         return cuda_fail(e, "allocating partial sums");
     (void)n_walkers;
     return ESP_OK;
-}
-
-Staged staged_view(esp_ctx *c, int64_t n)
-{
-    char *b = static_cast<char *>(c->stage.p);
-    Staged st;
-    st.x64 = reinterpret_cast<double *>(b);
-    st.y64 = st.x64 + n;
-    st.z64 = st.y64 + n;
-    float *f = reinterpret_cast<float *>(st.z64 + n);
-    st.xh = f;
-    st.yh = f + n;
-    st.zh = f + 2 * n;
-    st.xl = f + 3 * n;
-    st.yl = f + 4 * n;
-    st.zl = f + 5 * n;
-    return st;
 }
 
 // The device part of an evaluation over the view's tiles, enqueued on the
@@ -189,7 +205,9 @@ esp_status pipeline(esp_ctx *c, const TileView &v, int prec, const double *d_pos
     // distributions take FP64 there)
     const bool small_n = v.n_tiles > 0 && (n <= kSmallNDistributions || (n <= kSmallN && v.point_heavy));
     EvalArgs a;
-    const int splits = small_n ? small_n_splits(v.n_tiles, c->num_sms, int(n)) : plan_splits(c, v, int(n), prec, 1 << 20, a);
+    int dd_splits = 0;
+    const int splits = small_n ? small_n_splits(v.n_tiles, c->num_sms, int(n))
+                               : plan_splits(c, v, int(n), prec, 1 << 20, a, dd_splits);
     esp_status st = ensure_scratch(c, n, splits, false, n_walkers);
     if (st != ESP_OK)
         return st;
@@ -200,7 +218,7 @@ esp_status pipeline(esp_ctx *c, const TileView &v, int prec, const double *d_pos
     const bool sorted = !small_n && prec == 1 && n >= kSortMinPositions;
     if (sorted && (e = c->sortbuf.ensure(sort_scratch_ints(int(n)) * sizeof(int))) != cudaSuccess)
         return cuda_fail(e, "allocating the position order");
-    Staged stg = staged_view(c, n);
+    const Staged stg = staged_at(c->stage.p, size_t(n));
     int *slot_of = nullptr, *perm = nullptr;
     if (sorted && (e = launch_sort(d_pos, int(n), c->opt.qm_center, static_cast<int *>(c->sortbuf.p), &slot_of, &perm,
                                    s)) != cudaSuccess)
@@ -217,8 +235,11 @@ esp_status pipeline(esp_ctx *c, const TileView &v, int prec, const double *d_pos
     a.rec64 = static_cast<const double *>(c->rec64.p);
     a.boys32 = static_cast<const float *>(c->boys32.p);
     a.boys64 = static_cast<const double *>(c->boys64.p);
+    a.recdd = static_cast<const float *>(c->recdd.p);
+    a.boysdd = static_cast<const float *>(c->boysdd.p);
+    a.dd_lim = dd_limit(c);
     a.partial = static_cast<double *>(c->partial.p);
-    a.near_r = float(c->opt.near_radius < 0.0 ? kDefaultNearRadius : c->opt.near_radius);
+    a.near_r = near_radius(c);
     if (timing && (e = cudaEventRecord(c->ev[1], s)) != cudaSuccess)
         return cuda_fail(e, "recording a timing event");
     if (v.n_tiles == 0) {
@@ -243,7 +264,7 @@ esp_status pipeline(esp_ctx *c, const TileView &v, int prec, const double *d_pos
         sa.partial = a.partial;
         if ((e = launch_small_n(sa, splits, dV, s)) != cudaSuccess)
             return cuda_fail(e, "launching the few-position kernels");
-    } else if ((e = launch_potential(prec, a, c->threads[prec], c->ppt[prec], s)) != cudaSuccess) {
+    } else if ((e = launch_planned(c, v, prec, a, dd_splits, s)) != cudaSuccess) {
         return cuda_fail(e, "launching the potential kernel");
     }
     if (timing && (e = cudaEventRecord(c->ev[2], s)) != cudaSuccess)
@@ -279,7 +300,7 @@ esp_status run_eval(esp_ctx *c, const double *positions, int64_t n, double *V_ou
         return fail(ESP_ERR_INVALID, "positions and outputs must all be host memory or all be device memory of "
                                      "device %d", c->device);
     const bool host_io = sp == Space::Host;
-    const int prec = c->opt.precision == ESP_FP64 ? 0 : 1;
+    const int prec = view_precision(c, c->full);
     cudaStream_t s = c->stream;
     cudaError_t e;
     if (host_io) {
@@ -353,6 +374,33 @@ cudaError_t upload(DevBuf &b, const std::vector<T> &v, int64_t &bytes)
     return cudaMemcpy(b.p, v.data(), n, cudaMemcpyHostToDevice);
 }
 
+// The dd records of the uploaded tiles, made on the device from the FP64
+// records.  A device without room for them keeps the FP64 code (the tiles are
+// uploaded again without their dd offsets).
+cudaError_t build_dd(esp_ctx *c, int64_t &bytes)
+{
+    cudaError_t e;
+    if (c->env.dd_floats == 0)
+        return cudaSuccess;
+    if ((e = c->recdd.ensure(size_t(c->env.dd_floats) * sizeof(float))) == cudaErrorMemoryAllocation &&
+        !fault("alloc")) {
+        cudaGetLastError();
+        for (TileMeta &m : c->env.tiles)
+            m.offdd = -1;
+        c->env.dd_floats = 0;
+        return cudaMemcpy(c->tiles.p, c->env.tiles.data(), c->env.tiles.size() * sizeof(TileMeta),
+                          cudaMemcpyHostToDevice);
+    }
+    if (e != cudaSuccess || (e = upload(c->boysdd, boys_table_dd(), bytes)) != cudaSuccess ||
+        (e = launch_dd_build(static_cast<const TileMeta *>(c->tiles.p), int(c->env.tiles.size()),
+                             static_cast<const double *>(c->rec64.p), c->env.coord_quantum,
+                             static_cast<float *>(c->recdd.p), c->stream)) != cudaSuccess)
+        return e;
+    bytes += int64_t(c->recdd.bytes);
+    // (other streams may use the context's records next: a batch, a server)
+    return cudaStreamSynchronize(c->stream);
+}
+
 void release_all(esp_ctx *c)
 {
     for (cudaEvent_t &ev : c->ev)
@@ -360,7 +408,7 @@ void release_all(esp_ctx *c)
             cudaEventDestroy(ev);
             ev = nullptr;
         }
-    DevBuf *bufs[] = {&c->tiles, &c->rec32, &c->rec64, &c->boys32, &c->boys64,
+    DevBuf *bufs[] = {&c->tiles, &c->rec32, &c->rec64, &c->boys32, &c->boys64, &c->recdd, &c->boysdd, &c->ddlist,
                       &c->in, &c->stage, &c->partial, &c->vout, &c->eout, &c->sortbuf};
     for (DevBuf *b : bufs)
         b->release();
@@ -382,7 +430,7 @@ double host_eval_f32c(const esp_ctx *c, const double *C)
     }
     float S[1] = {0.0f}, Cc[1] = {0.0f};
     double acc64[1] = {0.0};
-    const float near_r = float(c->opt.near_radius < 0.0 ? kDefaultNearRadius : c->opt.near_radius);
+    const float near_r = near_radius(c);
     for (const TileMeta &m : c->env.tiles) {
         if (m.cls == kClassPoint) {
             tile_points_f64<1>(c->env.rec64.data() + m.off64, m.n, c64, acc64);
@@ -565,17 +613,22 @@ esp_status esp_create(const esp_point_charge *charges, int64_t n_charges, const 
     }
     cudaError_t e = fault("upload") ? cudaErrorInvalidValue : cudaSuccess;
     int64_t bytes = 0;
+    const std::vector<int> ddlist = dd_tile_list(c->env.tiles, near_radius(c) > 0.0f);
     if (e != cudaSuccess || (e = upload(c->tiles, c->env.tiles, bytes)) != cudaSuccess ||
+        (e = upload(c->ddlist, ddlist, bytes)) != cudaSuccess ||
         (e = upload(c->rec32, c->env.rec32, bytes)) != cudaSuccess ||
         (e = upload(c->rec64, c->env.rec64, bytes)) != cudaSuccess ||
         (e = upload(c->boys32, boys_table32(), bytes)) != cudaSuccess ||
-        (e = upload(c->boys64, boys_table64(), bytes)) != cudaSuccess) {
+        (e = upload(c->boys64, boys_table64(), bytes)) != cudaSuccess ||
+        (e = build_dd(c, bytes)) != cudaSuccess) {
         release_all(c);
         delete c;
         return cuda_fail(e, "uploading the environment");
     }
     c->device_bytes = bytes;
     c->full.tiles = static_cast<const TileMeta *>(c->tiles.p);
+    c->full.dd_list = static_cast<const int *>(c->ddlist.p);
+    c->full.n_dd = int(ddlist.size());
     // keep a host copy of the records only while it is small (test hook use)
     if (c->env.rec64.size() * sizeof(double) > (size_t(256) << 20)) {
         c->host_copy = false;
@@ -801,7 +854,7 @@ namespace {
 
 constexpr int64_t kNoallocMaxPositions = ESP_NOALLOC_MAX_POSITIONS;
 constexpr int kNoallocMaxSplits = 8;
-constexpr size_t kNoallocStageBytes = size_t(kNoallocMaxPositions) * (3 * sizeof(double) + 6 * sizeof(float));
+constexpr size_t kNoallocStageBytes = size_t(kNoallocMaxPositions) * kStagedBytes;
 constexpr size_t kNoallocBytes = kNoallocStageBytes + size_t(kNoallocMaxPositions) * kNoallocMaxSplits * sizeof(double);
 
 } // namespace
@@ -855,21 +908,12 @@ extern "C" esp_status esp_eval_noalloc(esp_ctx *ctx, const double *positions, in
     esp_status st = noalloc_scratch(&base);
     if (st != ESP_OK)
         return st;
-    const int prec = ctx->opt.precision == ESP_FP64 ? 0 : 1;
+    const int prec = view_precision(ctx, ctx->full);
     EvalArgs a;
-    const int splits = plan_splits(ctx, ctx->full, int(n), prec, kNoallocMaxSplits, a);
+    int dd_splits = 0;
+    const int splits = plan_splits(ctx, ctx->full, int(n), prec, kNoallocMaxSplits, a, dd_splits);
     char *b = static_cast<char *>(base);
-    Staged stg;
-    stg.x64 = reinterpret_cast<double *>(b);
-    stg.y64 = stg.x64 + n;
-    stg.z64 = stg.y64 + n;
-    float *f = reinterpret_cast<float *>(stg.z64 + n);
-    stg.xh = f;
-    stg.yh = f + n;
-    stg.zh = f + 2 * n;
-    stg.xl = f + 3 * n;
-    stg.yl = f + 4 * n;
-    stg.zl = f + 5 * n;
+    const Staged stg = staged_at(b, size_t(n));
     double *partial = reinterpret_cast<double *>(b + kNoallocStageBytes);
     cudaStream_t s = ctx->stream;
     cudaError_t e;
@@ -888,9 +932,12 @@ extern "C" esp_status esp_eval_noalloc(esp_ctx *ctx, const double *positions, in
         a.rec64 = static_cast<const double *>(ctx->rec64.p);
         a.boys32 = static_cast<const float *>(ctx->boys32.p);
         a.boys64 = static_cast<const double *>(ctx->boys64.p);
+        a.recdd = static_cast<const float *>(ctx->recdd.p);
+        a.boysdd = static_cast<const float *>(ctx->boysdd.p);
+        a.dd_lim = dd_limit(ctx);
         a.partial = partial;
-        a.near_r = float(ctx->opt.near_radius < 0.0 ? kDefaultNearRadius : ctx->opt.near_radius);
-        if ((e = launch_potential(prec, a, ctx->threads[prec], ctx->ppt[prec], s)) != cudaSuccess)
+        a.near_r = near_radius(ctx);
+        if ((e = launch_planned(ctx, ctx->full, prec, a, dd_splits, s)) != cudaSuccess)
             return cuda_fail(e, "launching the potential kernel");
     }
     if ((e = launch_reduce(partial, splits, int(n), V_out, s)) != cudaSuccess)

@@ -146,6 +146,11 @@ struct TileView {
     int n_groups = 1;
     int grp_tile[kMaxTileGroups + 1] = {0, 0};
     double grp_work[kMaxTileGroups] = {0.0};
+    // tiles the FP32C evaluation leaves to the dd kernel, in device memory: FP64
+    // point charges (tile group 0 where there are any), then near-capable tiles
+    const int *dd_list = nullptr;
+    int n_dd = 0;
+    int n_point_tiles = 0;
     bool point_heavy = false; // >= 90 % of the entries are FP32 point charges
     // FP32 point charges of the view: their records are contiguous in rec32
     // (the builder emits those tiles one after the other)
@@ -156,6 +161,8 @@ struct TileView {
 // Tile groups of a host tile list (in device order); with fewer than one
 // group per class, or tiles not grouped by class, the plain deal.
 void set_tile_groups(const std::vector<TileMeta> &T, TileView &v);
+// the view's dd list (host copy; near: tiles may be evaluated near at all)
+std::vector<int> dd_tile_list(const std::vector<TileMeta> &T, bool near);
 
 } // namespace esp
 
@@ -166,7 +173,7 @@ struct esp_ctx {
     esp_options opt;
     esp::HostEnv env;        // host copy of the tiles (kept for esp_get_info / test hook)
     bool host_copy = true;
-    esp::DevBuf tiles, rec32, rec64, boys32, boys64;
+    esp::DevBuf tiles, rec32, rec64, boys32, boys64, recdd, boysdd, ddlist;
     esp::DevBuf in, stage, partial, vout, eout, sortbuf;
     std::atomic<int> busy{0};
     int64_t device_bytes = 0;
@@ -182,12 +189,27 @@ struct esp_ctx {
 
 namespace esp {
 inline bool valid_ctx(const esp_ctx *c) { return c && c->magic == 0x45535021u; }
+// FP32C: distance from a tile's sphere below which its block is near (0: none)
+inline float near_radius(const esp_ctx *c)
+{
+    return float(c->opt.near_radius < 0.0 ? kDefaultNearRadius : c->opt.near_radius);
+}
+// Largest |coordinate| of a position whose dd offsets are exact: centres are
+// below 2^22 q, so the hi words' difference stays below 2^24 q.
+inline float dd_limit(const esp_ctx *c) { return float(0x1p23 * c->env.coord_quantum); }
 // per-split count for n positions in precision prec (0 FP64, 1 FP32C)
 int choose_splits(const esp_ctx *c, const TileView &v, int n, int prec);
+// Precision of an evaluation of the view (0 FP64, 1 FP32C): FP64 point charges
+// alone stay FP64 under FP32C, where no FP32 sum hides the 48 bits of a dd term.
+int view_precision(const esp_ctx *c, const TileView &v);
 // Fills the deal of the view's tiles (n_splits and the tile groups) for n
-// positions, with at most max_splits partial sums; returns n_splits.  FP32C
-// deals each tile group to its own splits, in proportion to the group's work.
-int plan_splits(const esp_ctx *c, const TileView &v, int n, int prec, int max_splits, EvalArgs &a);
+// positions, with at most max_splits partial sums; returns their number.  FP32C
+// deals each tile group to its own splits, in proportion to the group's work;
+// its first dd_splits partial sums (set here) are the dd kernel's, and
+// a.n_splits counts the rest.
+int plan_splits(const esp_ctx *c, const TileView &v, int n, int prec, int max_splits, EvalArgs &a, int &dd_splits);
+// The potential kernels of a planned evaluation on stream s.
+cudaError_t launch_planned(const esp_ctx *c, const TileView &v, int prec, EvalArgs a, int dd_splits, cudaStream_t s);
 // Potentials of the view's tiles at n device positions into device V (the
 // main pipeline of esp_eval: spatial order for FP32C calls of >= 4,096
 // positions, staging, potential kernel, fixed-order reduction), enqueued on

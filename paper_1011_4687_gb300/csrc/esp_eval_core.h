@@ -368,7 +368,8 @@ ESP_HD void classify_tile(const TileMeta &m, float cx, float cy, float cz, float
                           bool &relq)
 {
     float ex = cx - m.cx, ey = cy - m.cy, ez = cz - m.cz;
-    float d = sqrtf(ex * ex + ey * ey + ez * ez) - m.rad;
+    // (explicit operations: two kernels have to agree on which blocks are near)
+    float d = sqrtf(esp_fma(ez, ez, esp_fma(ey, ey, ex * ex))) - m.rad;
     nearq = near_r > 0.0f && m.vmax >= kNearVmax && d < near_r;
     farq = nearq || (d > 0.0f && m.pmin * d * d >= kBoys32Tmax);
     relq = nearq || (farq && d >= kRelRatio * m.rad);

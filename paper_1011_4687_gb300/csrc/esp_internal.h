@@ -103,7 +103,7 @@ struct TileMeta {
     float pmin;       // smallest exponent p in the tile (0 for point tiles)
     float qabs;       // sum of absolute charge bounds of the tile's entries
     float vmax;       // largest |Q_d| 2 sqrt(p_d/pi) of an unmerged distribution (0 if none)
-    float pad1;
+    int32_t offdd;    // first word of the tile's dd records (esp_dd.h) in units of 4 floats; -1: none
 };
 static_assert(sizeof(TileMeta) == 48, "TileMeta layout");
 

@@ -3,6 +3,7 @@
 // The potential kernels themselves are templates in esp_potential.cuh; each
 // launch shape is compiled into its own object from esp_shape.cu, and the
 // dispatchers below pick the shape's launcher.
+#include "esp_dd.h"
 #include "esp_potential.cuh"
 #include "esp_shapes.h"
 
@@ -17,6 +18,27 @@ namespace {
 // ---------------------------------------------------------------------------
 // staging: recentre in FP64, split into FP32 hi + lo
 // ---------------------------------------------------------------------------
+// One recentred coordinate: its FP64 value, hi word on the environment's grid
+// q (see the pair builder), lo word, and the rest in two words (esp_dd.h).
+__device__ __forceinline__ void stage_coord(double x, double q, double *x64, float *xh, float *xl, float *xm,
+                                            float *xr)
+{
+    float h, m, r;
+    const double rest = dd_split3(x, q, h, m, r);
+    *x64 = x;
+    *xh = h;
+    *xl = (float)rest;
+    *xm = m;
+    *xr = r;
+}
+
+__device__ __forceinline__ void stage_position(const Staged &st, int j, double x, double y, double z, double q)
+{
+    stage_coord(x, q, st.x64 + j, st.xh + j, st.xl + j, st.xm + j, st.xr + j);
+    stage_coord(y, q, st.y64 + j, st.yh + j, st.yl + j, st.ym + j, st.yr + j);
+    stage_coord(z, q, st.z64 + j, st.zh + j, st.zl + j, st.zm + j, st.zr + j);
+}
+
 // slot_of (optional): the staged slot of position i (spatial order, below)
 __global__ void stage_kernel(const double *__restrict__ pos, int n, double cx, double cy, double cz, double q,
                              Staged st, const int *__restrict__ slot_of)
@@ -26,17 +48,7 @@ __global__ void stage_kernel(const double *__restrict__ pos, int n, double cx, d
         return;
     double x = pos[3 * i] - cx, y = pos[3 * i + 1] - cy, z = pos[3 * i + 2] - cz;
     const int j = slot_of ? slot_of[i] : i;
-    st.x64[j] = x;
-    st.y64[j] = y;
-    st.z64[j] = z;
-    // hi words on the environment's coordinate grid q (see the pair builder)
-    double xh = nearbyint(x / q) * q, yh = nearbyint(y / q) * q, zh = nearbyint(z / q) * q;
-    st.xh[j] = (float)xh;
-    st.yh[j] = (float)yh;
-    st.zh[j] = (float)zh;
-    st.xl[j] = (float)(x - xh);
-    st.yl[j] = (float)(y - yh);
-    st.zl[j] = (float)(z - zh);
+    stage_position(st, j, x, y, z, q);
 }
 
 // ---------------------------------------------------------------------------
@@ -192,17 +204,7 @@ __global__ void batch_stage_kernel(const BatchHeader *__restrict__ hdr, const Sy
         const int i = g - d.pos_begin;
         double x = d.pos_in[3 * i] - d.qm[0], y = d.pos_in[3 * i + 1] - d.qm[1], z = d.pos_in[3 * i + 2] - d.qm[2];
         const int j = d.sorted ? d.slot_of[i] : i;
-        d.st.x64[j] = x;
-        d.st.y64[j] = y;
-        d.st.z64[j] = z;
-        const double q = d.quantum;
-        double xh = nearbyint(x / q) * q, yh = nearbyint(y / q) * q, zh = nearbyint(z / q) * q;
-        d.st.xh[j] = (float)xh;
-        d.st.yh[j] = (float)yh;
-        d.st.zh[j] = (float)zh;
-        d.st.xl[j] = (float)(x - xh);
-        d.st.yl[j] = (float)(y - yh);
-        d.st.zl[j] = (float)(z - zh);
+        stage_position(d.st, j, x, y, z, d.quantum);
     }
 }
 
@@ -536,7 +538,8 @@ cudaError_t launch_potential(int precision, const EvalArgs &a, int threads, int 
 }
 
 cudaError_t launch_batch(int precision, const BatchHeader *hdr, const SysDesc *sys, int max_sys, int *counter,
-                         int max_items, const float *boys32, const double *boys64, int tile_cap, int threads, int ppt,
+                         int max_items, const float *boys32, const double *boys64, const float *boysdd, int tile_cap,
+                         int threads, int ppt,
                          int num_sms, int max_pos_total, cudaStream_t s)
 {
     const int sgrid = std::max(1, std::min(4 * num_sms, (max_pos_total + 255) / 256));
@@ -555,7 +558,8 @@ cudaError_t launch_batch(int precision, const BatchHeader *hdr, const SysDesc *s
     bool launched = false;
 #define ESP_BLAUNCH(NT, PPT, PR)                                                                                \
     if (!launched && threads == NT && ppt == PPT && precision == PR) {                                        \
-        e = launch_batch_shape<NT, PPT, PR>(hdr, sys, counter, max_items, boys32, boys64, tile_cap, num_sms, smem, s); \
+        e = launch_batch_shape<NT, PPT, PR>(hdr, sys, counter, max_items, boys32, boys64, boysdd, tile_cap, num_sms, smem, \
+                                            s); \
         launched = true;                                                                                      \
     }
     ESP_BATCH_SHAPES(ESP_BLAUNCH)

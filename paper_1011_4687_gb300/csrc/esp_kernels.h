@@ -13,7 +13,25 @@ namespace esp {
 struct Staged {
     double *x64, *y64, *z64;
     float *xh, *yh, *zh, *xl, *yl, *zl;
+    // the same rest x - hi in two words, mid on the grid 2^-23 q (esp_dd.h)
+    float *xm, *ym, *zm, *xr, *yr, *zr;
 };
+constexpr size_t kStagedBytes = 3 * sizeof(double) + 12 * sizeof(float); // per position
+// the arrays of n positions, one after the other from b (8-byte aligned)
+inline Staged staged_at(void *b, size_t n)
+{
+    Staged st;
+    st.x64 = static_cast<double *>(b);
+    st.y64 = st.x64 + n;
+    st.z64 = st.y64 + n;
+    float *f = reinterpret_cast<float *>(st.z64 + n);
+    float **p[] = {&st.xh, &st.yh, &st.zh, &st.xl, &st.yl, &st.zl, &st.xm, &st.ym, &st.zm, &st.xr, &st.yr, &st.zr};
+    for (float **q : p) {
+        *q = f;
+        f += n;
+    }
+    return st;
+}
 
 // FP32C tile groups: FP64 point charges, FP32 point charges, then one group
 // per L (long- and short-range tiles of that L together).
@@ -30,6 +48,9 @@ struct EvalArgs {
     const double *rec64;
     const float *boys32;
     const double *boys64;
+    const float *recdd;   // dd records (TileMeta::offdd)
+    const float *boysdd;  // Boys table of the dd general form
+    float dd_lim;         // |coordinate| up to which the dd words of a position are exact
     double *partial;  // [n_splits][n_pos], FP64
     float near_r;     // FP32C: FP64 re-evaluation radius around a tile's bounding sphere
     // FP32C deal by tile group: group g holds tiles [grp_tile[g], grp_tile[g+1])
@@ -56,6 +77,8 @@ struct SysDesc {
     const TileMeta *tiles;
     const float *rec32;
     const double *rec64;
+    const float *recdd;
+    float dd_lim;
     const double *pos_in; // [n_pos][3] device
     double *V_out;        // [n_pos] device
     double *partial;      // [splits][n_pos]
@@ -78,9 +101,19 @@ struct BatchHeader {
 // max_sys: the number of systems (one spatial-order CTA each, for systems marked sorted)
 cudaError_t launch_batch(int precision, const BatchHeader *hdr, const SysDesc *sys, int max_sys, int *counter,
                          int max_items,
-                         const float *boys32, const double *boys64, int tile_cap, int threads, int ppt,
+                         const float *boys32, const double *boys64, const float *boysdd, int tile_cap, int threads,
+                         int ppt,
                          int num_sms, int max_pos_total, cudaStream_t s);
 bool batch_shape_supported(int precision, int threads, int ppt);
+
+// The tiles list[0..n_list) (FP64 point charges, and the tiles that can be near
+// a position, at their near positions) summed at FP64 accuracy into n_splits
+// partial sums from a.partial on (esp_ddsum.cu).
+int dd_sum_splits(int n, int n_list, int num_sms);
+cudaError_t launch_dd_sum(const EvalArgs &a, const int *list, int n_list, int n_splits, cudaStream_t s);
+// dd records (esp_dd.h) of the tiles with offdd >= 0, on the coordinate grid q
+cudaError_t launch_dd_build(const TileMeta *tiles, int n_tiles, const double *rec64, double q, float *recdd,
+                            cudaStream_t s);
 
 // slot_of (optional, from launch_sort): the staged slot of each input position
 cudaError_t launch_stage(const double *pos_in, int n, const double center[3], double quantum, const Staged &st,

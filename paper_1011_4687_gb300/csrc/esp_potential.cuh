@@ -17,6 +17,7 @@
 // compile in parallel.
 #pragma once
 
+#include "esp_ddsum.cuh"
 #include "esp_eval_core.h"
 #include "esp_kernels.h"
 
@@ -24,10 +25,15 @@ namespace esp {
 
 namespace {
 
-__device__ __forceinline__ void copy_tile(float4 *__restrict__ dst, const float4 *__restrict__ src, int nvec)
+// The dd sums as calls (the batched kernel keeps its registers for the FP32 sums).
+__device__ __noinline__ double dd_points_call(const float *__restrict__ s_rec, int n4, const DdPos c, float *r2min)
 {
-    for (int i = threadIdx.x; i < nvec; i += blockDim.x)
-        dst[i] = __ldg(src + i);
+    return dd_sum_points(s_rec, n4, c, r2min);
+}
+__device__ __noinline__ double dd_general_call(int L, const float *__restrict__ s_rec, int n4, const DdPos c,
+                                               const float *__restrict__ boysdd)
+{
+    return dd_sum_general(L, s_rec, n4, c, boysdd);
 }
 
 // ---------------------------------------------------------------------------
@@ -35,42 +41,36 @@ __device__ __forceinline__ void copy_tile(float4 *__restrict__ dst, const float4
 // ---------------------------------------------------------------------------
 // One CTA's work in the FP32C kernel: position block bx against the tiles of
 // split `split` (tiles split, split + n_splits, ...).  The Boys table is
-// already in shared memory (s_boys); s_tile4 holds one staged tile.
-template <int NT, int PPT>
+// already in shared memory (s_boys); s_tile4 holds one staged tile, s_acc one
+// FP64 sum per position (ALL).
+// ALL: also the FP64 point charges and the near blocks (the batched kernel);
+// otherwise the dd kernel (esp_ddsum.cu) sums those and this one only leaves
+// them out: their code and its calls cost the far form's loops registers
+// (65,536 positions x 109,368 distributions: 9.48 ms with, 9.1 ms without).
+template <int NT, int PPT, bool ALL>
 __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, float4 *s_tile4,
-                                         const float *s_boys)
+                                         const float *s_boys, double *s_acc)
 {
     const int base = bx * NT * PPT + threadIdx.x;
-    float ch[PPT][3], cl[PPT][3];
+    // Only the FP32 sums live in registers from tile to tile.  The positions'
+    // words come from L1 again for each tile (24 loads beside the thousands of
+    // operations of a tile) and the FP64 sums, which few tiles add to, stay in
+    // shared memory: the far form's inner loop has those 30 registers more.
+    auto pos_of = [&](int q) { return min(base + q * NT, a.n_pos - 1); };
+    double *acc64 = s_acc + threadIdx.x; // [q * NT]
     float S[PPT], Cc[PPT];
-    double acc64[PPT];
-    int idx[PPT];
 #pragma unroll
     for (int q = 0; q < PPT; ++q) {
-        int i = base + q * NT;
-        idx[q] = i;
-        int ic = min(i, a.n_pos - 1);
-        ch[q][0] = a.pos.xh[ic];
-        ch[q][1] = a.pos.yh[ic];
-        ch[q][2] = a.pos.zh[ic];
-        cl[q][0] = a.pos.xl[ic];
-        cl[q][1] = a.pos.yl[ic];
-        cl[q][2] = a.pos.zl[ic];
         S[q] = 0.0f;
         Cc[q] = 0.0f;
-        acc64[q] = 0.0;
+        if (ALL)
+            acc64[q * NT] = 0.0;
     }
-    // the same positions as lane pairs (used when PPT is even)
+    // the sums of position pairs (used when PPT is even)
     constexpr int NP = PPT / 2 > 0 ? PPT / 2 : 1;
-    f2 ch2[NP][3], cl2[NP][3], S2[NP], C2[NP];
+    f2 S2[NP], C2[NP];
 #pragma unroll
     for (int q = 0; q < NP; ++q) {
-        const int q0 = 2 * q < PPT ? 2 * q : 0, q1 = 2 * q + 1 < PPT ? 2 * q + 1 : 0;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            ch2[q][d] = f2(ch[q0][d], ch[q1][d]);
-            cl2[q][d] = f2(cl[q0][d], cl[q1][d]);
-        }
         S2[q] = f2(0.0f);
         C2[q] = f2(0.0f);
     }
@@ -83,13 +83,41 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
     const int g_end = a.grp_tile[g + 1];
     for (int t = a.grp_tile[g] + (split - a.grp_split[g]); t < g_end; t += g_stride) {
         const TileMeta m = a.tiles[t];
+        if (!ALL && m.cls == kClassPoint)
+            continue;
         __syncthreads(); // previous tile fully consumed
-        const bool pts = m.cls == kClassPoint;
-        const float4 *src = pts ? reinterpret_cast<const float4 *>(a.rec64 + m.off64)
+        const bool pts = ALL && m.cls == kClassPoint;
+        const bool ddt = m.offdd >= 0;
+        const int n4 = dd_pad(m.n);
+        const float4 *s_dd = reinterpret_cast<const float4 *>(a.recdd) + (ddt ? m.offdd : 0);
+        const float4 *src = pts ? (ddt ? s_dd : reinterpret_cast<const float4 *>(a.rec64 + m.off64))
                                 : reinterpret_cast<const float4 *>(a.rec32 + m.off32);
-        const int nvec = pts ? m.n * 2 : (m.n * rec32_stride_cls(m.cls)) / 4;
+        const int nvec = pts ? (ddt ? dd_words(kClassPoint) * n4 / 4 : m.n * 2)
+                             : (m.n * rec32_stride_cls(m.cls)) / 4;
         copy_tile(s_tile4, src, nvec);
         __syncthreads();
+        float ch[PPT][3], cl[PPT][3];
+#pragma unroll
+        for (int q = 0; q < PPT; ++q) {
+            const int ic = pos_of(q);
+            ch[q][0] = a.pos.xh[ic];
+            ch[q][1] = a.pos.yh[ic];
+            ch[q][2] = a.pos.zh[ic];
+            cl[q][0] = a.pos.xl[ic];
+            cl[q][1] = a.pos.yl[ic];
+            cl[q][2] = a.pos.zl[ic];
+        }
+        // the same positions as lane pairs
+        f2 ch2[NP][3], cl2[NP][3];
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            const int q0 = 2 * q < PPT ? 2 * q : 0, q1 = 2 * q + 1 < PPT ? 2 * q + 1 : 0;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                ch2[q][d] = f2(ch[q0][d], ch[q1][d]);
+                cl2[q][d] = f2(cl[q0][d], cl[q1][d]);
+            }
+        }
         if (m.cls == kClassPoint32) {
             // small point charges: the far form of an L = 0 record, no near path
             const float *s_rec = reinterpret_cast<const float *>(s_tile4);
@@ -116,16 +144,34 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
             }
             continue;
         }
-        if (pts) {
-            double c64[PPT][3];
+        if (ALL && pts && !ddt) {
+            double c64[PPT][3], v[PPT];
 #pragma unroll
             for (int q = 0; q < PPT; ++q) {
-                int ic = min(idx[q], a.n_pos - 1);
+                const int ic = pos_of(q);
                 c64[q][0] = a.pos.x64[ic];
                 c64[q][1] = a.pos.y64[ic];
                 c64[q][2] = a.pos.z64[ic];
+                v[q] = acc64[q * NT];
             }
-            tile_points_f64<PPT>(reinterpret_cast<const double *>(s_tile4), m.n, c64, acc64);
+            tile_points_f64<PPT>(reinterpret_cast<const double *>(s_tile4), m.n, c64, v);
+#pragma unroll
+            for (int q = 0; q < PPT; ++q)
+                acc64[q * NT] = v[q];
+            continue;
+        }
+        if (ALL && pts) {
+#pragma unroll 1
+            for (int q = 0; q < PPT; ++q) {
+                const int ic = pos_of(q);
+                const DdPos c = dd_position(a.pos, ic);
+                float r2min;
+                double v = dd_points_call(reinterpret_cast<const float *>(s_tile4), n4, c, &r2min);
+                // closer than the dd words resolve, or out of their range
+                if (!(r2min >= kDdMinR2) || !dd_in_range(c.h, a.dd_lim))
+                    v = point_tile_f64(a.rec64 + m.off64, m.n, a.pos.x64[ic], a.pos.y64[ic], a.pos.z64[ic]);
+                acc64[q * NT] += v;
+            }
             continue;
         }
         bool nearq[PPT];
@@ -215,13 +261,36 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
             }
 #undef ESP_TILE
         }
-        if (any_near) {
+        if (!ALL || m.vmax < kNearVmax || !(near_r > 0.0f))
+            continue; // (block-uniform) no position can be near
+        if (ddt) {
+            // the CTA stages the tile's dd records; a warp with a near lane
+            // sums them at its positions
+            if (!__syncthreads_or(any_near))
+                continue;
+            copy_tile(s_tile4, s_dd, dd_words(m.cls) * n4 / 4);
+            __syncthreads();
+            const float *s_rec_dd = reinterpret_cast<const float *>(s_tile4);
+#pragma unroll
+            for (int q = 0; q < PPT; ++q) {
+                if (!__any_sync(0xffffffffu, nearq[q]))
+                    continue;
+                const int ic = pos_of(q);
+                const DdPos c = dd_position(a.pos, ic);
+                double v = dd_general_call(m.cls, s_rec_dd, n4, c, a.boysdd);
+                if (nearq[q] && !dd_in_range(c.h, a.dd_lim))
+                    v = tile_f64_one_any(m.cls, a.rec64 + m.off64, m.n, a.pos.x64[ic], a.pos.y64[ic], a.pos.z64[ic],
+                                         a.boys64);
+                if (nearq[q])
+                    acc64[q * NT] += v;
+            }
+        } else if (any_near) {
 #pragma unroll
             for (int q = 0; q < PPT; ++q) {
                 if (nearq[q]) {
-                    int ic = min(idx[q], a.n_pos - 1);
-                    acc64[q] += tile_f64_one_any(m.cls, a.rec64 + m.off64, m.n, a.pos.x64[ic], a.pos.y64[ic],
-                                                 a.pos.z64[ic], a.boys64);
+                    const int ic = pos_of(q);
+                    acc64[q * NT] += tile_f64_one_any(m.cls, a.rec64 + m.off64, m.n, a.pos.x64[ic], a.pos.y64[ic],
+                                                      a.pos.z64[ic], a.boys64);
                 }
             }
         }
@@ -236,9 +305,11 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
         }
     }
 #pragma unroll
-    for (int q = 0; q < PPT; ++q)
-        if (idx[q] < a.n_pos)
-            a.partial[(size_t)split * a.n_pos + idx[q]] = ((double)S[q] + (double)Cc[q]) + acc64[q];
+    for (int q = 0; q < PPT; ++q) {
+        const int i = base + q * NT;
+        if (i < a.n_pos)
+            a.partial[(size_t)split * a.n_pos + i] = ((double)S[q] + (double)Cc[q]) + (ALL ? acc64[q * NT] : 0.0);
+    }
 }
 
 template <int NT, int PPT>
@@ -249,7 +320,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) potential_f32c_kernel(EvalArgs a
     float *s_boys = reinterpret_cast<float *>(smem4 + (a.tile_size * kRec32MaxStride) / 4);
     for (int i = threadIdx.x; i < kBoys32Rows * kBoys32Row; i += NT)
         s_boys[i] = a.boys32[i];
-    cta_f32c<NT, PPT>(a, blockIdx.x, blockIdx.y, s_tile4, s_boys);
+    cta_f32c<NT, PPT, false>(a, blockIdx.x, blockIdx.y, s_tile4, s_boys, nullptr);
 }
 
 // ---------------------------------------------------------------------------
@@ -351,7 +422,8 @@ __device__ __forceinline__ int find_sys(const SysDesc *__restrict__ sys, int n_s
     return lo;
 }
 
-__device__ __forceinline__ EvalArgs args_of(const SysDesc &d, const float *boys32, const double *boys64)
+__device__ __forceinline__ EvalArgs args_of(const SysDesc &d, const float *boys32, const double *boys64,
+                                            const float *boysdd)
 {
     EvalArgs a;
     a.n_pos = d.n_pos;
@@ -364,6 +436,9 @@ __device__ __forceinline__ EvalArgs args_of(const SysDesc &d, const float *boys3
     a.rec64 = d.rec64;
     a.boys32 = boys32;
     a.boys64 = boys64;
+    a.recdd = d.recdd;
+    a.boysdd = boysdd;
+    a.dd_lim = d.dd_lim;
     a.partial = d.partial;
     a.near_r = d.near_r;
     single_group(a);
@@ -374,10 +449,11 @@ template <int NT, int PPT, int PREC>
 __global__ void __launch_bounds__(NT, PREC == 1 ? 512 / NT : 1) batch_potential_kernel(const BatchHeader *__restrict__ hdr,
                                                              const SysDesc *__restrict__ sys, int *counter,
                                                              const float *boys32, const double *boys64,
-                                                             int tile_cap)
+                                                             const float *boysdd, int tile_cap)
 {
     extern __shared__ float4 smem4[];
     __shared__ int s_item;
+    __shared__ double s_acc[PREC == 1 ? NT * PPT : 1];
     float *s_boys = reinterpret_cast<float *>(smem4 + (tile_cap * kRec32MaxStride) / 4);
     if (PREC == 1)
         for (int i = threadIdx.x; i < kBoys32Rows * kBoys32Row; i += NT)
@@ -394,9 +470,9 @@ __global__ void __launch_bounds__(NT, PREC == 1 ? 512 / NT : 1) batch_potential_
         const int k = find_sys(sys, n_sys, item, true);
         const SysDesc &d = sys[k];
         const int local = item - d.item_begin;
-        const EvalArgs a = args_of(d, boys32, boys64);
+        const EvalArgs a = args_of(d, boys32, boys64, boysdd);
         if (PREC == 1)
-            cta_f32c<NT, PPT>(a, local / d.splits, local % d.splits, smem4, s_boys);
+            cta_f32c<NT, PPT, true>(a, local / d.splits, local % d.splits, smem4, s_boys, s_acc);
         else
             cta_f64<NT, PPT>(a, local / d.splits, local % d.splits, smem4);
     }

@@ -41,7 +41,7 @@ template cudaError_t launch_f64_shape<ESP_NT, ESP_PPT>(const EvalArgs &, dim3, s
 #elif defined(ESP_SHAPE_BATCH)
 template <int NT, int PPT, int PREC>
 cudaError_t launch_batch_shape(const BatchHeader *hdr, const SysDesc *sys, int *counter, int max_items,
-                               const float *boys32, const double *boys64, int tile_cap, int num_sms, size_t smem,
+                               const float *boys32, const double *boys64, const float *boysdd, int tile_cap, int num_sms, size_t smem,
                                cudaStream_t s)
 {
     auto k = batch_potential_kernel<NT, PPT, PREC>;
@@ -52,11 +52,11 @@ cudaError_t launch_batch_shape(const BatchHeader *hdr, const SysDesc *sys, int *
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NT, smem)) != cudaSuccess)
         return e;
     const int grid = std::max(1, std::min(per_sm * num_sms, max_items));
-    k<<<grid, NT, smem, s>>>(hdr, sys, counter, boys32, boys64, tile_cap);
+    k<<<grid, NT, smem, s>>>(hdr, sys, counter, boys32, boys64, boysdd, tile_cap);
     return cudaGetLastError();
 }
 template cudaError_t launch_batch_shape<ESP_NT, ESP_PPT, ESP_PREC>(const BatchHeader *, const SysDesc *, int *, int,
-                                                                   const float *, const double *, int, int, size_t,
+                                                                   const float *, const double *, const float *, int, int, size_t,
                                                                    cudaStream_t);
 #else
 #error "define ESP_SHAPE_F32C, ESP_SHAPE_F64 or ESP_SHAPE_BATCH"

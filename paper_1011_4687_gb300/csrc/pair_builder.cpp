@@ -22,6 +22,8 @@
 //      inside a band, and cut into tiles with a bounding sphere each.
 #include "pair_builder.h"
 
+#include "esp_dd.h"
+
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -277,6 +279,71 @@ const std::vector<double> &boys_table64()
     });
     return t;
 }
+
+const std::vector<float> &boys_table_dd()
+{
+    static std::vector<float> t;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        t.assign(size_t(kBoysDdRows) * kBoysDdRow, 0.0f);
+        double F[kBoysDdHi];
+        for (int i = 0; i < kBoysDdRows; ++i) {
+            float *row = t.data() + size_t(i) * kBoysDdRow;
+            boys_by_quadrature(i / 64.0, kBoysDdHi - 1, F);
+            for (int n = 0; n < kBoysDdHi; ++n) {
+                F[n] /= 0.88622692545275801365;
+                row[n] = float(F[n]);
+                if (n < kBoysDdRow - kBoysDdHi - 2)
+                    row[kBoysDdHi + n] = float(F[n] - double(row[n]));
+            }
+        }
+    });
+    return t;
+}
+
+namespace {
+
+// dd records for the tiles that are evaluated in pairs of FP32 numbers, when
+// every number of theirs and every product of them stays well inside FP32's
+// range (else those tiles keep the FP64 code).
+void plan_dd(HostEnv &env)
+{
+    const double big = 0x1p+60, small = 0x1p-60;
+    for (TileMeta &m : env.tiles) {
+        m.offdd = -1;
+        if (!(m.cls == kClassPoint || (m.vmax >= kNearVmax && (m.cls & kClassShortBit) == 0 &&
+                                       (m.cls & 7) <= kDdGeneralMaxL)))
+            continue;
+        const bool pts = is_point_class(m.cls);
+        const int st = pts ? kPointStride64 : rec64_stride(m.cls & 7);
+        const int nc = pts ? 0 : num_hermite(m.cls & 7);
+        bool ok = env.coord_quantum < 0x1p+30; // coordinates below 2^52: squares in range
+        double cmax = 0.0;
+        for (int j = 0; j < m.n && ok; ++j) {
+            const double *r = env.rec64.data() + m.off64 + size_t(j) * st;
+            if (pts) {
+                cmax = std::max(cmax, std::fabs(r[3]));
+            } else {
+                ok = r[3] > small && r[3] < big;
+                for (int k = 0; k < nc; ++k)
+                    cmax = std::max(cmax, std::fabs(r[4 + k]) * std::max(1.0, std::pow(r[3], -1.0 - (m.cls & 7))));
+            }
+        }
+        if (!ok || !(cmax > small) || !(cmax < big))
+            continue;
+        m.offdd = int32_t(env.dd_floats / 4);
+        env.dd_floats += int64_t(dd_words(m.cls)) * dd_pad(m.n);
+        if (env.dd_floats / 4 > INT32_MAX) {
+            // beyond the offsets' range: no dd records at all
+            for (TileMeta &t : env.tiles)
+                t.offdd = -1;
+            env.dd_floats = 0;
+            return;
+        }
+    }
+}
+
+} // namespace
 
 esp_status build_environment(const esp_point_charge *charges, int64_t n_charges,
                              const esp_gauss_pair *pairs, const double *weights, int64_t n_pairs,
@@ -666,6 +733,7 @@ esp_status build_environment(const esp_point_charge *charges, int64_t n_charges,
         err = "environment too large for 32-bit record offsets";
         return ESP_ERR_INVALID;
     }
+    plan_dd(out);
     return ESP_OK;
 }
 

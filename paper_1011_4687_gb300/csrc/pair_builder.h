@@ -25,6 +25,7 @@ struct HostEnv {
     // positions are split as x = hi + lo with hi a multiple of coord_quantum, so
     // P_hi - C_hi is exact in FP32 whenever |P_hi - C_hi| < 2^24 * coord_quantum.
     double coord_quantum = 1.0 / 1048576.0;
+    int64_t dd_floats = 0;         // size of the dd records (esp_dd.h) of the tiles with offdd >= 0
 };
 
 // hi word of x on the grid q (exact in double and in FP32 for |x| < 2^23 q)
@@ -39,5 +40,7 @@ esp_status build_environment(const esp_point_charge *charges, int64_t n_charges,
 // Boys tables for the FP32 and FP64 kernels (rows at T_i = i/8).
 const std::vector<float> &boys_table32();
 const std::vector<double> &boys_table64();
+// Boys table of the dd general form (esp_dd.h: rows at T_i = i/64).
+const std::vector<float> &boys_table_dd();
 
 } // namespace esp

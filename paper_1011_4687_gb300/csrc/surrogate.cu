@@ -89,7 +89,7 @@ struct esp_surrogate {
     // near / far split of the context's tiles
     std::vector<TileMeta> near_tiles, far_tiles;
     TileView near_view, far_view;
-    DevBuf d_near_tiles, d_far_tiles;
+    DevBuf d_near_tiles, d_far_tiles, d_near_dd, d_far_dd;
     // device state
     DevBuf d_params, d_params_bf, d_grad, d_m, d_v, d_coef, d_freq, d_trust;
     DevBuf d_X, d_Z, d_H, d_dZ, d_y, d_dy, d_part, d_t, d_loss;   // per-chunk activations
@@ -324,9 +324,16 @@ void split_tiles(esp_surrogate *s)
 esp_status upload_split(esp_surrogate *s)
 {
     cudaError_t e;
+    const bool near = near_radius(s->ctx) > 0.0f;
+    const std::vector<int> nd = dd_tile_list(s->near_tiles, near), fd = dd_tile_list(s->far_tiles, near);
     if ((e = upload_vec(s->d_near_tiles, s->near_tiles)) != cudaSuccess ||
-        (e = upload_vec(s->d_far_tiles, s->far_tiles)) != cudaSuccess)
+        (e = upload_vec(s->d_far_tiles, s->far_tiles)) != cudaSuccess ||
+        (e = upload_vec(s->d_near_dd, nd)) != cudaSuccess || (e = upload_vec(s->d_far_dd, fd)) != cudaSuccess)
         return cuda_fail(e, "uploading the near/far tile split");
+    s->near_view.dd_list = static_cast<const int *>(s->d_near_dd.p);
+    s->near_view.n_dd = int(nd.size());
+    s->far_view.dd_list = static_cast<const int *>(s->d_far_dd.p);
+    s->far_view.n_dd = int(fd.size());
     s->near_view.tiles = static_cast<const TileMeta *>(s->d_near_tiles.p);
     s->far_view.tiles = static_cast<const TileMeta *>(s->d_far_tiles.p);
     return ESP_OK;
@@ -527,7 +534,8 @@ void release_sur(esp_surrogate *s)
     DevBuf *bufs[] = {&s->d_params, &s->d_params_bf, &s->d_grad, &s->d_m, &s->d_v, &s->d_coef, &s->d_freq,
                       &s->d_trust, &s->d_X, &s->d_Z, &s->d_H, &s->d_dZ, &s->d_y, &s->d_dy, &s->d_part, &s->d_t,
                       &s->d_loss, &s->d_flag, &s->d_pre, &s->d_tot, &s->d_count, &s->d_cpos, &s->d_cidx, &s->d_cV,
-                      &s->d_nfail, &s->d_wpk, &s->d_tcerr, &s->d_ynet, &s->d_near_tiles, &s->d_far_tiles,
+                      &s->d_nfail, &s->d_wpk, &s->d_tcerr, &s->d_ynet, &s->d_near_tiles, &s->d_far_tiles, &s->d_near_dd,
+                      &s->d_far_dd,
                       &s->d_gemmerr};
     for (DevBuf *b : bufs)
         b->release();
