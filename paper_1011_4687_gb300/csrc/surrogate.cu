@@ -619,28 +619,37 @@ esp_status build_trust(esp_surrogate *s, const std::vector<double> &pos, const s
     esp_status r = nearby_point_charges(s, h * 1.7321 + excl, pts);
     if (r != ESP_OK)
         return r;
+    // voxels whose centre lies within excl of a point charge: each charge marks
+    // those of its own box (trying every charge for every voxel took 115 of the
+    // 130 ms of a small training)
+    std::vector<unsigned char> excluded(vmax.size(), 0);
+    auto centre_of = [&](int i, int d) { return s->centre[d] - h + (i + 0.5) * vox; };
+    for (size_t p = 0; p + 2 < pts.size(); p += 3) {
+        int lo[3], hi[3];
+        for (int d = 0; d < 3; ++d) { // (one voxel of margin: the test below decides)
+            const double x = (pts[p + d] - s->centre[d] + h) / vox - 0.5, r = std::fabs(excl) / vox;
+            lo[d] = int(std::max(0.0, std::min(double(dim), std::floor(x - r) - 1.0)));
+            hi[d] = int(std::max(0.0, std::min(double(dim), std::ceil(x + r) + 2.0)));
+        }
+        for (int ix = lo[0]; ix < hi[0]; ++ix)
+            for (int iy = lo[1]; iy < hi[1]; ++iy)
+                for (int iz = lo[2]; iz < hi[2]; ++iz) {
+                    const double dx = pts[p] - centre_of(ix, 0), dy = pts[p + 1] - centre_of(iy, 1),
+                                 dz = pts[p + 2] - centre_of(iz, 2);
+                    if (dx * dx + dy * dy + dz * dz < excl * excl)
+                        excluded[(size_t(ix) * dim + iy) * dim + iz] = 1;
+                }
+    }
     size_t ntrust = 0, nvis = 0;
-    for (int ix = 0; ix < dim; ++ix)
-        for (int iy = 0; iy < dim; ++iy)
-            for (int iz = 0; iz < dim; ++iz) {
-                const size_t k = (size_t(ix) * dim + iy) * dim + iz;
-                if (vmax[k] < 0.0f)
-                    continue;
-                ++nvis;
-                if (vmax[k] > 0.5 * s->cfg.tol)
-                    continue;
-                const double cx = s->centre[0] - h + (ix + 0.5) * vox, cy = s->centre[1] - h + (iy + 0.5) * vox,
-                             cz = s->centre[2] - h + (iz + 0.5) * vox;
-                bool nearp = false;
-                for (size_t p = 0; p + 2 < pts.size() && !nearp; p += 3) {
-                    double dx = pts[p] - cx, dy = pts[p + 1] - cy, dz = pts[p + 2] - cz;
-                    nearp = dx * dx + dy * dy + dz * dz < excl * excl;
-                }
-                if (!nearp) {
-                    s->trust[k] = 1;
-                    ++ntrust;
-                }
-            }
+    for (size_t k = 0; k < vmax.size(); ++k) {
+        if (vmax[k] < 0.0f)
+            continue;
+        ++nvis;
+        if (vmax[k] <= 0.5 * s->cfg.tol && !excluded[k]) {
+            s->trust[k] = 1;
+            ++ntrust;
+        }
+    }
     s->trusted_fraction = nvis ? double(ntrust) / double(nvis) : 0.0;
     return ESP_OK;
 }
