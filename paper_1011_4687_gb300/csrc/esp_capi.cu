@@ -102,6 +102,36 @@ int esp::plan_splits(const esp_ctx *c, const TileView &v, int n, int prec, int m
     return dd_splits + sum;
 }
 
+SmallArgs esp::small_args(const esp_ctx *c, const TileView &v, int prec, const double *d_pos, int n, int *counters)
+{
+    SmallArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.n_pos = n;
+    a.n_tiles = v.n_tiles;
+    a.pos_in = d_pos;
+    a.cx = c->opt.qm_center[0];
+    a.cy = c->opt.qm_center[1];
+    a.cz = c->opt.qm_center[2];
+    a.tiles = v.tiles;
+    a.rec64 = static_cast<const double *>(c->rec64.p);
+    a.rec32 = static_cast<const float *>(c->rec32.p);
+    a.recdd = static_cast<const float *>(c->recdd.p);
+    a.boys64 = static_cast<const double *>(c->boys64.p);
+    a.quantum = c->env.coord_quantum;
+    a.inv_quantum = 1.0 / c->env.coord_quantum;
+    a.dd_lim = dd_limit(c);
+    a.p32_off = v.p32_off;
+    a.n_p32 = prec == 1 ? v.n_p32 : 0;
+    a.n_skip = a.n_p32 > 0 ? v.n_p32_tiles : 0;
+    a.skip_begin = v.p32_tile;
+    a.n_other = v.n_tiles - a.n_skip;
+    a.tile_halves = c->env.tile_size / 32;
+    a.points_dd = a.n_p32 > 0 && v.points_have_dd;
+    a.any64 = v.n_tiles > a.n_skip + (a.points_dd ? v.n_point_tiles : 0);
+    a.counters = counters;
+    return a;
+}
+
 cudaError_t esp::launch_planned(const esp_ctx *c, const TileView &v, int prec, EvalArgs a, int dd_splits,
                                 cudaStream_t s)
 {
@@ -131,17 +161,23 @@ void esp::set_tile_groups(const std::vector<TileMeta> &T, TileView &v)
     int64_t n_small = 0, n_all = 0;
     v.n_p32 = 0;
     v.p32_off = 0;
+    v.p32_tile = v.n_p32_tiles = 0;
     v.n_point_tiles = 0;
-    for (const TileMeta &m : T)
+    v.points_have_dd = true;
+    for (const TileMeta &m : T) {
         v.n_point_tiles += m.cls == kClassPoint;
+        v.points_have_dd &= m.cls != kClassPoint || m.offdd >= 0;
+    }
     bool contiguous = true;
     for (const TileMeta &m : T) {
         n_all += m.n;
         if (m.cls != kClassPoint32)
             continue;
-        if (n_small == 0)
+        ++v.n_p32_tiles;
+        if (n_small == 0) {
             v.p32_off = m.off32;
-        else if (int64_t(m.off32) != v.p32_off + n_small * rec32_stride(0))
+            v.p32_tile = int(&m - T.data());
+        } else if (int64_t(m.off32) != v.p32_off + n_small * rec32_stride(0))
             contiguous = false;
         n_small += m.n;
     }
@@ -206,13 +242,15 @@ esp_status pipeline(esp_ctx *c, const TileView &v, int prec, const double *d_pos
     const bool small_n = v.n_tiles > 0 && (n <= kSmallNDistributions || (n <= kSmallN && v.point_heavy));
     EvalArgs a;
     int dd_splits = 0;
-    const int splits = small_n ? small_n_splits(v.n_tiles, c->num_sms, int(n))
-                               : plan_splits(c, v, int(n), prec, 1 << 20, a, dd_splits);
-    esp_status st = ensure_scratch(c, n, splits, false, n_walkers);
-    if (st != ESP_OK)
-        return st;
+    const int splits = small_n ? 0 : plan_splits(c, v, int(n), prec, 1 << 20, a, dd_splits);
     cudaStream_t s = c->stream;
     cudaError_t e;
+    if (small_n) {
+        if ((e = c->partial.ensure(small_n_bytes(v.n_tiles, c->num_sms, int(n)))) != cudaSuccess)
+            return cuda_fail(e, "allocating partial sums");
+    } else if (esp_status st = ensure_scratch(c, n, splits, false, n_walkers); st != ESP_OK) {
+        return st;
+    }
     // FP32C with many positions: stage them in spatial order (the kernel's
     // warp-uniform far/near votes then see compact groups of positions)
     const bool sorted = !small_n && prec == 1 && n >= kSortMinPositions;
@@ -246,23 +284,8 @@ esp_status pipeline(esp_ctx *c, const TileView &v, int prec, const double *d_pos
         if ((e = cudaMemsetAsync(a.partial, 0, size_t(n) * splits * sizeof(double), s)) != cudaSuccess)
             return cuda_fail(e, "clearing partial sums");
     } else if (small_n) {
-        SmallArgs sa;
-        sa.n_pos = int(n);
-        sa.n_tiles = v.n_tiles;
-        sa.pos_in = d_pos;
-        sa.cx = c->opt.qm_center[0];
-        sa.cy = c->opt.qm_center[1];
-        sa.cz = c->opt.qm_center[2];
-        sa.tiles = v.tiles;
-        sa.rec64 = a.rec64;
-        sa.rec32 = a.rec32;
-        sa.boys64 = a.boys64;
-        sa.quantum = c->env.coord_quantum;
-        sa.fp32 = prec == 1 && v.n_p32 > 0;
-        sa.p32_off = v.p32_off;
-        sa.n_p32 = v.n_p32;
-        sa.partial = a.partial;
-        if ((e = launch_small_n(sa, splits, dV, s)) != cudaSuccess)
+        const SmallArgs sa = small_args(c, v, prec, d_pos, int(n), static_cast<int *>(c->counters.p));
+        if ((e = launch_small_n(sa, c->partial.p, c->num_sms, dV, s)) != cudaSuccess)
             return cuda_fail(e, "launching the few-position kernels");
     } else if ((e = launch_planned(c, v, prec, a, dd_splits, s)) != cudaSuccess) {
         return cuda_fail(e, "launching the potential kernel");
@@ -388,17 +411,18 @@ cudaError_t build_dd(esp_ctx *c, int64_t &bytes)
         for (TileMeta &m : c->env.tiles)
             m.offdd = -1;
         c->env.dd_floats = 0;
+        c->full.points_have_dd = c->full.n_point_tiles == 0;
         return cudaMemcpy(c->tiles.p, c->env.tiles.data(), c->env.tiles.size() * sizeof(TileMeta),
                           cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess || (e = upload(c->boysdd, boys_table_dd(), bytes)) != cudaSuccess ||
         (e = launch_dd_build(static_cast<const TileMeta *>(c->tiles.p), int(c->env.tiles.size()),
                              static_cast<const double *>(c->rec64.p), c->env.coord_quantum,
-                             static_cast<float *>(c->recdd.p), c->stream)) != cudaSuccess)
-        return e;
+                             static_cast<float *>(c->recdd.p), cudaStreamLegacy)) != cudaSuccess)
+        return e; // (the legacy stream: after the uploads)
     bytes += int64_t(c->recdd.bytes);
-    // (other streams may use the context's records next: a batch, a server)
-    return cudaStreamSynchronize(c->stream);
+    // (the context's, a batch's or a server's stream uses the records next)
+    return cudaStreamSynchronize(cudaStreamLegacy);
 }
 
 void release_all(esp_ctx *c)
@@ -408,7 +432,7 @@ void release_all(esp_ctx *c)
             cudaEventDestroy(ev);
             ev = nullptr;
         }
-    DevBuf *bufs[] = {&c->tiles, &c->rec32, &c->rec64, &c->boys32, &c->boys64, &c->recdd, &c->boysdd, &c->ddlist,
+    DevBuf *bufs[] = {&c->tiles, &c->rec32, &c->rec64, &c->boys32, &c->boys64, &c->recdd, &c->boysdd, &c->ddlist, &c->counters,
                       &c->in, &c->stage, &c->partial, &c->vout, &c->eout, &c->sortbuf};
     for (DevBuf *b : bufs)
         b->release();
@@ -616,6 +640,7 @@ esp_status esp_create(const esp_point_charge *charges, int64_t n_charges, const 
     const std::vector<int> ddlist = dd_tile_list(c->env.tiles, near_radius(c) > 0.0f);
     if (e != cudaSuccess || (e = upload(c->tiles, c->env.tiles, bytes)) != cudaSuccess ||
         (e = upload(c->ddlist, ddlist, bytes)) != cudaSuccess ||
+        (e = upload(c->counters, std::vector<int>(kSmallMaxChunks, 0), bytes)) != cudaSuccess ||
         (e = upload(c->rec32, c->env.rec32, bytes)) != cudaSuccess ||
         (e = upload(c->rec64, c->env.rec64, bytes)) != cudaSuccess ||
         (e = upload(c->boys32, boys_table32(), bytes)) != cudaSuccess ||

@@ -151,11 +151,13 @@ struct TileView {
     const int *dd_list = nullptr;
     int n_dd = 0;
     int n_point_tiles = 0;
+    bool points_have_dd = true; // every FP64 point tile has dd records
     bool point_heavy = false; // >= 90 % of the entries are FP32 point charges
     // FP32 point charges of the view: their records are contiguous in rec32
     // (the builder emits those tiles one after the other)
     int64_t p32_off = 0;
     int n_p32 = 0;
+    int p32_tile = 0, n_p32_tiles = 0; // their tiles (one range)
 };
 
 // Tile groups of a host tile list (in device order); with fewer than one
@@ -173,7 +175,7 @@ struct esp_ctx {
     esp_options opt;
     esp::HostEnv env;        // host copy of the tiles (kept for esp_get_info / test hook)
     bool host_copy = true;
-    esp::DevBuf tiles, rec32, rec64, boys32, boys64, recdd, boysdd, ddlist;
+    esp::DevBuf tiles, rec32, rec64, boys32, boys64, recdd, boysdd, ddlist, counters;
     esp::DevBuf in, stage, partial, vout, eout, sortbuf;
     std::atomic<int> busy{0};
     int64_t device_bytes = 0;
@@ -208,6 +210,9 @@ int view_precision(const esp_ctx *c, const TileView &v);
 // its first dd_splits partial sums (set here) are the dd kernel's, and
 // a.n_splits counts the rest.
 int plan_splits(const esp_ctx *c, const TileView &v, int n, int prec, int max_splits, EvalArgs &a, int &dd_splits);
+// Arguments of the few-position kernel over the view's tiles (positions,
+// scratch and output are the caller's; counters: kSmallMaxChunks zeroed ints).
+SmallArgs small_args(const esp_ctx *c, const TileView &v, int prec, const double *d_pos, int n, int *counters);
 // The potential kernels of a planned evaluation on stream s.
 cudaError_t launch_planned(const esp_ctx *c, const TileView &v, int prec, EvalArgs a, int dd_splits, cudaStream_t s);
 // Potentials of the view's tiles at n device positions into device V (the

@@ -199,10 +199,10 @@ ESP_HD dd dd_form(dd x, dd y, dd z, C c)
 }
 
 // x = h + m + l as described above; returns the rest x - h.  (q is a power of
-// two: the products with 1 / q are exact.)
-ESP_HD double dd_split3(double x, double q, float &h, float &m, float &l)
+// two: the products with iq = 1 / q are exact.)
+ESP_HD double dd_split3(double x, double q, double iq, float &h, float &m, float &l)
 {
-    const double iq = 1.0 / q, qm = q * 0x1p-23;
+    const double qm = q * 0x1p-23;
     const double xh = nearbyint(x * iq) * q, r = x - xh, xm = nearbyint(r * (iq * 0x1p+23)) * qm;
     h = float(xh);
     m = float(xm);
@@ -297,7 +297,7 @@ ESP_HD void dd_convert_dist(const double *r, bool shortr, float *out, int n4)
 ESP_HD void dd_convert(int cls, const double *r, double q, float *out, int n4)
 {
     for (int d = 0; d < 3; ++d)
-        dd_split3(r[d], q, out[d * n4], out[(3 + d) * n4], out[(6 + d) * n4]);
+        dd_split3(r[d], q, 1.0 / q, out[d * n4], out[(3 + d) * n4], out[(6 + d) * n4]);
     const bool sh = (cls & kClassShortBit) != 0;
     if (is_point_class(cls)) {
         dd_split_rel(r[3], out[9 * n4], out[10 * n4]);

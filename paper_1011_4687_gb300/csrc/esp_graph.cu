@@ -3,8 +3,8 @@
 // The paper evaluates one electron position per GPU call, once per Metropolis
 // move (Sec. III, Fig. codeStructure: r_new in, U_ES out).  At that size the
 // launch overhead matters as much as the sum itself, so this entry point
-// captures the few-position pipeline (entries spread over all SMs, then one
-// CTA per position for the fixed-order sum) for a fixed device position
+// captures the few-position launch (entries spread over all SMs, the sums joined
+// in a fixed order by the last CTA) for a fixed device position
 // buffer and output once, and each call replays the graph: the caller writes
 // the new positions into the same buffer between calls.
 #include <cuda_runtime.h>
@@ -65,23 +65,12 @@ esp_status esp_graph_create(esp_ctx *ctx, const double *positions, int64_t n, do
         return fail(ESP_ERR_OOM, "host allocation of the graph");
     g->ctx = ctx;
     g->n = int(n);
-    const int splits = small_n_splits(ctx->n_tiles, ctx->num_sms, int(n));
-    SmallArgs sa;
-    sa.n_pos = int(n);
-    sa.n_tiles = ctx->n_tiles;
-    sa.pos_in = positions;
-    sa.cx = ctx->opt.qm_center[0];
-    sa.cy = ctx->opt.qm_center[1];
-    sa.cz = ctx->opt.qm_center[2];
-    sa.tiles = ctx->full.tiles;
-    sa.rec64 = static_cast<const double *>(ctx->rec64.p);
-    sa.rec32 = static_cast<const float *>(ctx->rec32.p);
-    sa.boys64 = static_cast<const double *>(ctx->boys64.p);
-    sa.quantum = ctx->env.coord_quantum;
-    sa.fp32 = ctx->opt.precision == ESP_FP32C && ctx->full.n_p32 > 0;
-    sa.p32_off = ctx->full.p32_off;
-    sa.n_p32 = ctx->full.n_p32;
-    cudaError_t e = g->partial.ensure(size_t(splits) * size_t(n) * sizeof(double));
+    // scratch, then the launch's own counters
+    const size_t bytes = small_n_bytes(ctx->n_tiles, ctx->num_sms, int(n));
+    cudaError_t e = g->partial.ensure(bytes + kSmallMaxChunks * sizeof(int));
+    int *counters = reinterpret_cast<int *>(static_cast<char *>(g->partial.p) + bytes);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(counters, 0, kSmallMaxChunks * sizeof(int), ctx->stream);
     if (e == cudaSuccess)
         e = cudaStreamCreateWithFlags(&g->cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
@@ -89,9 +78,9 @@ esp_status esp_graph_create(esp_ctx *ctx, const double *positions, int64_t n, do
         delete g;
         return cuda_fail(e, "allocating the graph's scratch");
     }
-    sa.partial = static_cast<double *>(g->partial.p);
+    const SmallArgs sa = small_args(ctx, ctx->full, ctx->opt.precision == ESP_FP32C ? 1 : 0, positions, int(n), counters);
     e = cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal);
-    cudaError_t e1 = e == cudaSuccess ? launch_small_n(sa, splits, V_out, g->cap) : e;
+    cudaError_t e1 = e == cudaSuccess ? launch_small_n(sa, g->partial.p, ctx->num_sms, V_out, g->cap) : e;
     cudaGraph_t graph = nullptr;
     if (e == cudaSuccess)
         e = cudaStreamEndCapture(g->cap, &graph);

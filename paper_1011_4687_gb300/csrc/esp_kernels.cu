@@ -3,7 +3,6 @@
 // The potential kernels themselves are templates in esp_potential.cuh; each
 // launch shape is compiled into its own object from esp_shape.cu, and the
 // dispatchers below pick the shape's launcher.
-#include "esp_dd.h"
 #include "esp_potential.cuh"
 #include "esp_shapes.h"
 
@@ -20,11 +19,11 @@ namespace {
 // ---------------------------------------------------------------------------
 // One recentred coordinate: its FP64 value, hi word on the environment's grid
 // q (see the pair builder), lo word, and the rest in two words (esp_dd.h).
-__device__ __forceinline__ void stage_coord(double x, double q, double *x64, float *xh, float *xl, float *xm,
+__device__ __forceinline__ void stage_coord(double x, double q, double iq, double *x64, float *xh, float *xl, float *xm,
                                             float *xr)
 {
     float h, m, r;
-    const double rest = dd_split3(x, q, h, m, r);
+    const double rest = dd_split3(x, q, iq, h, m, r);
     *x64 = x;
     *xh = h;
     *xl = (float)rest;
@@ -34,9 +33,10 @@ __device__ __forceinline__ void stage_coord(double x, double q, double *x64, flo
 
 __device__ __forceinline__ void stage_position(const Staged &st, int j, double x, double y, double z, double q)
 {
-    stage_coord(x, q, st.x64 + j, st.xh + j, st.xl + j, st.xm + j, st.xr + j);
-    stage_coord(y, q, st.y64 + j, st.yh + j, st.yl + j, st.ym + j, st.yr + j);
-    stage_coord(z, q, st.z64 + j, st.zh + j, st.zl + j, st.zm + j, st.zr + j);
+    const double iq = 1.0 / q;
+    stage_coord(x, q, iq, st.x64 + j, st.xh + j, st.xl + j, st.xm + j, st.xr + j);
+    stage_coord(y, q, iq, st.y64 + j, st.yh + j, st.yl + j, st.ym + j, st.yr + j);
+    stage_coord(z, q, iq, st.z64 + j, st.zh + j, st.zl + j, st.zm + j, st.zr + j);
 }
 
 // slot_of (optional): the staged slot of position i (spatial order, below)
@@ -252,13 +252,20 @@ __global__ void __launch_bounds__(kSortThreads) batch_sort_kernel(const BatchHea
 // move).  The roles of the main kernels turn back to the paper's: threads
 // take environment entries (cells, point charges, distributions) and evaluate
 // them at the positions of their CTA's chunk (up to kSmallChunk of the n <=
-// kSmallN positions; grid.y = chunk), the CTA reduces per position in a fixed
-// order, and CTA (b, chunk) writes partial[b][q] for its chunk's q.  FP32
-// point charges are read in one flat coalesced pass over their contiguous
-// records (each once per chunk); the other tiles are dealt round-robin to the
-// CTAs of a chunk and read from the FP64 records.
+// kSmallN positions; grid.y = chunk).  FP32 point charges are read in one flat
+// coalesced pass over their contiguous records (each once per chunk), two
+// positions per packed FP32 operation; the entries of the other tiles go to
+// warps one tile half and one position at a time.  Every CTA writes its sums,
+// and the last CTA of a chunk to finish adds them up in a fixed order.
+//
+// One launch, bound by its latency at one position (records from L2, two
+// reductions) and by FP32 at many.  Before, 128-thread CTAs evaluated one
+// position per operation, reduced every position over all lanes, put the
+// nuclei's FP64 terms of all positions on one CTA and left the sum of 1,216
+// partials to a second kernel: 268,818 cells at 1 / 16 / 128 positions took
+// 18.4 / 39 / 78 us.
 // ---------------------------------------------------------------------------
-constexpr int kSmallThreads = 128;
+constexpr int kSmallWarps = kSmallThreads / 32;
 
 // (s, c) += (s2, c2) with the rounding error of s + s2 kept in c (TwoSum)
 __device__ __forceinline__ void two_sum_pair(float &s, float &c, float s2, float c2)
@@ -269,153 +276,286 @@ __device__ __forceinline__ void two_sum_pair(float &s, float &c, float s2, float
     s = t;
     c = (c + c2) + e;
 }
-
-__global__ void __launch_bounds__(kSmallThreads, 4) small_n_kernel(SmallArgs a)
+__device__ __forceinline__ void two_sum_pair_xor(float &s, float &c, int o)
 {
-    // grid: x = slice of the environment's entries, y = chunk of kSmallChunk
-    // positions; each (slice, position) partial sum is written by one CTA
-    __shared__ double s_pos[kSmallChunk][3];
-    __shared__ float s_ph[kSmallChunk][3], s_pl[kSmallChunk][3]; // FP32 hi (on the records' grid) and lo words
-    __shared__ float s_red32[kSmallThreads / 32][kSmallChunk][2];
-    __shared__ double s_red64[kSmallThreads / 32][kSmallChunk];
-    const int n = a.n_pos;
-    const int q0 = blockIdx.y * kSmallChunk;
-    const int nq = min(kSmallChunk, n - q0);
-    for (int i = threadIdx.x; i < nq * 3; i += kSmallThreads) {
-        const int c = i % 3;
-        const double x = a.pos_in[3 * q0 + i] - (c == 0 ? a.cx : c == 1 ? a.cy : a.cz);
-        const double h = nearbyint(x / a.quantum) * a.quantum;
-        s_pos[i / 3][c] = x;
-        s_ph[i / 3][c] = float(h);
-        s_pl[i / 3][c] = float(x - h);
-    }
-    // does this CTA evaluate any entry in FP64?  (then its FP64 sums need a
-    // FP64 reduction; FP64 instructions run at 1/64 of the FP32 rate here)
-    bool has64 = false;
-    for (int t = blockIdx.x; t < a.n_tiles && !has64; t += gridDim.x)
-        has64 = !(a.tiles[t].cls == kClassPoint32 && a.fp32);
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int gtid = blockIdx.x * kSmallThreads + threadIdx.x, gthreads = gridDim.x * kSmallThreads;
-    float acc32[kSmallChunk];
-    double acc[kSmallChunk];
+    const float s2 = __shfl_xor_sync(0xffffffffu, s, o), c2 = __shfl_xor_sync(0xffffffffu, c, o);
+    two_sum_pair(s, c, s2, c2);
+}
+
+// Sums of NQ values per lane over the 32 lanes, halving the values with the
+// lanes: lane l ends with the sum of value small_owner<NQ>(l).
+template <int NQ>
+__device__ __forceinline__ void warp_sums(float (&s)[NQ], float (&c)[NQ], int lane)
+{
+    int o = 16;
 #pragma unroll
-    for (int q = 0; q < kSmallChunk; ++q) {
-        acc32[q] = 0.0f;
-        acc[q] = 0.0;
-    }
-    // FP32 point charges: one flat, coalesced pass over their contiguous
-    // records (thread g takes entries g, g + G, ...: the paper's coalesced
-    // mapping); a thread's few terms sum in FP32
-    if (a.fp32 && a.n_p32 > 0) {
-        for (int e = gtid; e < a.n_p32; e += gthreads) {
-            const float *r = a.rec32 + a.p32_off + (size_t)e * rec32_stride(0);
-            const float4 r0 = reinterpret_cast<const float4 *>(r)[0];
-            const float4 r1 = reinterpret_cast<const float4 *>(r)[1];
-            const float qh = r[rec32_m(0)], ql = r1.w;
+    for (int half = NQ / 2; half > 0; half >>= 1, o >>= 1) {
+        const bool up = lane & o;
 #pragma unroll
-            for (int q = 0; q < kSmallChunk; ++q) {
-                if (q >= nq)
-                    break;
-                const float dx = (r0.x - s_ph[q][0]) + (r1.x - s_pl[q][0]);
-                const float dy = (r0.y - s_ph[q][1]) + (r1.y - s_pl[q][1]);
-                const float dz = (r0.z - s_ph[q][2]) + (r1.z - s_pl[q][2]);
-                const float rs = esp_rsqrt(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-                acc32[q] += fmaf(qh, rs, ql * rs);
-            }
+        for (int k = 0; k < half; ++k) {
+            const float so = up ? s[k] : s[k + half], co = up ? c[k] : c[k + half];
+            const float s2 = __shfl_xor_sync(0xffffffffu, so, o), c2 = __shfl_xor_sync(0xffffffffu, co, o);
+            s[k] = up ? s[k + half] : s[k];
+            c[k] = up ? c[k + half] : c[k];
+            two_sum_pair(s[k], c[k], s2, c2);
         }
     }
-    // every other tile (FP64 points, distributions; FP32 points under FP64),
-    // dealt round-robin to the CTAs, one entry per thread
-    if (has64) {
-        for (int t = blockIdx.x; t < a.n_tiles; t += gridDim.x) {
-            const TileMeta m = a.tiles[t];
-            if (m.cls == kClassPoint32 && a.fp32)
-                continue;
-            const bool pts = is_point_class(m.cls);
-            const int st = pts ? kPointStride64 : rec64_stride(m.cls & 7);
-            for (int j = threadIdx.x; j < m.n; j += kSmallThreads) {
-                const double *r = a.rec64 + m.off64 + (size_t)j * st;
+    for (; o > 0; o >>= 1)
+        two_sum_pair_xor(s[0], c[0], o);
+}
+template <int NQ>
+__device__ __forceinline__ int small_owner(int lane)
+{
+    int q = 0, o = 16;
 #pragma unroll
-                for (int q = 0; q < kSmallChunk; ++q) {
-                    if (q >= nq)
-                        break;
-                        if (pts) {
-                        const double dx = r[0] - s_pos[q][0], dy = r[1] - s_pos[q][1], dz = r[2] - s_pos[q][2];
-                        acc[q] += r[3] * esp_rsqrt(dx * dx + dy * dy + dz * dz);
-                    } else {
-                        acc[q] += tile_f64_one_any(m.cls, r, 1, s_pos[q][0], s_pos[q][1], s_pos[q][2],
-                                                   a.boys64);
-                    }
+    for (int half = NQ / 2; half > 0; half >>= 1, o >>= 1)
+        q += lane & o ? half : 0;
+    return q;
+}
+
+// one entry of a tile at one position, FP64
+// (a call: its registers would spill those of the FP32 pass)
+__device__ __noinline__ double entry_f64(const SmallArgs &a, const TileMeta &m, int j, const double *p)
+{
+    if (is_point_class(m.cls)) {
+        const double *r = a.rec64 + m.off64 + (size_t)j * kPointStride64;
+        const double dx = r[0] - p[0], dy = r[1] - p[1], dz = r[2] - p[2];
+        return r[3] * esp_rsqrt(dx * dx + dy * dy + dz * dz);
+    }
+    return tile_f64_one_any(m.cls, a.rec64 + m.off64 + (size_t)j * rec64_stride(m.cls & 7), 1, p[0], p[1], p[2],
+                            a.boys64);
+}
+
+// the words of two positions
+struct PairPos {
+    f2 xh, yh, zh, xl, yl, zl;
+    __device__ __forceinline__ explicit PairPos(const float *s)
+    {
+        const float4 a = reinterpret_cast<const float4 *>(s)[0], b = reinterpret_cast<const float4 *>(s)[1],
+                     c = reinterpret_cast<const float4 *>(s)[2];
+        xh = f2(a.x, a.y), yh = f2(a.z, a.w), zh = f2(b.x, b.y);
+        xl = f2(b.z, b.w), yl = f2(c.x, c.y), zl = f2(c.z, c.w);
+    }
+};
+// one FP32 point charge
+struct P32Entry {
+    f2 xh, yh, zh, xl, yl, zl, qh, ql;
+    __device__ __forceinline__ explicit P32Entry(const float *__restrict__ r)
+    {
+        const float4 a = __ldg(reinterpret_cast<const float4 *>(r));
+        const float4 b = __ldg(reinterpret_cast<const float4 *>(r) + 1);
+        xh = f2(a.x), yh = f2(a.y), zh = f2(a.z), xl = f2(b.x), yl = f2(b.y), zl = f2(b.z);
+        qh = f2(__ldg(r + rec32_m(0))), ql = f2(b.w);
+    }
+    __device__ __forceinline__ f2 term(const PairPos &p) const
+    {
+        const f2 dx = (xh - p.xh) + (xl - p.xl), dy = (yh - p.yh) + (yl - p.yl), dz = (zh - p.zh) + (zl - p.zl);
+        const f2 rs = esp_rsqrt(esp_fma(dx, dx, esp_fma(dy, dy, dz * dz)));
+        return esp_fma(qh, rs, ql * rs);
+    }
+};
+
+template <int NQ>
+__global__ void __launch_bounds__(kSmallThreads, NQ <= 4 ? 2 : 1) small_n_kernel(SmallArgs a, double *__restrict__ V)
+{
+    // grid: x = slice of the environment's entries, y = chunk of positions
+    __shared__ double s_pos[NQ][3];
+    __shared__ DdPos s_dd[NQ];
+    __shared__ __align__(16) float s_pair[NQ / 2 > 0 ? NQ / 2 : 1][12]; // lanes' hi x y z, lo x y z of position pairs
+    __shared__ float2 s_red[kSmallWarps][NQ]; // sums in FP32 with compensation
+    __shared__ double s_red64[kSmallWarps][NQ];
+    __shared__ int s_last;
+    const int n = a.n_pos, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int q0 = blockIdx.y * kSmallChunk;
+    const int nq = min(NQ, n - q0);
+    // does this CTA take any entry in FP64 (or as dd sums)?
+    const int units = a.n_other * a.tile_halves;
+    const bool has64 = int(blockIdx.x) < units * nq;
+    if (t < 3 * NQ) {
+        const int q = min(t / 3, nq - 1), d = t % 3; // (padding repeats the last position)
+        const double x = a.pos_in[3 * (q0 + q) + d] - (d == 0 ? a.cx : d == 1 ? a.cy : a.cz);
+        float h, m, r;
+        const double rest = dd_split3(x, a.quantum, a.inv_quantum, h, m, r);
+        s_pos[t / 3][d] = x;
+        s_dd[t / 3].h[d] = h;
+        s_dd[t / 3].m[d] = m;
+        s_dd[t / 3].l[d] = r;
+        s_pair[t / 6][2 * d + (t / 3) % 2] = h;
+        s_pair[t / 6][6 + 2 * d + (t / 3) % 2] = float(rest);
+    }
+    if (t < kSmallWarps * NQ) {
+        s_red[t / NQ][t % NQ] = make_float2(0.0f, 0.0f);
+        s_red64[t / NQ][t % NQ] = 0.0;
+    }
+    __syncthreads();
+    // FP32 point charges: thread g takes entries g, g + G, ... (the paper's
+    // coalesced mapping) and sums its terms in FP32
+    const int g0 = blockIdx.x * kSmallThreads + t;
+    if (a.n_p32 > 0) {
+        constexpr int NP = NQ / 2;
+        f2 acc[NP];
+#pragma unroll
+        for (int k = 0; k < NP; ++k)
+            acc[k] = f2(0.0f);
+        if (g0 < a.g_threads) {
+            const float *rec = a.rec32 + a.p32_off;
+            const size_t step = (size_t)a.g_threads * rec32_stride(0);
+            const float *r = rec + (size_t)g0 * rec32_stride(0);
+            int e = g0;
+            // two entries per pass over the positions (their words come from
+            // shared memory once for both), each sum in the entries' order
+            for (; e + a.g_threads < a.n_p32; e += 2 * a.g_threads, r += 2 * step) {
+                const P32Entry u(r), v(r + step);
+#pragma unroll
+                for (int k = 0; k < NP; ++k) {
+                    const PairPos p(s_pair[k]);
+                    const f2 x = u.term(p), y = v.term(p);
+                    acc[k] += x;
+                    acc[k] += y;
                 }
             }
-        }
-    }
-    // fixed-order reduction per position: the FP32 sums as (sum,
-    // compensation) pairs by warp shuffles, the FP64 sums (only where this
-    // CTA has any) likewise in FP64, then the warps in order in FP64
+            if (e < a.n_p32) {
+                const P32Entry u(r);
 #pragma unroll
-    for (int q = 0; q < kSmallChunk; ++q) {
-        if (q >= nq)
-            break;
-        float sv = acc32[q], cv = 0.0f;
-        for (int o = 16; o; o >>= 1) {
-            const float so = __shfl_xor_sync(0xffffffffu, sv, o), co = __shfl_xor_sync(0xffffffffu, cv, o);
-            two_sum_pair(sv, cv, so, co);
+                for (int k = 0; k < NP; ++k)
+                    acc[k] += u.term(PairPos(s_pair[k]));
+            }
         }
-        double v = 0.0;
-        if (has64) {
-            v = acc[q];
-            for (int o = 16; o; o >>= 1)
-                v += __shfl_xor_sync(0xffffffffu, v, o);
+        float s[NQ], c[NQ];
+#pragma unroll
+        for (int k = 0; k < NQ; ++k) {
+            s[k] = k % 2 ? acc[k / 2].y : acc[k / 2].x;
+            c[k] = 0.0f;
         }
-        if (lane == 0) {
-            s_red32[warp][q][0] = sv;
-            s_red32[warp][q][1] = cv;
-            s_red64[warp][q] = v;
+        warp_sums<NQ>(s, c, lane);
+        s_red[warp][small_owner<NQ>(lane)] = make_float2(s[0], c[0]); // (lanes of one owner hold the same sum)
+        __syncwarp();
+    }
+    // the other tiles: warp w of CTA b takes (half tile, position) items b + grid w, ...
+    if (has64) {
+        for (int item = blockIdx.x + gridDim.x * warp; item < units * nq; item += gridDim.x * kSmallWarps) {
+            const int u = item % units, q = item / units;
+            const int o = u / a.tile_halves;
+            const TileMeta m = a.tiles[o < a.skip_begin ? o : o + a.n_skip];
+            const int j = (u % a.tile_halves) * 32 + lane;
+            if (m.cls == kClassPoint && a.points_dd) {
+                // beside FP32 sums: a dd sum, pairs of charges on the first lanes
+                const int n4 = dd_pad(m.n);
+                const float *rec = a.recdd + (size_t)m.offdd * 4;
+                float s = 0.0f, c = 0.0f;
+                if (j < m.n) {
+                    const DdTile tile = {rec, n4};
+                    f2 r2;
+                    const dd v = dd_point(tile, j & ~1, s_dd[q], r2);
+                    s = j & 1 ? v.h.y : v.h.x;
+                    c = j & 1 ? v.l.y : v.l.x;
+                    if (!((j & 1 ? r2.y : r2.x) >= kDdMinR2) || !dd_in_range(s_dd[q].h, a.dd_lim)) {
+                        const double x = entry_f64(a, m, j, s_pos[q]);
+                        s = float(x);
+                        c = float(x - double(s));
+                    }
+                }
+#pragma unroll
+                for (int w = 16; w > 0; w >>= 1)
+                    two_sum_pair_xor(s, c, w);
+                if (lane == 0) {
+                    float2 x = s_red[warp][q];
+                    two_sum_pair(x.x, x.y, s, c);
+                    s_red[warp][q] = x;
+                }
+            } else {
+                double v = j < m.n ? entry_f64(a, m, j, s_pos[q]) : 0.0;
+#pragma unroll
+                for (int w = 16; w > 0; w >>= 1)
+                    v += __shfl_xor_sync(0xffffffffu, v, w);
+                if (lane == 0)
+                    s_red64[warp][q] += v;
+            }
+            __syncwarp();
         }
     }
     __syncthreads();
-    if (threadIdx.x < nq) {
-        double v = 0.0;
-        for (int w = 0; w < kSmallThreads / 32; ++w)
-            v += (double(s_red32[w][threadIdx.x][0]) + double(s_red32[w][threadIdx.x][1])) +
-                 s_red64[w][threadIdx.x];
-        a.partial[(size_t)blockIdx.x * n + q0 + threadIdx.x] = v;
+    // this CTA's sums, warps in order
+    float2 *part32 = a.part32 + (size_t)blockIdx.y * gridDim.x * NQ;
+    double *part64 = a.part64 + (size_t)blockIdx.y * gridDim.x * NQ;
+    if (t < NQ) {
+        float2 x = s_red[0][t];
+        double v = s_red64[0][t];
+        for (int w = 1; w < kSmallWarps; ++w) {
+            two_sum_pair(x.x, x.y, s_red[w][t].x, s_red[w][t].y);
+            if (has64 && a.any64)
+                v += s_red64[w][t];
+        }
+        part32[blockIdx.x * NQ + t] = x;
+        if (has64 && a.any64)
+            part64[blockIdx.x * NQ + t] = v;
+        __threadfence();
     }
+    __syncthreads();
+    if (t == 0)
+        s_last = atomicAdd(&a.counters[blockIdx.y], 1) == int(gridDim.x) - 1;
+    __syncthreads();
+    if (!s_last)
+        return;
+    // last CTA of the chunk: thread t takes position t % NQ of the slices t / NQ, ...
+    __threadfence();
+    const int n64 = a.any64 ? min(units * nq, int(gridDim.x)) : 0;
+    constexpr int rows = kSmallThreads / NQ;
+    const int q = t % NQ;
+    float s = 0.0f, c = 0.0f;
+    for (int k = t / NQ; k < int(gridDim.x); k += rows) {
+        const float2 x = __ldcg(part32 + (size_t)k * NQ + q);
+        two_sum_pair(s, c, x.x, x.y);
+    }
+    double s64 = 0.0, c64 = 0.0;
+    for (int k = t / NQ; k < n64; k += rows)
+        two_sum_acc(s64, c64, __ldcg(part64 + (size_t)k * NQ + q));
+    // the warp's lanes of one position, then the warps
+#pragma unroll
+    for (int o = 16; o >= NQ; o >>= 1) {
+        two_sum_pair_xor(s, c, o);
+        if (n64 > 0) {
+            const double a2 = __shfl_xor_sync(0xffffffffu, s64, o), b2 = __shfl_xor_sync(0xffffffffu, c64, o);
+            two_sum_acc(s64, c64, a2);
+            c64 += b2;
+        }
+    }
+    __shared__ double s_fin[kSmallWarps][NQ][2];
+    __syncthreads();
+    if (lane < NQ) {
+        s_red[warp][lane] = make_float2(s, c);
+        s_fin[warp][lane][0] = s64;
+        s_fin[warp][lane][1] = c64;
+    }
+    __syncthreads();
+    if (warp < nq) { // warp q: position q, lane w the sums of warp w
+        float2 x = lane < kSmallWarps ? s_red[lane][warp] : make_float2(0.0f, 0.0f);
+        double v = 0.0, w = 0.0;
+        if (n64 > 0 && lane < kSmallWarps) {
+            v = s_fin[lane][warp][0];
+            w = s_fin[lane][warp][1];
+        }
+#pragma unroll
+        for (int o = kSmallWarps / 2; o > 0; o >>= 1) {
+            two_sum_pair_xor(x.x, x.y, o);
+            if (n64 > 0) {
+                const double v2 = __shfl_xor_sync(0xffffffffu, v, o), w2 = __shfl_xor_sync(0xffffffffu, w, o);
+                two_sum_acc(v, w, v2);
+                w += w2;
+            }
+        }
+        if (lane == 0) {
+            const double y = double(x.x) + double(x.y);
+            V[q0 + warp] = n64 > 0 ? y + (v + w) : y;
+        }
+    }
+    if (t == 0)
+        a.counters[blockIdx.y] = 0; // for the next call
 }
 
 // ---------------------------------------------------------------------------
 // reductions
 // ---------------------------------------------------------------------------
-// Many partials for few positions: one CTA per position, strided TwoSum per
-// thread, then a fixed-order tree over the threads' (sum, compensation) pairs.
-constexpr int kWideThreads = 256;
-
-__global__ void __launch_bounds__(kWideThreads) reduce_wide_kernel(const double *__restrict__ partial, int n_splits,
-                                                                    int n, double *__restrict__ V)
-{
-    __shared__ double s_s[kWideThreads], s_c[kWideThreads];
-    const int q = blockIdx.x, t = threadIdx.x;
-    double sum = 0.0, cmp = 0.0;
-    for (int k = t; k < n_splits; k += kWideThreads)
-        two_sum_acc(sum, cmp, partial[(size_t)k * n + q]);
-    s_s[t] = sum;
-    s_c[t] = cmp;
-    __syncthreads();
-    for (int o = kWideThreads / 2; o > 0; o >>= 1) {
-        if (t < o) {
-            double a = s_s[t], c = s_c[t] + s_c[t + o];
-            two_sum_acc(a, c, s_s[t + o]);
-            s_s[t] = a;
-            s_c[t] = c;
-        }
-        __syncthreads();
-    }
-    if (t == 0)
-        V[q] = s_s[0] + s_c[0];
-}
-
 // (s, c) += (s2, c2)
 __device__ __forceinline__ void two_sum_join(double &s, double &c, double s2, double c2)
 {
@@ -579,25 +719,46 @@ bool batch_shape_supported(int precision, int threads, int ppt)
 #undef ESP_BSHAPE_IS
 }
 
-// Slices of the environment's entries: about 8 CTAs per SM over all chunks of
-// positions, so that with more positions each thread takes more entries and
-// the per-position reduction is amortised over more terms.
-int small_n_splits(int n_tiles, int num_sms, int n)
+// The sums of one thread: entries g, g + G, ... of the FP32 point charges, G =
+// 128 threads for each of about 8 slices per SM over all chunks of positions,
+// so that with more positions each thread takes more entries and the
+// per-position reductions are amortised over more terms.
+int small_n_threads(int n_tiles, int num_sms, int n)
 {
     const int chunks = std::max(1, (n + kSmallChunk - 1) / kSmallChunk);
-    return std::max(1, std::min(n_tiles, 8 * num_sms / chunks));
+    return 128 * std::max(1, std::min(n_tiles, 8 * num_sms / chunks));
 }
 
-cudaError_t launch_small_n(const SmallArgs &a, int n_splits, double *V, cudaStream_t s)
+namespace {
+
+// positions a chunk holds: two (one pair) up to kSmallChunk
+int small_nq(int n) { return n <= 2 ? 2 : n <= 4 ? 4 : n <= 8 ? 8 : 16; }
+
+int small_grid(int g_threads) { return (g_threads + kSmallThreads - 1) / kSmallThreads; }
+
+} // namespace
+
+size_t small_n_bytes(int n_tiles, int num_sms, int n)
+{
+    const int chunks = std::max(1, (n + kSmallChunk - 1) / kSmallChunk);
+    return (size_t)small_grid(small_n_threads(n_tiles, num_sms, n)) * chunks * small_nq(n) * (sizeof(float2) + sizeof(double));
+}
+
+cudaError_t launch_small_n(SmallArgs a, void *scratch, int num_sms, double *V, cudaStream_t s)
 {
     if (a.n_pos <= 0 || a.n_pos > kSmallN)
         return cudaErrorInvalidValue;
-    const dim3 grid(n_splits, (a.n_pos + kSmallChunk - 1) / kSmallChunk);
-    small_n_kernel<<<grid, kSmallThreads, 0, s>>>(a);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess)
-        return e;
-    reduce_wide_kernel<<<a.n_pos, kWideThreads, 0, s>>>(a.partial, n_splits, a.n_pos, V);
+    a.g_threads = small_n_threads(a.n_tiles, num_sms, a.n_pos);
+    const int nq = small_nq(a.n_pos);
+    const dim3 grid(small_grid(a.g_threads), (a.n_pos + kSmallChunk - 1) / kSmallChunk);
+    a.part64 = static_cast<double *>(scratch);
+    a.part32 = reinterpret_cast<float2 *>(a.part64 + (size_t)grid.x * grid.y * nq);
+    switch (nq) {
+    case 2: small_n_kernel<2><<<grid, kSmallThreads, 0, s>>>(a, V); break;
+    case 4: small_n_kernel<4><<<grid, kSmallThreads, 0, s>>>(a, V); break;
+    case 8: small_n_kernel<8><<<grid, kSmallThreads, 0, s>>>(a, V); break;
+    default: small_n_kernel<16><<<grid, kSmallThreads, 0, s>>>(a, V); break;
+    }
     return cudaGetLastError();
 }
 

@@ -138,15 +138,16 @@ size_t potential_smem_bytes(int precision, int tile_size);
 // FP32C (64,{2,4}), (128,{1,2,4}), (256,{1,2}).
 bool potential_shape_supported(int precision, int threads, int ppt);
 // Few positions per call (n <= kSmallN): environment entries spread over the
-// threads of n_splits CTAs per chunk of kSmallChunk positions (grid n_splits x
-// chunks), partial[split][n], then one CTA per position sums the partials
-// into V in a fixed order.  Entries are evaluated in FP64, except the FP32
-// point charges (class kClassPoint32) when fp32 is set: those take the
-// compensated FP32 form of the main kernel (hi/lo offsets, symmetric rsqrt,
-// low word of the charge), sum per thread in FP32 and reduce across the CTA
-// as (sum, compensation) pairs before the FP64 partial.
+// threads of one launch, a chunk of up to kSmallChunk positions per CTA row.
+// Entries are evaluated in FP64, except the FP32 point charges (class
+// kClassPoint32) when n_p32 is set: those take the compensated FP32 form of
+// the main kernel (hi/lo offsets, symmetric rsqrt, low word of the charge),
+// sum per thread in FP32 and across threads as (sum, compensation) pairs; the
+// FP64 point charges beside them take the dd form.
 constexpr int kSmallN = 128;
-constexpr int kSmallChunk = 16;      // positions of one CTA, held in registers
+constexpr int kSmallChunk = 16;      // positions of one CTA
+constexpr int kSmallThreads = 512;
+constexpr int kSmallMaxChunks = (kSmallN + kSmallChunk - 1) / kSmallChunk;
 constexpr int kSmallNDistributions = 16; // calls above this many positions take the
                                          // few-position path only for environments of point charges
 struct SmallArgs {
@@ -157,15 +158,26 @@ struct SmallArgs {
     const TileMeta *tiles;
     const double *rec64;
     const float *rec32;
+    const float *recdd;
     const double *boys64;
-    double quantum;        // coordinate grid of the FP32 hi words
-    int fp32;              // FP32 point charges in compensated FP32
+    double quantum, inv_quantum; // coordinate grid of the FP32 hi words
+    float dd_lim;
+    int points_dd;         // FP64 point charges beside FP32 ones: as dd sums
+    int any64;             // some entry is summed in FP64
     int64_t p32_off;       // float offset of the FP32 point records (contiguous, n_p32 of them)
-    int n_p32;
-    double *partial;
+    int n_p32;             // 0: every entry in FP64
+    // the tiles outside the flat FP32 pass: n_other of them, tile o or, from
+    // skip_begin on, o + n_skip, in tile_halves parts of 32 entries each
+    int n_other, skip_begin, n_skip, tile_halves;
+    int *counters;         // [kSmallMaxChunks], zero before and after every launch
+    // set by launch_small_n
+    int g_threads;
+    float2 *part32;
+    double *part64;
 };
-int small_n_splits(int n_tiles, int num_sms, int n);
-cudaError_t launch_small_n(const SmallArgs &a, int n_splits, double *V, cudaStream_t s);
+// scratch of one launch
+size_t small_n_bytes(int n_tiles, int num_sms, int n);
+cudaError_t launch_small_n(SmallArgs a, void *scratch, int num_sms, double *V, cudaStream_t s);
 // perm (optional, from launch_sort): V[perm[slot]] receives the sum of slot
 cudaError_t launch_reduce(const double *partial, int n_splits, int n, double *V, cudaStream_t s,
                           const int *perm = nullptr);
