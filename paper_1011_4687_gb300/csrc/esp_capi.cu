@@ -48,7 +48,7 @@ int esp::choose_splits(const esp_ctx *c, const TileView &v, int n, int prec)
     // against 894 tiles: 128 CTAs of 64 splits left 24 SMs idle and the others
     // with one CTA)
     const int fill = (8 * c->num_sms + blocks - 1) / blocks;
-    s = std::min(s, std::max(64, fill));
+    s = std::min(s, v.labels ? 64 : std::max(64, fill));
     s = std::min(s, std::max(v.n_tiles, 1));
     return std::max(s, 1);
 }
@@ -58,19 +58,34 @@ int esp::view_precision(const esp_ctx *c, const TileView &v)
     return c->opt.precision == ESP_FP64 || (v.n_tiles > 0 && v.n_tiles == v.n_point_tiles) ? 0 : 1;
 }
 
+bool esp::use_td(const esp_ctx *c, const TileView &v, int prec)
+{
+    return prec == 0 && !v.labels && c->recdd.p && c->opt.threads_per_block == 0 && c->opt.positions_per_thread == 0 &&
+           c->opt.pair_splits == 0 && v.n_entries >= kTdMinEntries;
+}
+
 int esp::plan_splits(const esp_ctx *c, const TileView &v, int n, int prec, int max_splits, EvalArgs &a, int &dd_splits)
 {
     a.n_tiles = v.n_tiles;
     a.tiles = v.tiles;
     dd_splits = 0;
-    if (prec == 1 && v.n_dd > 0) // (with few partial sums allowed, at most a quarter of them)
+    if (use_td(c, v, prec)) {
+        a.n_splits = std::min(td_splits(n, v.n_tiles, c->num_sms), max_splits);
+        single_group(a);
+        return a.n_splits;
+    }
+    if (prec == 1 && v.n_dd > 0 && !v.labels) // (with few partial sums allowed, at most a quarter of them)
         dd_splits = std::max(1, std::min(dd_sum_splits(n, v.n_dd, c->num_sms), max_splits / 4));
     const int total = std::max(1, std::min(choose_splits(c, v, n, prec), max_splits - dd_splits));
     a.n_splits = total;
     single_group(a);
-    // the dd kernel takes the point charges: the groups after theirs
-    const int g0 = prec == 1 && v.n_point_tiles > 0 && v.n_groups > 1 ? 1 : 0;
+    // the dd kernel takes the point charges: the groups after theirs (labels:
+    // with the splits that the point charges get beside the others)
+    const int gp = prec == 1 && v.n_point_tiles > 0 && v.n_groups > 1 ? 1 : 0;
+    const int g0 = v.labels ? 0 : gp;
     const int ng = v.n_groups - g0;
+    if (prec == 1 && v.labels && v.n_dd > 0)
+        dd_splits = 1;
     if (prec == 0 || c->opt.pair_splits > 0 || v.n_groups <= 1 || ng > total)
         return dd_splits + total;
     double work = 0.0;
@@ -91,13 +106,17 @@ int esp::plan_splits(const esp_ctx *c, const TileView &v, int n, int prec, int m
         --S[big];
         --sum;
     }
-    a.n_groups = ng;
-    a.grp_split[0] = 0;
-    for (int g = 0; g < ng; ++g) {
-        a.grp_tile[g] = v.grp_tile[g0 + g];
-        a.grp_split[g + 1] = a.grp_split[g] + S[g0 + g];
+    if (v.labels && gp) {
+        dd_splits = S[0];
+        sum -= S[0];
     }
-    a.grp_tile[ng] = v.grp_tile[v.n_groups];
+    a.n_groups = v.n_groups - gp;
+    a.grp_split[0] = 0;
+    for (int g = 0; g < a.n_groups; ++g) {
+        a.grp_tile[g] = v.grp_tile[gp + g];
+        a.grp_split[g + 1] = a.grp_split[g] + S[gp + g];
+    }
+    a.grp_tile[a.n_groups] = v.grp_tile[v.n_groups];
     a.n_splits = sum;
     return dd_splits + sum;
 }
@@ -138,6 +157,8 @@ cudaError_t esp::launch_planned(const esp_ctx *c, const TileView &v, int prec, E
     cudaError_t e = cudaSuccess;
     if (dd_splits > 0 && (e = launch_dd_sum(a, v.dd_list, v.n_dd, dd_splits, s)) != cudaSuccess)
         return e;
+    if (use_td(c, v, prec))
+        return launch_td(a, s);
     a.partial += size_t(dd_splits) * a.n_pos;
     return launch_potential(prec, a, c->threads[prec], c->ppt[prec], s);
 }
@@ -154,9 +175,9 @@ std::vector<int> esp::dd_tile_list(const std::vector<TileMeta> &T, bool near)
 void esp::set_tile_groups(const std::vector<TileMeta> &T, TileView &v)
 {
     // FP32 operations per evaluation by L (the kernel's algorithmic count) and
-    // an FP64 point charge (in pairs of FP32 numbers), for the split of the work between groups
+    // a point charge, for the split of the work between groups
     static const double kCost[kMaxL + 1] = {10.0, 26.0, 52.0, 95.0, 170.0};
-    const double kPointCost = 54.0, kPoint32Cost = 10.0;
+    const double kPointCost = 12.0, kPoint32Cost = 10.0;
     v.n_tiles = int(T.size());
     int64_t n_small = 0, n_all = 0;
     v.n_p32 = 0;
@@ -181,6 +202,7 @@ void esp::set_tile_groups(const std::vector<TileMeta> &T, TileView &v)
             contiguous = false;
         n_small += m.n;
     }
+    v.n_entries = n_all;
     v.point_heavy = n_all > 0 && n_small * 10 >= n_all * 9;
     v.n_p32 = contiguous ? int(n_small) : 0;
     v.n_groups = 1;
@@ -253,7 +275,7 @@ esp_status pipeline(esp_ctx *c, const TileView &v, int prec, const double *d_pos
     }
     // FP32C with many positions: stage them in spatial order (the kernel's
     // warp-uniform far/near votes then see compact groups of positions)
-    const bool sorted = !small_n && prec == 1 && n >= kSortMinPositions;
+    const bool sorted = !small_n && (prec == 1 ? n >= kSortMinPositions : use_td(c, v, prec) && n >= kSortMinTd);
     if (sorted && (e = c->sortbuf.ensure(sort_scratch_ints(int(n)) * sizeof(int))) != cudaSuccess)
         return cuda_fail(e, "allocating the position order");
     const Staged stg = staged_at(c->stage.p, size_t(n));
@@ -292,7 +314,7 @@ esp_status pipeline(esp_ctx *c, const TileView &v, int prec, const double *d_pos
     }
     if (timing && (e = cudaEventRecord(c->ev[2], s)) != cudaSuccess)
         return cuda_fail(e, "recording a timing event");
-    if ((!small_n || v.n_tiles == 0) && (e = launch_reduce(a.partial, splits, int(n), dV, s, perm)) != cudaSuccess)
+    if ((!small_n || v.n_tiles == 0) && (e = launch_reduce(a.partial, splits, int(n), dV, s, perm, v.labels)) != cudaSuccess)
         return cuda_fail(e, "launching the partial-sum reduction");
     if (dE && (e = launch_walkers(dV, int(n_walkers), int(n_elec), dE, s)) != cudaSuccess)
         return cuda_fail(e, "launching the walker-energy reduction");

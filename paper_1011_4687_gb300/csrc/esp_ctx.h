@@ -151,6 +151,11 @@ struct TileView {
     const int *dd_list = nullptr;
     int n_dd = 0;
     int n_point_tiles = 0;
+    int64_t n_entries = 0;
+    // labels of a training: the sums of the FP64 and FP32C kernels in one fixed
+    // grouping and order (Adam turns a changed last bit of a target into a
+    // changed weight, so the grouping must not follow the tuning of the others)
+    bool labels = false;
     bool points_have_dd = true; // every FP64 point tile has dd records
     bool point_heavy = false; // >= 90 % of the entries are FP32 point charges
     // FP32 point charges of the view: their records are contiguous in rec32
@@ -204,6 +209,10 @@ int choose_splits(const esp_ctx *c, const TileView &v, int n, int prec);
 // Precision of an evaluation of the view (0 FP64, 1 FP32C): FP64 point charges
 // alone stay FP64 under FP32C, where no FP32 sum hides the 48 bits of a dd term.
 int view_precision(const esp_ctx *c, const TileView &v);
+// FP64 evaluations by launch_td: default launch shape, dd records, and enough
+// entries (kTdMinEntries) that its order of summation is no worse than FP64's.
+constexpr int kTdMinEntries = 512;
+bool use_td(const esp_ctx *c, const TileView &v, int prec);
 // Fills the deal of the view's tiles (n_splits and the tile groups) for n
 // positions, with at most max_splits partial sums; returns their number.  FP32C
 // deals each tile group to its own splits, in proportion to the group's work;

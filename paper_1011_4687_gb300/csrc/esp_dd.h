@@ -27,10 +27,11 @@
 // A dd tile holds word w of record j at w * n4 + j, n4 = n rounded up to 4 (the
 // padding repeats the last record's coordinates with zero coefficients):
 //   0..2 h(x, y, z)   3..5 m   6..8 l
-//   points:        9 Z (h), 10 Z (l)
-//   distributions: far block [9, 9 + 2 nh): coefficients h, then l;
-//                  L <= 2: general block of 2 + 2 nh words: sqrt(p) h, l,
-//                  sqrt(pi)/2 G h, then l (nh = number of Hermite coefficients).
+//   points:        9..11 Z (three words), 12 (Z - word 9) / word 9
+//   distributions: far block [9, 11 + 2 nh): the monopole's third word, p, then
+//                  the coefficients h, then l (nh = number of Hermite coefficients);
+//                  L <= 2, near-capable tiles: general block of 2 + 2 nh words: sqrt(p) h, l,
+//                  sqrt(pi)/2 G h, then l.
 #pragma once
 
 #include "esp_internal.h"
@@ -41,15 +42,20 @@ constexpr int kDdGeneralMaxL = 2;         // larger L takes the FP64 code when n
 constexpr double kDdMinDist = 0x1p-10;    // closer offsets may lack the 48 bits: FP64
 constexpr float kDdMinR2 = 0x1p-20f;
 ESP_HD constexpr int dd_pad(int n) { return (n + 3) & ~3; }
-ESP_HD constexpr int dd_far_words(int L) { return 9 + 2 * num_hermite(L); }
+constexpr int kDdPointWords = 13;
+ESP_HD constexpr int dd_far_words(int L) { return 11 + 2 * num_hermite(L); }
 ESP_HD constexpr int dd_gen_words(int L) { return L <= kDdGeneralMaxL ? 2 + 2 * num_hermite(L) : 0; }
-ESP_HD constexpr int dd_words(int cls)
+// does a tile hold the general block (it can be near a position of an FP32C call)?
+ESP_HD bool dd_has_general(const TileMeta &m)
 {
-    return is_point_class(cls) ? 11 : dd_far_words(cls & 7) + dd_gen_words(cls & 7);
+    return m.cls <= kDdGeneralMaxL && m.vmax >= kNearVmax;
 }
-// words staged in shared memory at most: coordinates and one of the two blocks
-ESP_HD constexpr int dd_stage_words(int L) { return dd_far_words(L) > 9 + dd_gen_words(L) ? dd_far_words(L) : 9 + dd_gen_words(L); }
-constexpr int kDdStageWords = 80; // >= dd_stage_words of every class
+ESP_HD int dd_words(const TileMeta &m)
+{
+    if (is_point_class(m.cls))
+        return kDdPointWords;
+    return dd_far_words(m.cls & 7) + (dd_has_general(m) ? dd_gen_words(m.cls & 7) : 0);
+}
 
 // Boys table of the dd general form: rows at T_i = i / 64 up to 45, F_0..F_8 in
 // units of sqrt(pi)/2 in FP32, then the low words of F_0..F_4, pad: 16 floats (one 64-byte line).
@@ -265,7 +271,7 @@ ESP_HD void dd_project(double *c)
 
 // The dd words of one FP64 record r of class cls, word w to out[w * n4].
 template <int L>
-ESP_HD void dd_convert_dist(const double *r, bool shortr, float *out, int n4)
+ESP_HD void dd_convert_dist(const double *r, bool shortr, bool general, float *out, int n4)
 {
     constexpr int nh = num_hermite(L);
     double M[nh];
@@ -285,30 +291,40 @@ ESP_HD void dd_convert_dist(const double *r, bool shortr, float *out, int n4)
     if constexpr (L >= 4)
         dd_project<4>(M + 20);
     for (int k = 0; k < nh; ++k)
-            dd_split2(M[k], out[(9 + k) * n4], out[(9 + nh + k) * n4]);
-    if constexpr (L <= kDdGeneralMaxL) {
-        constexpr int go = 9 + 2 * nh;
+        dd_split2(M[k], out[(11 + k) * n4], out[(11 + nh + k) * n4]);
+    out[9 * n4] = float(M[0] - double(out[11 * n4]) - double(out[(11 + nh) * n4]));
+    out[10 * n4] = float(r[3] * r[3]);
+    if (L <= kDdGeneralMaxL && general) {
+        constexpr int go = dd_far_words(L);
         dd_split2(L == 0 ? r[3] * r[3] : r[3], out[go * n4], out[(go + 1) * n4]);
         for (int k = 0; k < nh; ++k)
             dd_split2(r[4 + k] * 0.88622692545275801365, out[(go + 2 + k) * n4], out[(go + 2 + nh + k) * n4]);
     }
 }
 
-ESP_HD void dd_convert(int cls, const double *r, double q, float *out, int n4)
+ESP_HD void dd_convert(const TileMeta &m, const double *r, double q, float *out, int n4)
 {
+    const int cls = m.cls;
+    const bool gen = dd_has_general(m);
     for (int d = 0; d < 3; ++d)
         dd_split3(r[d], q, 1.0 / q, out[d * n4], out[(3 + d) * n4], out[(6 + d) * n4]);
     const bool sh = (cls & kClassShortBit) != 0;
     if (is_point_class(cls)) {
-        dd_split_rel(r[3], out[9 * n4], out[10 * n4]);
+        float h, rho, l;
+        dd_split_rel(r[3], h, rho);
+        dd_split2(r[3], h, l);
+        out[9 * n4] = h;
+        out[10 * n4] = l;
+        out[11 * n4] = float(r[3] - double(h) - double(l));
+        out[12 * n4] = rho;
         return;
     }
     switch (cls & 7) {
-    case 0: dd_convert_dist<0>(r, sh, out, n4); break;
-    case 1: dd_convert_dist<1>(r, sh, out, n4); break;
-    case 2: dd_convert_dist<2>(r, sh, out, n4); break;
-    case 3: dd_convert_dist<3>(r, sh, out, n4); break;
-    default: dd_convert_dist<4>(r, sh, out, n4); break;
+    case 0: dd_convert_dist<0>(r, sh, gen, out, n4); break;
+    case 1: dd_convert_dist<1>(r, sh, gen, out, n4); break;
+    case 2: dd_convert_dist<2>(r, sh, gen, out, n4); break;
+    case 3: dd_convert_dist<3>(r, sh, gen, out, n4); break;
+    default: dd_convert_dist<4>(r, sh, gen, out, n4); break;
     }
 }
 
@@ -343,15 +359,15 @@ ESP_HD void td_acc(f2 &b, f2 &c, f2 x)
 }
 ESP_HD Td td_norm2(const TdOff &x, const TdOff &y, const TdOff &z)
 {
-    f2 ex, ey, ez, e1, e2, fx, fy, fz;
+    f2 ex, ey, ez, e1, e2, fx, fy, fz, e;
     const f2 px = two_prod(x.s, x.s, ex), py = two_prod(y.s, y.s, ey), pz = two_prod(z.s, z.s, ez);
     const f2 x2 = x.s + x.s, y2 = y.s + y.s, z2 = z.s + z.s;
     const f2 qx = two_prod(x2, x.e, fx), qy = two_prod(y2, y.e, fy), qz = two_prod(z2, z.e, fz);
     f2 a = two_sum(px, py, e1);
     a = two_sum(a, pz, e2);
-    f2 c = esp_fma(x2, x.l, esp_fma(x.e, x.e, fx)) + esp_fma(y2, y.l, esp_fma(y.e, y.e, fy)) +
-           esp_fma(z2, z.l, esp_fma(z.e, z.e, fz));
-    f2 b = qx, e;
+    f2 c = esp_fma(x2, x.l, esp_fma(x.e, x.e, fx)) +
+           (esp_fma(y2, y.l, esp_fma(y.e, y.e, fy)) + esp_fma(z2, z.l, esp_fma(z.e, z.e, fz)));
+    f2 b = qx;
     td_acc(b, c, qy);
     td_acc(b, c, qz);
     td_acc(b, c, ex);
@@ -362,36 +378,60 @@ ESP_HD Td td_norm2(const TdOff &x, const TdOff &y, const TdOff &z)
     a = fast_two_sum(a, b, e);
     return {a, e, c};
 }
-// z / sqrt(r2) for z = zh + zl: h + m with m holding everything below the
-// leading product; y receives 1 / sqrt(r2) to 48 bits.
-ESP_HD dd td_div_sqrt(f2 zh, f2 zl, const Td &r2, dd &y48)
-{
-    const f2 y = esp_rsqrt(r2.a);
-    f2 pe, qe, fe, ge, he, ze;
-    const f2 p = two_prod(y, y, pe);
-    const f2 q = two_prod(r2.a, p, qe);
-    const f2 t1 = q - f2(1.0f); // exact
-    const f2 f = two_prod(r2.a, pe, fe), g = two_prod(r2.b, p, ge);
-    const f2 mid = (qe + f) + g;
-    const f2 low = esp_fma(r2.b, pe, esp_fma(r2.c, p, fe + ge));
-    const f2 t = t1 + mid;
-    // 1 / sqrt = y (1 - t/2 + 3/8 t^2)
-    const f2 u3 = esp_fma(0.375f * t, t, -0.5f * low);
-    const f2 u1 = -0.5f * t1, u2 = -0.5f * mid;
-    y48 = {y, y * (u1 + (u2 + u3))};
-    const f2 v = two_prod(zh, y, ze);
-    const f2 h = two_prod(v, u1, he);
-    // (rounded sums of terms near 2^-25 of v, smallest first)
-    const f2 lo = esp_fma(v, u2, ze) + esp_fma(zl, y, esp_fma(v, u3, he));
-    return {v, h + lo};
-}
+// Sum of three-word values over a few records: a the leading products, b what
+// lies about 2^-24 below, c the roundings of both.
+struct TdSum {
+    f2 a, b, c;
+    ESP_HD void clear() { a = b = c = f2(0.0f); }
+    ESP_HD void mid(f2 x) { td_acc(b, c, x); }
+    // add z / sqrt(r2) for z = zh + zl + zm; returns 1 / sqrt(r2) to 48 bits
+    ESP_HD dd div_sqrt(f2 zh, f2 zl, f2 zm, const Td &r2)
+    {
+        const f2 y = esp_rsqrt(r2.a);
+        f2 pe, qe, fe, ge, he, ze, ke, le, e;
+        const f2 p = two_prod(y, y, pe);
+        const f2 q = two_prod(r2.a, p, qe);
+        const f2 t1 = q - f2(1.0f); // exact
+        // t = r2 y^2 - 1 = t1 + mid + low
+        const f2 f = two_prod(r2.a, pe, fe), g = two_prod(r2.b, p, ge);
+        f2 low = esp_fma(r2.b, pe, esp_fma(r2.c, p, fe + ge)), md = qe;
+        td_acc(md, low, f);
+        td_acc(md, low, g);
+        // 1 / sqrt = y (1 - t/2 + 3/8 t^2)
+        const f2 t = t1 + md;
+        const f2 u3 = esp_fma(0.375f * t, t, -0.5f * low);
+        const f2 u1 = -0.5f * t1, u2 = -0.5f * md;
+        const f2 v = two_prod(zh, y, ze);
+        const f2 h = two_prod(v, u1, he), k = two_prod(v, u2, ke), l = two_prod(zl, y, le);
+        a = two_sum(a, v, e);
+        mid(e);
+        mid(h);
+        mid(k);
+        mid(l);
+        mid(ze);
+        const f2 u = u1 + u2;
+        c += esp_fma(v, u3, esp_fma(l + ze, u, esp_fma(zm, y, (he + ke) + le)));
+        return {y, y * (u + u3)};
+    }
+    ESP_HD void add(const dd &x)
+    {
+        f2 e;
+        a = two_sum(a, x.h, e);
+        mid(e);
+        mid(x.l);
+    }
+    ESP_HD double total() const
+    {
+        return ((double)a.x + (double)a.y) + (((double)b.x + (double)b.y) + (double)(c.x + c.y));
+    }
+};
 
 // padding records: zero every coefficient (the exponent words stay)
-ESP_HD void dd_zero_coefficients(int cls, float *out, int n4)
+ESP_HD void dd_zero_coefficients(const TileMeta &m, float *out, int n4)
 {
-    const int L = cls & 7, far_end = is_point_class(cls) ? 11 : dd_far_words(L);
-    for (int w = 9; w < dd_words(cls); ++w)
-        if (w < far_end || w >= far_end + 2)
+    const int far_end = is_point_class(m.cls) ? kDdPointWords : dd_far_words(m.cls & 7);
+    for (int w = 9; w < dd_words(m); ++w)
+        if (is_point_class(m.cls) || (w != 10 && w != far_end && w != far_end + 1))
             out[w * n4] = 0.0f;
 }
 
@@ -430,25 +470,30 @@ ESP_HD dd dd_point(const DdTile &t, int j, const DdPos &c, f2 &r2)
     dd_offsets(t, j, c, d);
     const dd s = dd_norm2(d[0], d[1], d[2]);
     r2 = s.h;
-    return dd_div_sqrt(t(9, j), t(10, j), s);
+    return dd_div_sqrt(t(9, j), t(12, j), s);
 }
 
 // Far form of distributions j, j + 1, the monopole at FP64 accuracy and the
-// higher orders (which fall off as (size / distance)^N) in 48 bits.
+// higher orders (which fall off as (size / distance)^N) in 48 bits, added to
+// sum.  Lanes with use = 0 add nothing, whatever their offset; r2 receives
+// |P - C|^2 (1 for those).
 template <int L>
-ESP_HD dd dd_far(const DdTile &t, int j, const DdPos &c)
+ESP_HD void td_far(const DdTile &t, int j, const DdPos &c, bool use0, bool use1, TdSum &sum, f2 &r2)
 {
     constexpr int nh = num_hermite(L);
     TdOff o[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k)
         o[k] = td_offset(t(k, j), t(3 + k, j), t(6 + k, j), c.h[k], c.m[k], c.l[k]);
-    dd y;
-    const dd v = td_div_sqrt(t(9, j), t(9 + nh, j), td_norm2(o[0], o[1], o[2]), y);
-    if constexpr (L == 0) {
-        return v;
-    } else {
-        auto coef = [&](int k) { return dd{t(9 + k, j), t(9 + nh + k, j)}; };
+    Td s = td_norm2(o[0], o[1], o[2]);
+    s.a = f2(use0 ? s.a.x : 1.0f, use1 ? s.a.y : 1.0f);
+    s.b = f2(use0 ? s.b.x : 0.0f, use1 ? s.b.y : 0.0f);
+    s.c = f2(use0 ? s.c.x : 0.0f, use1 ? s.c.y : 0.0f);
+    r2 = s.a;
+    const f2 w(use0 ? 1.0f : 0.0f, use1 ? 1.0f : 0.0f);
+    const dd y = sum.div_sqrt(w * t(11, j), w * t(11 + nh, j), w * t(9, j), s);
+    if constexpr (L > 0) {
+        auto coef = [&](int k) { return dd{t(11 + k, j), t(11 + nh + k, j)}; };
         dd d[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k)
@@ -473,8 +518,20 @@ ESP_HD dd dd_far(const DdTile &t, int j, const DdPos &c)
             }
             a = dd_add(dd_form<1>(d[0], d[1], d[2], [&](int k) { return coef(1 + k); }), dd_mul(i2, b));
         }
-        return dd_add(v, dd_mul(dd_mul(i2, a), y));
+        const dd v = dd_mul(dd_mul(i2, a), y);
+        sum.add(dd{w * v.h, w * v.l});
     }
+}
+// Point charges j, j + 1 at FP64 accuracy.
+ESP_HD void td_point(const DdTile &t, int j, const DdPos &c, TdSum &sum, f2 &r2)
+{
+    TdOff o[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        o[k] = td_offset(t(k, j), t(3 + k, j), t(6 + k, j), c.h[k], c.m[k], c.l[k]);
+    const Td s = td_norm2(o[0], o[1], o[2]);
+    r2 = s.a;
+    sum.div_sqrt(t(9, j), t(10, j), t(11, j), s);
 }
 
 // F_0..F_L of one lane's T (h + l, below kBoysDdTmax) from the table: Taylor
@@ -524,7 +581,7 @@ ESP_HD void boys_dd(float Th, float Tl, const float *__restrict__ tab, float (&F
 
 // General form of distributions j, j + 1 (L <= 2, not the short-range kind,
 // whose difference from the monopole needs FP64).  go: word of the general
-// block; for L = 0 also reads the far block (words 9, 10).
+// block; for L = 0 also reads the far block (words 11, 12).
 template <int L>
 ESP_HD dd dd_general(const DdTile &t, int j, const DdPos &c, int go, const float *__restrict__ tab)
 {
@@ -536,7 +593,7 @@ ESP_HD dd dd_general(const DdTile &t, int j, const DdPos &c, int go, const float
     auto G = [&](int k) { return dd{t(go + 2 + k, j), t(go + 2 + nh + k, j)}; };
     if constexpr (L == 0) {
         const dd r2 = dd_norm2(x[0], x[1], x[2]);
-        dd v = dd_mul({t(9, j), t(10, j)}, dd_rsqrt(r2)); // asymptotic form
+        dd v = dd_mul({t(11, j), t(12, j)}, dd_rsqrt(r2)); // asymptotic form
         const dd T = dd_norm(dd_mul(sp, r2));
         const bool a0 = T.h.x >= kBoysDdTmax, a1 = T.h.y >= kBoysDdTmax;
         if (!(a0 && a1)) {

@@ -17,7 +17,7 @@ namespace esp {
 namespace {
 
 constexpr int kDdThreads = 128;
-constexpr int kDdWordsMax = dd_words(kDdGeneralMaxL); // the largest tile staged here
+constexpr int kDdWordsMax = dd_far_words(kDdGeneralMaxL) + dd_gen_words(kDdGeneralMaxL); // the largest tile staged
 
 __global__ void __launch_bounds__(kDdThreads, 4) dd_sum_kernel(EvalArgs a, const int *__restrict__ list, int n_list)
 {
@@ -36,15 +36,20 @@ __global__ void __launch_bounds__(kDdThreads, 4) dd_sum_kernel(EvalArgs a, const
         // (also: the previous tile is fully consumed)
         if (!__syncthreads_or(mine))
             continue;
-        if (m.offdd < 0) {
-            if (mine)
-                acc += pts ? point_tile_f64(a.rec64 + m.off64, m.n, a.pos.x64[ic], a.pos.y64[ic], a.pos.z64[ic])
-                           : tile_f64_one_any(m.cls, a.rec64 + m.off64, m.n, a.pos.x64[ic], a.pos.y64[ic],
-                                              a.pos.z64[ic], a.boys64);
+        if (m.offdd < 0 || !(pts || dd_has_general(m))) {
+            if (pts) { // (one chain of additions over the tiles)
+                const double p[1][3] = {{a.pos.x64[ic], a.pos.y64[ic], a.pos.z64[ic]}};
+                double v[1] = {acc};
+                tile_points_f64<1>(a.rec64 + m.off64, m.n, p, v);
+                acc = v[0];
+            } else if (mine) {
+                acc += tile_f64_one_any(m.cls, a.rec64 + m.off64, m.n, a.pos.x64[ic], a.pos.y64[ic], a.pos.z64[ic],
+                                        a.boys64);
+            }
             continue;
         }
         const int n4 = dd_pad(m.n);
-        copy_tile(smem4, reinterpret_cast<const float4 *>(a.recdd) + m.offdd, dd_words(m.cls) * n4 / 4);
+        copy_tile(smem4, reinterpret_cast<const float4 *>(a.recdd) + m.offdd, dd_words(m) * n4 / 4);
         __syncthreads();
         if (pts) {
             float r2min;
@@ -65,6 +70,137 @@ __global__ void __launch_bounds__(kDdThreads, 4) dd_sum_kernel(EvalArgs a, const
         a.partial[(size_t)blockIdx.y * a.n_pos + i] = acc;
 }
 
+// ---------------------------------------------------------------------------
+// FP64 evaluations.  Every entry whose Gaussian is negligible at the positions
+// of a warp (T = p |P - C|^2 >= 45 and a margin) takes the far form of esp_dd.h:
+// the monopole in three FP32 words (an error of 1e-20 of the term), the higher
+// orders in two; the others take the FP64 code for the warp.  Bound by the FP32
+// pipe (about 200 packed operations per two monopoles) and, where exponents are
+// small, by the FP64 pipe (near entries: some 40 operations of 64 cycles).
+// ---------------------------------------------------------------------------
+constexpr int kTdWordsMax = dd_far_words(kMaxL);
+constexpr float kTdNearT = 46.0f; // (T from the hi words: 1e-2 relative at most beyond kDdMinR2)
+
+// The far pairs of a chunk of at most 64 records; near: bits of the records to
+// leave out.  lo: the smallest |P - C|^2 met.
+template <int L>
+__device__ __noinline__ double td_chunk(const float *__restrict__ s_rec, int n4, int j0, int j1, const DdPos c,
+                                        unsigned long long near, float *lo)
+{
+    const DdTile t = {s_rec, n4};
+    double acc = 0.0;
+    float r2min = *lo;
+    for (int b = j0; b < j1; b += 16) {
+        TdSum sum;
+        sum.clear();
+        const int e = min(j1, b + 16);
+#pragma unroll 1
+        for (int j = b; j < e; j += 2) {
+            const bool u0 = !(near >> (j - j0) & 1), u1 = !(near >> (j - j0 + 1) & 1);
+            if (!u0 && !u1)
+                continue;
+            f2 r2;
+            td_far<L>(t, j, c, u0, u1, sum, r2);
+            r2min = fminf(r2min, fminf(r2.x, r2.y));
+        }
+        acc += sum.total();
+    }
+    *lo = r2min;
+    return acc;
+}
+__device__ __noinline__ double td_points(const float *__restrict__ s_rec, int n4, const DdPos c, float *lo)
+{
+    const DdTile t = {s_rec, n4};
+    double acc = 0.0;
+    float r2min = *lo;
+    for (int b = 0; b < n4; b += 16) {
+        TdSum sum;
+        sum.clear();
+        const int e = min(n4, b + 16);
+#pragma unroll 1
+        for (int j = b; j < e; j += 2) {
+            f2 r2;
+            td_point(t, j, c, sum, r2);
+            r2min = fminf(r2min, fminf(r2.x, r2.y));
+        }
+        acc += sum.total();
+    }
+    *lo = r2min;
+    return acc;
+}
+__device__ __noinline__ double near_entry(int cls, const double *__restrict__ r, double x, double y, double z,
+                                          const double *__restrict__ boys64)
+{
+    return tile_f64_one_any(cls, r, 1, x, y, z, boys64);
+}
+
+__global__ void __launch_bounds__(kDdThreads, 4) potential_td_kernel(EvalArgs a)
+{
+    extern __shared__ float4 smem4[];
+    const float *s_rec = reinterpret_cast<const float *>(smem4);
+    const int i = blockIdx.x * kDdThreads + threadIdx.x, ic = min(i, a.n_pos - 1);
+    const DdPos c = dd_position(a.pos, ic);
+    const double x = a.pos.x64[ic], y = a.pos.y64[ic], z = a.pos.z64[ic];
+    const bool in_range = dd_in_range(c.h, a.dd_lim);
+    double S = 0.0, Cc = 0.0;
+    for (int k = blockIdx.y; k < a.n_tiles; k += gridDim.y) {
+        const TileMeta m = a.tiles[k];
+        const bool pts = is_point_class(m.cls);
+        const double *rec64 = a.rec64 + m.off64;
+        if (m.offdd < 0) {
+            two_sum_acc(S, Cc, pts ? point_tile_f64(rec64, m.n, x, y, z)
+                                   : tile_f64_one_any(m.cls, rec64, m.n, x, y, z, a.boys64));
+            continue;
+        }
+        const int n4 = dd_pad(m.n), L = m.cls & 7;
+        __syncthreads(); // the previous tile is fully consumed
+        copy_tile(smem4, reinterpret_cast<const float4 *>(a.recdd) + m.offdd,
+                  (pts ? kDdPointWords : dd_far_words(L)) * n4 / 4);
+        __syncthreads();
+        float r2min = 1.0f;
+        double v = 0.0;
+        if (pts) {
+            v = td_points(s_rec, n4, c, &r2min);
+        } else {
+            const float ex = c.h[0] - m.cx, ey = c.h[1] - m.cy, ez = c.h[2] - m.cz;
+            const float d = sqrtf(ex * ex + ey * ey + ez * ez) - m.rad;
+            const bool far = __all_sync(0xffffffffu, d > 0.0f && m.pmin * d * d >= kTdNearT);
+            const DdTile t = {s_rec, n4};
+            for (int j0 = 0; j0 < n4; j0 += 64) {
+                const int j1 = min(n4, j0 + 64);
+                unsigned long long near = 0ull;
+                if (!far) { // which records are near any of the warp's positions
+                    for (int j = j0; j < j1; j += 2) {
+                        const f2 dx = t(0, j) - f2(c.h[0]), dy = t(1, j) - f2(c.h[1]), dz = t(2, j) - f2(c.h[2]);
+                        const f2 T = t(10, j) * esp_fma(dx, dx, esp_fma(dy, dy, dz * dz));
+                        const unsigned b0 = __any_sync(0xffffffffu, !(T.x >= kTdNearT)),
+                                       b1 = __any_sync(0xffffffffu, !(T.y >= kTdNearT));
+                        near |= (unsigned long long)((b0 ? 1u : 0u) | (b1 ? 2u : 0u)) << (j - j0);
+                    }
+                }
+                switch (L) {
+                case 0: v += td_chunk<0>(s_rec, n4, j0, j1, c, near, &r2min); break;
+                case 1: v += td_chunk<1>(s_rec, n4, j0, j1, c, near, &r2min); break;
+                case 2: v += td_chunk<2>(s_rec, n4, j0, j1, c, near, &r2min); break;
+                case 3: v += td_chunk<3>(s_rec, n4, j0, j1, c, near, &r2min); break;
+                default: v += td_chunk<4>(s_rec, n4, j0, j1, c, near, &r2min); break;
+                }
+                for (unsigned long long b = near; b; b &= b - 1) {
+                    const int j = j0 + __ffsll((long long)b) - 1;
+                    if (j < m.n) // (padding repeats the last record)
+                        v += near_entry(m.cls, rec64 + (size_t)j * rec64_stride(L), x, y, z, a.boys64);
+                }
+            }
+        }
+        // closer than the words resolve, or out of their range
+        if (!(r2min >= kDdMinR2) || !in_range)
+            v = pts ? point_tile_f64(rec64, m.n, x, y, z) : tile_f64_one_any(m.cls, rec64, m.n, x, y, z, a.boys64);
+        two_sum_acc(S, Cc, v);
+    }
+    if (i < a.n_pos)
+        a.partial[(size_t)blockIdx.y * a.n_pos + i] = S + Cc;
+}
+
 // dd records of one tile per CTA; the padding repeats the last record's
 // coordinates with zero coefficients
 __global__ void dd_build_kernel(const TileMeta *__restrict__ tiles, const double *__restrict__ rec64, double q,
@@ -77,9 +213,9 @@ __global__ void dd_build_kernel(const TileMeta *__restrict__ tiles, const double
     const int n4 = dd_pad(m.n), st = pts ? kPointStride64 : rec64_stride(m.cls & 7);
     float *out = recdd + (size_t)m.offdd * 4;
     for (int j = threadIdx.x; j < n4; j += blockDim.x) {
-        dd_convert(m.cls, rec64 + m.off64 + (size_t)min(j, m.n - 1) * st, q, out + j, n4);
+        dd_convert(m, rec64 + m.off64 + (size_t)min(j, m.n - 1) * st, q, out + j, n4);
         if (j >= m.n)
-            dd_zero_coefficients(m.cls, out + j, n4);
+            dd_zero_coefficients(m, out + j, n4);
     }
 }
 
@@ -103,6 +239,28 @@ cudaError_t launch_dd_sum(const EvalArgs &a, const int *list, int n_list, int n_
         return e;
     const dim3 grid((a.n_pos + kDdThreads - 1) / kDdThreads, n_splits);
     dd_sum_kernel<<<grid, kDdThreads, smem, s>>>(a, list, n_list);
+    return cudaGetLastError();
+}
+
+int td_splits(int n, int n_tiles, int num_sms)
+{
+    const int blocks = (n + kDdThreads - 1) / kDdThreads;
+    // 16 CTAs per SM where the tiles allow it; not more partial sums than 64
+    // where the blocks alone give every SM several
+    const int fill = (16 * num_sms + blocks - 1) / blocks;
+    return std::max(1, std::min(n_tiles, std::min(fill, std::max(64, (8 * num_sms + blocks - 1) / blocks))));
+}
+
+cudaError_t launch_td(const EvalArgs &a, cudaStream_t s)
+{
+    if (a.n_pos <= 0)
+        return cudaSuccess;
+    const size_t smem = (size_t)a.tile_size * kTdWordsMax * sizeof(float);
+    cudaError_t e = cudaFuncSetAttribute(potential_td_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess)
+        return e;
+    const dim3 grid((a.n_pos + kDdThreads - 1) / kDdThreads, a.n_splits);
+    potential_td_kernel<<<grid, kDdThreads, smem, s>>>(a);
     return cudaGetLastError();
 }
 

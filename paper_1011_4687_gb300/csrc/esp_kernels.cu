@@ -762,13 +762,16 @@ cudaError_t launch_small_n(SmallArgs a, void *scratch, int num_sms, double *V, c
     return cudaGetLastError();
 }
 
-cudaError_t launch_reduce(const double *partial, int n_splits, int n, double *V, cudaStream_t s, const int *perm)
+cudaError_t launch_reduce(const double *partial, int n_splits, int n, double *V, cudaStream_t s, const int *perm,
+                          bool in_order)
 {
     if (n <= 0)
         return cudaSuccess;
     const int grid = (n + 31) / 32;
     // more slices where the partials are many and the positions few
-    if (n_splits > 64)
+    if (in_order)
+        reduce_kernel<1><<<grid, 32, 0, s>>>(partial, n_splits, n, V, perm);
+    else if (n_splits > 64)
         reduce_kernel<32><<<grid, 32 * 32, 0, s>>>(partial, n_splits, n, V, perm);
     else
         reduce_kernel<8><<<grid, 32 * 8, 0, s>>>(partial, n_splits, n, V, perm);

@@ -111,6 +111,10 @@ bool batch_shape_supported(int precision, int threads, int ppt);
 // partial sums from a.partial on (esp_ddsum.cu).
 int dd_sum_splits(int n, int n_list, int num_sms);
 cudaError_t launch_dd_sum(const EvalArgs &a, const int *list, int n_list, int n_splits, cudaStream_t s);
+// All tiles at FP64 accuracy into a.n_splits partial sums (esp_ddsum.cu): far
+// entries in FP32 words, the others in FP64.
+int td_splits(int n, int n_tiles, int num_sms);
+cudaError_t launch_td(const EvalArgs &a, cudaStream_t s);
 // dd records (esp_dd.h) of the tiles with offdd >= 0, on the coordinate grid q
 cudaError_t launch_dd_build(const TileMeta *tiles, int n_tiles, const double *rec64, double q, float *recdd,
                             cudaStream_t s);
@@ -128,6 +132,7 @@ constexpr int kSortThreads = 1024;
 constexpr int kSortCtas = 8; // the cluster that orders one call's positions
 constexpr double kSortHalf = 8.0;
 constexpr int kSortMinPositions = 4096; // fewer: the order is not worth its three launches
+constexpr int kSortMinTd = 512;        // FP64: compact warps have fewer near entries
 size_t sort_scratch_ints(int n);
 cudaError_t launch_sort(const double *pos_in, int n, const double center[3], int *scratch, int **slot_of, int **perm,
                         cudaStream_t s);
@@ -179,8 +184,9 @@ struct SmallArgs {
 size_t small_n_bytes(int n_tiles, int num_sms, int n);
 cudaError_t launch_small_n(SmallArgs a, void *scratch, int num_sms, double *V, cudaStream_t s);
 // perm (optional, from launch_sort): V[perm[slot]] receives the sum of slot
+// in_order: the partials one after the other (else several chains, joined)
 cudaError_t launch_reduce(const double *partial, int n_splits, int n, double *V, cudaStream_t s,
-                          const int *perm = nullptr);
+                          const int *perm = nullptr, bool in_order = false);
 cudaError_t launch_walkers(const double *V, int n_walkers, int n_elec, double *E, cudaStream_t s);
 
 } // namespace esp

@@ -92,7 +92,7 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
         const float4 *s_dd = reinterpret_cast<const float4 *>(a.recdd) + (ddt ? m.offdd : 0);
         const float4 *src = pts ? (ddt ? s_dd : reinterpret_cast<const float4 *>(a.rec64 + m.off64))
                                 : reinterpret_cast<const float4 *>(a.rec32 + m.off32);
-        const int nvec = pts ? (ddt ? dd_words(kClassPoint) * n4 / 4 : m.n * 2)
+        const int nvec = pts ? (ddt ? kDdPointWords * n4 / 4 : m.n * 2)
                              : (m.n * rec32_stride_cls(m.cls)) / 4;
         copy_tile(s_tile4, src, nvec);
         __syncthreads();
@@ -263,12 +263,12 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
         }
         if (!ALL || m.vmax < kNearVmax || !(near_r > 0.0f))
             continue; // (block-uniform) no position can be near
-        if (ddt) {
+        if (ddt && dd_has_general(m)) {
             // the CTA stages the tile's dd records; a warp with a near lane
             // sums them at its positions
             if (!__syncthreads_or(any_near))
                 continue;
-            copy_tile(s_tile4, s_dd, dd_words(m.cls) * n4 / 4);
+            copy_tile(s_tile4, s_dd, dd_words(m) * n4 / 4);
             __syncthreads();
             const float *s_rec_dd = reinterpret_cast<const float *>(s_tile4);
 #pragma unroll

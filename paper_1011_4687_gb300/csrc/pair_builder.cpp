@@ -303,36 +303,31 @@ const std::vector<float> &boys_table_dd()
 
 namespace {
 
-// dd records for the tiles that are evaluated in pairs of FP32 numbers, when
-// every number of theirs and every product of them stays well inside FP32's
-// range (else those tiles keep the FP64 code).
+// dd records for the tiles, when every number of theirs and every product of
+// them stays well inside FP32's range (else a tile keeps the FP64 code).
 void plan_dd(HostEnv &env)
 {
     const double big = 0x1p+60, small = 0x1p-60;
+    const bool ok_coord = env.coord_quantum < 0x1p+30; // coordinates below 2^52: squares in range
     for (TileMeta &m : env.tiles) {
         m.offdd = -1;
-        if (!(m.cls == kClassPoint || (m.vmax >= kNearVmax && (m.cls & kClassShortBit) == 0 &&
-                                       (m.cls & 7) <= kDdGeneralMaxL)))
-            continue;
         const bool pts = is_point_class(m.cls);
         const int st = pts ? kPointStride64 : rec64_stride(m.cls & 7);
-        const int nc = pts ? 0 : num_hermite(m.cls & 7);
-        bool ok = env.coord_quantum < 0x1p+30; // coordinates below 2^52: squares in range
-        double cmax = 0.0;
-        for (int j = 0; j < m.n && ok; ++j) {
+        const int nc = pts ? 1 : num_hermite(m.cls & 7);
+        double cmax = 0.0, smax = 0.0;
+        for (int j = 0; j < m.n; ++j) {
             const double *r = env.rec64.data() + m.off64 + size_t(j) * st;
-            if (pts) {
-                cmax = std::max(cmax, std::fabs(r[3]));
-            } else {
-                ok = r[3] > small && r[3] < big;
-                for (int k = 0; k < nc; ++k)
-                    cmax = std::max(cmax, std::fabs(r[4 + k]) * std::max(1.0, std::pow(r[3], -1.0 - (m.cls & 7))));
-            }
+            smax = std::max(smax, r[3]);
+            for (int k = 0; k < nc; ++k)
+                cmax = std::max(cmax, std::fabs(r[pts ? 3 : 4 + k]));
         }
-        if (!ok || !(cmax > small) || !(cmax < big))
+        if (!pts) // far-field moments: G sqrt(pi)/2 p^{-(N + 1)/2}
+            cmax *= std::max(1.0, std::pow(double(m.pmin), -0.5 * ((m.cls & 7) + 1)));
+        if (!ok_coord || !(cmax > small) || !(cmax < big) ||
+            (!pts && !(m.pmin > float(small * small) && smax < 0x1p+30)))
             continue;
         m.offdd = int32_t(env.dd_floats / 4);
-        env.dd_floats += int64_t(dd_words(m.cls)) * dd_pad(m.n);
+        env.dd_floats += int64_t(dd_words(m)) * dd_pad(m.n);
         if (env.dd_floats / 4 > INT32_MAX) {
             // beyond the offsets' range: no dd records at all
             for (TileMeta &t : env.tiles)

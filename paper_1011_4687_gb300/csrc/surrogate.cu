@@ -317,15 +317,19 @@ void split_tiles(esp_surrogate *s)
         (far ? s->far_tiles : s->near_tiles).push_back(m);
         (far ? s->n_far_entries : s->n_near_entries) += m.n;
     }
+    // the far tiles only make labels: FP64 code and a fixed grouping (TileView)
+    for (TileMeta &m : s->far_tiles)
+        m.offdd = -1;
     set_tile_groups(s->near_tiles, s->near_view);
     set_tile_groups(s->far_tiles, s->far_view);
+    s->far_view.labels = true;
 }
 
 esp_status upload_split(esp_surrogate *s)
 {
     cudaError_t e;
     const bool near = near_radius(s->ctx) > 0.0f;
-    const std::vector<int> nd = dd_tile_list(s->near_tiles, near), fd = dd_tile_list(s->far_tiles, near);
+    const std::vector<int> nd = dd_tile_list(s->near_tiles, near), fd = dd_tile_list(s->far_tiles, false);
     if ((e = upload_vec(s->d_near_tiles, s->near_tiles)) != cudaSuccess ||
         (e = upload_vec(s->d_far_tiles, s->far_tiles)) != cudaSuccess ||
         (e = upload_vec(s->d_near_dd, nd)) != cudaSuccess || (e = upload_vec(s->d_far_dd, fd)) != cudaSuccess)
