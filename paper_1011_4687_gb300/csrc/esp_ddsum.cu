@@ -79,7 +79,6 @@ __global__ void __launch_bounds__(kDdThreads, 4) dd_sum_kernel(EvalArgs a, const
 // small, by the FP64 pipe (near entries: some 40 operations of 64 cycles).
 // ---------------------------------------------------------------------------
 constexpr int kTdWordsMax = dd_far_words(kMaxL);
-constexpr float kTdNearT = 46.0f; // (T from the hi words: 1e-2 relative at most beyond kDdMinR2)
 
 // The far pairs of a chunk of at most 64 records; near: bits of the records to
 // leave out.  lo: the smallest |P - C|^2 met.

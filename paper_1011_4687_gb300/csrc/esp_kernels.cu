@@ -266,6 +266,8 @@ __global__ void __launch_bounds__(kSortThreads) batch_sort_kernel(const BatchHea
 // 18.4 / 39 / 78 us.
 // ---------------------------------------------------------------------------
 constexpr int kSmallWarps = kSmallThreads / 32;
+constexpr int kNearList = 64;  // near entries a warp keeps for the end
+constexpr int kNearDense = 24; // more of them in one item are evaluated at once
 
 // (s, c) += (s2, c2) with the rounding error of s + s2 kept in c (TwoSum)
 __device__ __forceinline__ void two_sum_pair(float &s, float &c, float s2, float c2)
@@ -325,6 +327,73 @@ __device__ __noinline__ double entry_f64(const SmallArgs &a, const TileMeta &m, 
     return tile_f64_one_any(m.cls, a.rec64 + m.off64 + (size_t)j * rec64_stride(m.cls & 7), 1, p[0], p[1], p[2],
                             a.boys64);
 }
+// entries j, j + 1 where they exist
+__device__ __forceinline__ double entries_f64(const SmallArgs &a, const TileMeta &m, int j, const double *p)
+{
+    double v = 0.0;
+    if (j < m.n)
+        v = entry_f64(a, m, j, p);
+    if (j + 1 < m.n)
+        v += entry_f64(a, m, j + 1, p);
+    return v;
+}
+
+// The same at FP64 accuracy with the far entries in FP32 words (as in
+// potential_td_kernel, but two entries per lane); j differs by lane, the tile
+// does not.
+template <int L>
+__device__ __noinline__ double far_pair(const DdTile t, int j, const DdPos &c, bool u0, bool u1, float *r2min)
+{
+    TdSum sum;
+    sum.clear();
+    f2 r2;
+    td_far<L>(t, j, c, u0, u1, sum, r2);
+    *r2min = fminf(r2.x, r2.y);
+    return sum.total();
+}
+__device__ __noinline__ double point_pair(const DdTile t, int j, const DdPos &c, float *r2min)
+{
+    TdSum sum;
+    sum.clear();
+    f2 r2;
+    td_point(t, j, c, sum, r2);
+    *r2min = fminf(r2.x, r2.y);
+    return sum.total();
+}
+// n0, n1: entries left to FP64.
+__device__ __forceinline__ double entries_words(const SmallArgs &a, const TileMeta &m, int j, const DdPos &c,
+                                                bool &n0, bool &n1)
+{
+    const int n4 = dd_pad(m.n);
+    const DdTile t = {a.recdd + (size_t)m.offdd * 4, n4};
+    const bool mine = j < m.n;
+    double v = 0.0;
+    float r2min = 1.0f;
+    n0 = n1 = false;
+    if (is_point_class(m.cls)) {
+        if (mine)
+            v = point_pair(t, j, c, &r2min);
+    } else if (mine) {
+        const f2 dx = t(0, j) - f2(c.h[0]), dy = t(1, j) - f2(c.h[1]), dz = t(2, j) - f2(c.h[2]);
+        const f2 T = t(10, j) * esp_fma(dx, dx, esp_fma(dy, dy, dz * dz));
+        n0 = !(T.x >= kTdNearT);
+        n1 = !(T.y >= kTdNearT);
+        switch (m.cls & 7) {
+        case 0: v = far_pair<0>(t, j, c, !n0, !n1, &r2min); break;
+        case 1: v = far_pair<1>(t, j, c, !n0, !n1, &r2min); break;
+        case 2: v = far_pair<2>(t, j, c, !n0, !n1, &r2min); break;
+        case 3: v = far_pair<3>(t, j, c, !n0, !n1, &r2min); break;
+        default: v = far_pair<4>(t, j, c, !n0, !n1, &r2min); break;
+        }
+    }
+    if (!(r2min >= kDdMinR2)) { // closer than the words resolve
+        v = 0.0;
+        n0 = n1 = true;
+    }
+    n0 &= mine;
+    n1 &= j + 1 < m.n;
+    return v;
+}
 
 // the words of two positions
 struct PairPos {
@@ -364,13 +433,17 @@ __global__ void __launch_bounds__(kSmallThreads, NQ <= 4 ? 2 : 1) small_n_kernel
     __shared__ __align__(16) float s_pair[NQ / 2 > 0 ? NQ / 2 : 1][12]; // lanes' hi x y z, lo x y z of position pairs
     __shared__ float2 s_red[kSmallWarps][NQ]; // sums in FP32 with compensation
     __shared__ double s_red64[kSmallWarps][NQ];
+    __shared__ int2 s_list[kSmallWarps][kNearList]; // tile, entry * kSmallChunk + position
+    __shared__ double s_val[kSmallWarps * kNearList];
+    __shared__ unsigned char s_own[kSmallWarps * kNearList];
+    __shared__ int s_listed[kSmallWarps];
     __shared__ int s_last;
     const int n = a.n_pos, t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int q0 = blockIdx.y * kSmallChunk;
     const int nq = min(NQ, n - q0);
     // does this CTA take any entry in FP64 (or as dd sums)?
-    const int units = a.n_other * a.tile_halves;
-    const bool has64 = int(blockIdx.x) < units * nq;
+    const int units = a.n_other * a.tile_parts;
+    const bool has64 = int(blockIdx.x) < units;
     if (t < 3 * NQ) {
         const int q = min(t / 3, nq - 1), d = t % 3; // (padding repeats the last position)
         const double x = a.pos_in[3 * (q0 + q) + d] - (d == 0 ? a.cx : d == 1 ? a.cy : a.cz);
@@ -431,26 +504,29 @@ __global__ void __launch_bounds__(kSmallThreads, NQ <= 4 ? 2 : 1) small_n_kernel
         s_red[warp][small_owner<NQ>(lane)] = make_float2(s[0], c[0]); // (lanes of one owner hold the same sum)
         __syncwarp();
     }
-    // the other tiles: warp w of CTA b takes (half tile, position) items b + grid w, ...
+    // the other tiles: CTA b takes the parts b, b + grid, ..., its warps one
+    // (part, position) item after the other, two entries per lane
     if (has64) {
-        for (int item = blockIdx.x + gridDim.x * warp; item < units * nq; item += gridDim.x * kSmallWarps) {
-            const int u = item % units, q = item / units;
-            const int o = u / a.tile_halves;
-            const TileMeta m = a.tiles[o < a.skip_begin ? o : o + a.n_skip];
-            const int j = (u % a.tile_halves) * 32 + lane;
+        int listed = 0; // entries in this warp's list
+        const int my_units = (units - int(blockIdx.x) + int(gridDim.x) - 1) / int(gridDim.x);
+        for (int item = warp; item < my_units * nq; item += kSmallWarps) {
+            const int u = blockIdx.x + gridDim.x * (item / nq), q = item % nq;
+            const int o = u / a.tile_parts;
+            const int tile = o < a.skip_begin ? o : o + a.n_skip;
+            const TileMeta m = a.tiles[tile];
+            const int j = (u % a.tile_parts) * 64 + 2 * lane;
+            const bool words = m.offdd >= 0 && dd_in_range(s_dd[q].h, a.dd_lim);
             if (m.cls == kClassPoint && a.points_dd) {
-                // beside FP32 sums: a dd sum, pairs of charges on the first lanes
-                const int n4 = dd_pad(m.n);
-                const float *rec = a.recdd + (size_t)m.offdd * 4;
+                // beside FP32 sums: dd sums
                 float s = 0.0f, c = 0.0f;
                 if (j < m.n) {
-                    const DdTile tile = {rec, n4};
+                    const DdTile tile = {a.recdd + (size_t)m.offdd * 4, dd_pad(m.n)};
                     f2 r2;
-                    const dd v = dd_point(tile, j & ~1, s_dd[q], r2);
-                    s = j & 1 ? v.h.y : v.h.x;
-                    c = j & 1 ? v.l.y : v.l.x;
-                    if (!((j & 1 ? r2.y : r2.x) >= kDdMinR2) || !dd_in_range(s_dd[q].h, a.dd_lim)) {
-                        const double x = entry_f64(a, m, j, s_pos[q]);
+                    const dd v = dd_point(tile, j, s_dd[q], r2);
+                    s = v.h.x, c = v.l.x;
+                    two_sum_pair(s, c, v.h.y, v.l.y); // (a padding charge is zero)
+                    if (!(fminf(r2.x, r2.y) >= kDdMinR2) || !words) {
+                        const double x = entries_f64(a, m, j, s_pos[q]);
                         s = float(x);
                         c = float(x - double(s));
                     }
@@ -464,7 +540,27 @@ __global__ void __launch_bounds__(kSmallThreads, NQ <= 4 ? 2 : 1) small_n_kernel
                     s_red[warp][q] = x;
                 }
             } else {
-                double v = j < m.n ? entry_f64(a, m, j, s_pos[q]) : 0.0;
+                double v = 0.0;
+                bool n0 = j < m.n, n1 = j + 1 < m.n;
+                if (words)
+                    v = entries_words(a, m, j, s_dd[q], n0, n1);
+                // near entries: an FP64 operation takes its 64 cycles whatever
+                // the number of lanes, so few of them wait in the warp's list
+                const unsigned b0 = __ballot_sync(0xffffffffu, n0), b1 = __ballot_sync(0xffffffffu, n1);
+                const int c0 = __popc(b0), cnt = c0 + __popc(b1);
+                if (cnt <= kNearDense && listed + cnt <= kNearList) {
+                    const unsigned below = (1u << lane) - 1u;
+                    if (n0)
+                        s_list[warp][listed + __popc(b0 & below)] = make_int2(tile, j * kSmallChunk + q);
+                    if (n1)
+                        s_list[warp][listed + c0 + __popc(b1 & below)] = make_int2(tile, (j + 1) * kSmallChunk + q);
+                    listed += cnt;
+                } else {
+                    if (n0)
+                        v += entry_f64(a, m, j, s_pos[q]);
+                    if (n1)
+                        v += entry_f64(a, m, j + 1, s_pos[q]);
+                }
 #pragma unroll
                 for (int w = 16; w > 0; w >>= 1)
                     v += __shfl_xor_sync(0xffffffffu, v, w);
@@ -472,6 +568,34 @@ __global__ void __launch_bounds__(kSmallThreads, NQ <= 4 ? 2 : 1) small_n_kernel
                     s_red64[warp][q] += v;
             }
             __syncwarp();
+        }
+        if (lane == 0)
+            s_listed[warp] = listed;
+        __syncthreads();
+        // the listed entries, one per thread, then each position's values by its warp
+        int total = 0;
+        for (int w = 0; w < kSmallWarps; ++w)
+            total += s_listed[w];
+        for (int k = t; k < total; k += kSmallThreads) {
+            int w = 0, i = k;
+            while (i >= s_listed[w])
+                i -= s_listed[w++];
+            const int2 x = s_list[w][i];
+            const TileMeta m = a.tiles[x.x];
+            s_val[k] = entry_f64(a, m, x.y / kSmallChunk, s_pos[x.y % kSmallChunk]);
+            s_own[k] = (unsigned char)(x.y % kSmallChunk);
+        }
+        __syncthreads();
+        if (warp < nq && total > 0) {
+            double v = 0.0;
+            for (int k = lane; k < total; k += 32)
+                if (s_own[k] == warp)
+                    v += s_val[k];
+#pragma unroll
+            for (int w = 16; w > 0; w >>= 1)
+                v += __shfl_xor_sync(0xffffffffu, v, w);
+            if (lane == 0)
+                s_red64[warp][warp] += v; // (row warp: only this thread adds to it now)
         }
     }
     __syncthreads();
@@ -499,7 +623,7 @@ __global__ void __launch_bounds__(kSmallThreads, NQ <= 4 ? 2 : 1) small_n_kernel
         return;
     // last CTA of the chunk: thread t takes position t % NQ of the slices t / NQ, ...
     __threadfence();
-    const int n64 = a.any64 ? min(units * nq, int(gridDim.x)) : 0;
+    const int n64 = a.any64 ? min(units, int(gridDim.x)) : 0;
     constexpr int rows = kSmallThreads / NQ;
     const int q = t % NQ;
     float s = 0.0f, c = 0.0f;
@@ -734,14 +858,20 @@ namespace {
 // positions a chunk holds: two (one pair) up to kSmallChunk
 int small_nq(int n) { return n <= 2 ? 2 : n <= 4 ? 4 : n <= 8 ? 8 : 16; }
 
-int small_grid(int g_threads) { return (g_threads + kSmallThreads - 1) / kSmallThreads; }
+// CTAs of a chunk: its FP32 threads; without FP32 entries one CTA per SM over
+// all chunks (5 positions x 889 tiles: 223 CTAs, a second wave of 71, took 50 us)
+int small_grid(int g_threads, int num_sms, int chunks, bool fp32)
+{
+    const int grid = (g_threads + kSmallThreads - 1) / kSmallThreads;
+    return fp32 ? grid : std::min(grid, std::max(1, num_sms / chunks));
+}
 
 } // namespace
 
 size_t small_n_bytes(int n_tiles, int num_sms, int n)
 {
     const int chunks = std::max(1, (n + kSmallChunk - 1) / kSmallChunk);
-    return (size_t)small_grid(small_n_threads(n_tiles, num_sms, n)) * chunks * small_nq(n) * (sizeof(float2) + sizeof(double));
+    return (size_t)small_grid(small_n_threads(n_tiles, num_sms, n), num_sms, chunks, true) * chunks * small_nq(n) * (sizeof(float2) + sizeof(double));
 }
 
 cudaError_t launch_small_n(SmallArgs a, void *scratch, int num_sms, double *V, cudaStream_t s)
@@ -750,7 +880,8 @@ cudaError_t launch_small_n(SmallArgs a, void *scratch, int num_sms, double *V, c
         return cudaErrorInvalidValue;
     a.g_threads = small_n_threads(a.n_tiles, num_sms, a.n_pos);
     const int nq = small_nq(a.n_pos);
-    const dim3 grid(small_grid(a.g_threads), (a.n_pos + kSmallChunk - 1) / kSmallChunk);
+    const int chunks = (a.n_pos + kSmallChunk - 1) / kSmallChunk;
+    const dim3 grid(small_grid(a.g_threads, num_sms, chunks, a.n_p32 > 0), chunks);
     a.part64 = static_cast<double *>(scratch);
     a.part32 = reinterpret_cast<float2 *>(a.part64 + (size_t)grid.x * grid.y * nq);
     switch (nq) {

@@ -144,7 +144,7 @@ size_t potential_smem_bytes(int precision, int tile_size);
 bool potential_shape_supported(int precision, int threads, int ppt);
 // Few positions per call (n <= kSmallN): environment entries spread over the
 // threads of one launch, a chunk of up to kSmallChunk positions per CTA row.
-// Entries are evaluated in FP64, except the FP32 point charges (class
+// Entries are evaluated at FP64 accuracy (far ones in FP32 words), except the FP32 point charges (class
 // kClassPoint32) when n_p32 is set: those take the compensated FP32 form of
 // the main kernel (hi/lo offsets, symmetric rsqrt, low word of the charge),
 // sum per thread in FP32 and across threads as (sum, compensation) pairs; the
@@ -172,8 +172,8 @@ struct SmallArgs {
     int64_t p32_off;       // float offset of the FP32 point records (contiguous, n_p32 of them)
     int n_p32;             // 0: every entry in FP64
     // the tiles outside the flat FP32 pass: n_other of them, tile o or, from
-    // skip_begin on, o + n_skip, in tile_halves parts of 32 entries each
-    int n_other, skip_begin, n_skip, tile_halves;
+    // skip_begin on, o + n_skip, in tile_parts parts of 64 entries each
+    int n_other, skip_begin, n_skip, tile_parts;
     int *counters;         // [kSmallMaxChunks], zero before and after every launch
     // set by launch_small_n
     int g_threads;
