@@ -69,6 +69,7 @@ int esp::plan_splits(const esp_ctx *c, const TileView &v, int n, int prec, int m
     a.n_tiles = v.n_tiles;
     a.tiles = v.tiles;
     dd_splits = 0;
+    a.pairs = prec == 1 && !v.labels && v.n_tiles > 0;
     if (use_td(c, v, prec)) {
         a.n_splits = std::min(td_splits(n, v.n_tiles, c->num_sms), max_splits);
         single_group(a);
@@ -314,7 +315,7 @@ esp_status pipeline(esp_ctx *c, const TileView &v, int prec, const double *d_pos
     }
     if (timing && (e = cudaEventRecord(c->ev[2], s)) != cudaSuccess)
         return cuda_fail(e, "recording a timing event");
-    if ((!small_n || v.n_tiles == 0) && (e = launch_reduce(a.partial, splits, int(n), dV, s, perm, v.labels)) != cudaSuccess)
+    if ((!small_n || v.n_tiles == 0) && (e = launch_reduce(a.partial, splits, int(n), dV, s, perm, v.labels, a.pairs ? dd_splits : -1)) != cudaSuccess)
         return cuda_fail(e, "launching the partial-sum reduction");
     if (dE && (e = launch_walkers(dV, int(n_walkers), int(n_elec), dE, s)) != cudaSuccess)
         return cuda_fail(e, "launching the walker-energy reduction");
@@ -987,7 +988,7 @@ extern "C" esp_status esp_eval_noalloc(esp_ctx *ctx, const double *positions, in
         if ((e = launch_planned(ctx, ctx->full, prec, a, dd_splits, s)) != cudaSuccess)
             return cuda_fail(e, "launching the potential kernel");
     }
-    if ((e = launch_reduce(partial, splits, int(n), V_out, s)) != cudaSuccess)
+    if ((e = launch_reduce(partial, splits, int(n), V_out, s, nullptr, false, a.pairs ? dd_splits : -1)) != cudaSuccess)
         return cuda_fail(e, "launching the partial-sum reduction");
     return ESP_OK;
 }

@@ -720,6 +720,51 @@ __global__ void __launch_bounds__(32 * SLICES) reduce_kernel(const double *__res
         V[perm ? perm[i] : i] = s + c;
 }
 
+// The same where the partials after the first n64 (the dd kernel's, FP64) are
+// FP32 (sum, compensation) pairs, as an FP32C kernel holds them: few FP64
+// operations (FP64 partials of 1,001 positions in 512 splits took 38 us, of
+// 65,536 in 60 splits 65 us).
+template <int SLICES>
+__global__ void __launch_bounds__(32 * SLICES) reduce_pairs_kernel(const double *__restrict__ partial, int n64,
+                                                                    int n_splits, int n, double *__restrict__ V,
+                                                                    const int *__restrict__ perm)
+{
+    __shared__ float2 s_p[SLICES][32];
+    __shared__ double s_s[SLICES][32], s_c[SLICES][32];
+    const float2 *pairs = reinterpret_cast<const float2 *>(partial);
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + x;
+    float s = 0.0f, c = 0.0f;
+    double s64 = 0.0, c64 = 0.0;
+    if (i < n) {
+        for (int k = y; k < n64; k += SLICES)
+            two_sum_acc(s64, c64, partial[(size_t)k * n + i]);
+#pragma unroll 4
+        for (int k = n64 + y; k < n_splits; k += SLICES) {
+            const float2 p = pairs[(size_t)k * n + i];
+            two_sum_pair(s, c, p.x, p.y);
+        }
+    }
+    s_p[y][x] = make_float2(s, c);
+    s_s[y][x] = s64;
+    s_c[y][x] = c64;
+#pragma unroll
+    for (int o = SLICES / 2; o > 0; o >>= 1) {
+        __syncthreads();
+        if (y < o) {
+            two_sum_pair(s, c, s_p[y + o][x].x, s_p[y + o][x].y);
+            s_p[y][x] = make_float2(s, c);
+            if (y + o < n64) { // (slices from n64 on hold no FP64 partial)
+                two_sum_join(s64, c64, s_s[y + o][x], s_c[y + o][x]);
+                s_s[y][x] = s64;
+                s_c[y][x] = c64;
+            }
+        }
+    }
+    if (y == 0 && i < n)
+        V[perm ? perm[i] : i] = (s64 + c64) + (double(s) + double(c));
+}
+
 // one warp per walker: its lanes' electrons by TwoSum, then the lanes in a fixed order
 __global__ void walker_kernel(const double *__restrict__ V, int n_walkers, int n_elec, double *__restrict__ E)
 {
@@ -894,13 +939,17 @@ cudaError_t launch_small_n(SmallArgs a, void *scratch, int num_sms, double *V, c
 }
 
 cudaError_t launch_reduce(const double *partial, int n_splits, int n, double *V, cudaStream_t s, const int *perm,
-                          bool in_order)
+                          bool in_order, int n64)
 {
     if (n <= 0)
         return cudaSuccess;
     const int grid = (n + 31) / 32;
     // more slices where the partials are many and the positions few
-    if (in_order)
+    if (n64 >= 0 && n_splits > 64)
+        reduce_pairs_kernel<32><<<grid, 32 * 32, 0, s>>>(partial, n64, n_splits, n, V, perm);
+    else if (n64 >= 0)
+        reduce_pairs_kernel<8><<<grid, 32 * 8, 0, s>>>(partial, n64, n_splits, n, V, perm);
+    else if (in_order)
         reduce_kernel<1><<<grid, 32, 0, s>>>(partial, n_splits, n, V, perm);
     else if (n_splits > 64)
         reduce_kernel<32><<<grid, 32 * 32, 0, s>>>(partial, n_splits, n, V, perm);

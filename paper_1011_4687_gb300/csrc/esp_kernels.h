@@ -52,6 +52,7 @@ struct EvalArgs {
     const float *boysdd;  // Boys table of the dd general form
     float dd_lim;         // |coordinate| up to which the dd words of a position are exact
     double *partial;  // [n_splits][n_pos], FP64
+    int pairs;        // FP32C kernel: its partials as float2 (sum, compensation), in the same places
     float near_r;     // FP32C: FP64 re-evaluation radius around a tile's bounding sphere
     // FP32C deal by tile group: group g holds tiles [grp_tile[g], grp_tile[g+1])
     // and takes the splits [grp_split[g], grp_split[g+1]) (grp_split[n_groups] =
@@ -184,9 +185,10 @@ struct SmallArgs {
 size_t small_n_bytes(int n_tiles, int num_sms, int n);
 cudaError_t launch_small_n(SmallArgs a, void *scratch, int num_sms, double *V, cudaStream_t s);
 // perm (optional, from launch_sort): V[perm[slot]] receives the sum of slot
-// in_order: the partials one after the other (else several chains, joined)
+// in_order: the partials one after the other (else several chains, joined);
+// n64 >= 0: the partials after the first n64 as float2 (sum, compensation)
 cudaError_t launch_reduce(const double *partial, int n_splits, int n, double *V, cudaStream_t s,
-                          const int *perm = nullptr, bool in_order = false);
+                          const int *perm = nullptr, bool in_order = false, int n64 = -1);
 cudaError_t launch_walkers(const double *V, int n_walkers, int n_elec, double *E, cudaStream_t s);
 
 } // namespace esp

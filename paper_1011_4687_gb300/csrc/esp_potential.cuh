@@ -95,6 +95,8 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
         const int nvec = pts ? (ddt ? kDdPointWords * n4 / 4 : m.n * 2)
                              : (m.n * rec32_stride_cls(m.cls)) / 4;
         copy_tile(s_tile4, src, nvec);
+        if (!ALL)
+            asm volatile("cp.async.wait_all;" ::: "memory"); // the Boys table, once
         __syncthreads();
         float ch[PPT][3], cl[PPT][3];
 #pragma unroll
@@ -307,7 +309,10 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
 #pragma unroll
     for (int q = 0; q < PPT; ++q) {
         const int i = base + q * NT;
-        if (i < a.n_pos)
+        if (!ALL && a.pairs) {
+            if (i < a.n_pos)
+                reinterpret_cast<float2 *>(a.partial)[(size_t)split * a.n_pos + i] = make_float2(S[q], Cc[q]);
+        } else if (i < a.n_pos)
             a.partial[(size_t)split * a.n_pos + i] = ((double)S[q] + (double)Cc[q]) + (ALL ? acc64[q * NT] : 0.0);
     }
 }
@@ -318,9 +323,17 @@ __global__ void __launch_bounds__(NT, 512 / NT) potential_f32c_kernel(EvalArgs a
     extern __shared__ float4 smem4[];
     float4 *s_tile4 = smem4;
     float *s_boys = reinterpret_cast<float *>(smem4 + (a.tile_size * kRec32MaxStride) / 4);
-    for (int i = threadIdx.x; i < kBoys32Rows * kBoys32Row; i += NT)
-        s_boys[i] = a.boys32[i];
+    // The Boys table comes in asynchronously beside the first tile (a CTA of a
+    // short call has one or two tiles; the copy through registers took a fifth
+    // of its time); the loop's first barrier follows the wait.
+    constexpr int nb = kBoys32Rows * kBoys32Row;
+    const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(s_boys));
+    for (int i = threadIdx.x; i < nb / 4; i += NT)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * i), "l"(a.boys32 + 4 * i) : "memory");
+    if (threadIdx.x < nb % 4)
+        s_boys[nb - 1 - threadIdx.x] = a.boys32[nb - 1 - threadIdx.x];
     cta_f32c<NT, PPT, false>(a, blockIdx.x, blockIdx.y, s_tile4, s_boys, nullptr);
+    asm volatile("cp.async.wait_all;" ::: "memory"); // (a CTA without tiles)
 }
 
 // ---------------------------------------------------------------------------
@@ -439,6 +452,7 @@ __device__ __forceinline__ EvalArgs args_of(const SysDesc &d, const float *boys3
     a.recdd = d.recdd;
     a.boysdd = boysdd;
     a.dd_lim = d.dd_lim;
+    a.pairs = 0;
     a.partial = d.partial;
     a.near_r = d.near_r;
     single_group(a);
