@@ -13,7 +13,7 @@
 // issues the four K = 16 MMAs of a chunk and commits them to the stage's
 // mbarrier; the stage is refilled once that commit has completed, so the
 // loads of chunk c + 1 overlap the MMAs of chunk c.  The epilogue reads the
-// accumulator back with tcgen05.ld (thread t: row t, 32 columns at a time).
+// accumulator back with tcgen05.ld (thread t: row t) through shared memory.
 // grid.z splits K into slices of kchunk (partials to C + z M ldc).
 //
 // Every mbarrier wait is bounded; a CTA whose wait gives up sets *err, waits
@@ -41,6 +41,13 @@ __device__ __forceinline__ float silu_grad_f(float z)
 {
     float s = 1.0f / (1.0f + __expf(-z));
     return s * (1.0f + z * (1.0f - s));
+}
+
+constexpr int kEpiStride = 68; // floats of a staged row: 16-byte aligned, conflict-free float4 columns
+
+__device__ __forceinline__ void store_bf16x4(__nv_bfloat16 *p, float a, float b, float c, float d)
+{
+    *reinterpret_cast<uint2 *>(p) = make_uint2(tc::pack_bf16x2(a, b), tc::pack_bf16x2(c, d));
 }
 
 // op(X)[r][k] for operand row r (M for A, N for B) and K index k:
@@ -171,42 +178,63 @@ __global__ void __launch_bounds__(kGemmThreads)
     }
     tc::fence_after();
     if (ok) {
-        const int row = tid; // TMEM lane = row of the tile
-        const int m = m0 + row;
+        // 64 columns at a time: each thread's row of the accumulator goes to
+        // shared memory (the stages are free now), then half a warp takes a row,
+        // four columns per lane, and every global access is a whole 128-byte
+        // line.  (One thread per row with a store per element took 62 us for
+        // 8,192 x 256 x 256, most of it in partial sectors.)
+        float *s_c = reinterpret_cast<float *>(smem);
         const uint32_t lane_addr = tmem + (uint32_t(warp * 32) << 16);
 #pragma unroll 1
-        for (int c0 = 0; c0 < BN; c0 += 32) {
-            float v[32];
-            if (nc > 0) {
-                tc::tmem_ld32(lane_addr + uint32_t(c0), v);
-            } else {
+        for (int c0 = 0; c0 < BN; c0 += 64) {
 #pragma unroll
-                for (int e = 0; e < 32; ++e)
-                    v[e] = 0.0f;
-            }
-            if (m >= g.M)
-                continue;
+            for (int h = 0; h < 64; h += 32) {
+                float v[32];
+                if (nc > 0) {
+                    tc::tmem_ld32(lane_addr + uint32_t(c0 + h), v);
+                } else {
 #pragma unroll
-            for (int e = 0; e < 32; ++e) {
-                const int n = n0 + c0 + e;
-                if (n >= g.N)
-                    continue;
-                const size_t o = (size_t)m * g.ldc + n;
-                switch (g.epi) {
-                case kEpiSiluFwd: {
-                    const float z = v[e] + g.bias[n];
-                    if (g.Cf)
-                        g.Cf[o] = z;
-                    g.Cb[o] = __float2bfloat16(silu_f(z));
-                    break;
+                    for (int e = 0; e < 32; ++e)
+                        v[e] = 0.0f;
                 }
-                case kEpiGradSilu:
-                    g.Cb[o] = __float2bfloat16(v[e] * silu_grad_f(g.aux[o]));
-                    break;
-                default:
-                    g.Cf[(size_t)blockIdx.z * g.M * g.ldc + o] = v[e];
+#pragma unroll
+                for (int e = 0; e < 32; e += 4)
+                    *reinterpret_cast<float4 *>(s_c + tid * kEpiStride + h + e) =
+                        make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+            }
+            __syncthreads();
+            const int col = (tid & 15) * 4, n = n0 + c0 + col;
+            if (n < g.N) {
+                float4 bias = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (g.epi == kEpiSiluFwd)
+                    bias = *reinterpret_cast<const float4 *>(g.bias + n);
+#pragma unroll 4
+                for (int r = tid >> 4; r < kTileM; r += kGemmThreads / 16) {
+                    const int m = m0 + r;
+                    if (m >= g.M)
+                        break;
+                    const float4 v = *reinterpret_cast<const float4 *>(s_c + r * kEpiStride + col);
+                    const size_t o = (size_t)m * g.ldc + n;
+                    switch (g.epi) {
+                    case kEpiSiluFwd: {
+                        const float4 z = make_float4(v.x + bias.x, v.y + bias.y, v.z + bias.z, v.w + bias.w);
+                        if (g.Cf)
+                            *reinterpret_cast<float4 *>(g.Cf + o) = z;
+                        store_bf16x4(g.Cb + o, silu_f(z.x), silu_f(z.y), silu_f(z.z), silu_f(z.w));
+                        break;
+                    }
+                    case kEpiGradSilu: {
+                        const float4 z = __ldg(reinterpret_cast<const float4 *>(g.aux + o));
+                        store_bf16x4(g.Cb + o, v.x * silu_grad_f(z.x), v.y * silu_grad_f(z.y),
+                                     v.z * silu_grad_f(z.z), v.w * silu_grad_f(z.w));
+                        break;
+                    }
+                    default:
+                        *reinterpret_cast<float4 *>(g.Cf + (size_t)blockIdx.z * g.M * g.ldc + o) = v;
+                    }
                 }
             }
+            __syncthreads();
         }
     }
     if (tid == 0) {
@@ -249,6 +277,10 @@ cudaError_t gemm_tc(bool a_t, bool b_t, const GemmArgs &g, int ksplit, int *err,
 {
     if (g.M <= 0 || g.N <= 0)
         return cudaSuccess;
+    // (the epilogue's 16-byte accesses)
+    if (g.N % 64 || g.ldc % 4 || ((reinterpret_cast<uintptr_t>(g.Cf) | reinterpret_cast<uintptr_t>(g.Cb) |
+                                   reinterpret_cast<uintptr_t>(g.bias) | reinterpret_cast<uintptr_t>(g.aux)) & 15))
+        return cudaErrorInvalidValue;
     if (g.N > 256 || ksplit < 1 || g.kchunk < 1 || !err || wait_limit < 0)
         return cudaErrorInvalidValue;
     // 256-column tiles only when they alone give every SM two CTAs; the

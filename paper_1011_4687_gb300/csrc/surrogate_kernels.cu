@@ -35,13 +35,23 @@ __global__ void features_kernel(const double *__restrict__ pos, int n, const flo
         return;
     const float ux = float((pos[3 * i] - cx) * inv_r), uy = float((pos[3 * i + 1] - cy) * inv_r),
                 uz = float((pos[3 * i + 2] - cz) * inv_r);
-#pragma unroll 4
-    for (int f = 0; f < kFreq; ++f) {
-        float ph = 6.283185307179586f * (freq[3 * f] * ux + freq[3 * f + 1] * uy + freq[3 * f + 2] * uz);
-        float s, c;
-        __sincosf(ph, &s, &c);
-        X[(size_t)i * kFeat + f] = __float2bfloat16(s);
-        X[(size_t)i * kFeat + kFreq + f] = __float2bfloat16(c);
+    // eight features per 16-byte store (a store per feature, 128 bytes apart
+    // across the warp, took 21 us for 8,192 positions)
+    uint4 *row = reinterpret_cast<uint4 *>(X + (size_t)i * kFeat);
+#pragma unroll 1
+    for (int f0 = 0; f0 < kFreq; f0 += 8) {
+        __align__(16) __nv_bfloat16 vs[8], vc[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int f = f0 + e;
+            float ph = 6.283185307179586f * (freq[3 * f] * ux + freq[3 * f + 1] * uy + freq[3 * f + 2] * uz);
+            float s, c;
+            __sincosf(ph, &s, &c);
+            vs[e] = __float2bfloat16(s);
+            vc[e] = __float2bfloat16(c);
+        }
+        row[f0 / 8] = *reinterpret_cast<const uint4 *>(vs);
+        row[(kFreq + f0) / 8] = *reinterpret_cast<const uint4 *>(vc);
     }
 }
 
@@ -92,6 +102,7 @@ __global__ void out_grad_kernel(const float *__restrict__ dy, const __nv_bfloat1
     const int k = threadIdx.x; // blockDim = 256 = kHidden
     const int r0 = blockIdx.x * rows, r1 = min(n, r0 + rows);
     float s = 0.0f, sb = 0.0f;
+#pragma unroll 8
     for (int i = r0; i < r1; ++i) {
         s += dy[i] * __bfloat162float(H[(size_t)i * kHidden + k]);
         sb += dy[i];
@@ -107,6 +118,7 @@ __global__ void colsum_kernel(const __nv_bfloat16 *__restrict__ M, int n, int ro
     const int k = threadIdx.x;
     const int r0 = blockIdx.x * rows, r1 = min(n, r0 + rows);
     float s = 0.0f;
+#pragma unroll 8
     for (int i = r0; i < r1; ++i)
         s += __bfloat162float(M[(size_t)i * kHidden + k]);
     part[(size_t)blockIdx.x * kHidden + k] = s;
@@ -119,7 +131,8 @@ __global__ void sum_parts_kernel(const float *__restrict__ part, int nparts, int
     if (j >= len)
         return;
     float s = 0.0f;
-    for (int z = 0; z < nparts; ++z)
+#pragma unroll 16
+    for (int z = 0; z < nparts; ++z) // (loads of 16 partials in flight)
         s += part[(size_t)z * len + j];
     out[j] = s;
 }
@@ -260,7 +273,7 @@ cudaError_t features(const double *pos, int n, const float *freq, const double c
 {
     if (n <= 0)
         return cudaSuccess;
-    features_kernel<<<(n + 255) / 256, 256, 0, s>>>(pos, n, freq, c[0], c[1], c[2], inv_r, X);
+    features_kernel<<<(n + 63) / 64, 64, 0, s>>>(pos, n, freq, c[0], c[1], c[2], inv_r, X);
     return cudaGetLastError();
 }
 
