@@ -5,7 +5,7 @@
 // (Eq. FMO), and QMC runs many walkers, so the batch driver evaluates many
 // (environment, positions) systems of uneven size together: one staging
 // kernel, one persistent potential kernel that takes (system, position block,
-// pair split) work items from an atomic counter, largest systems first, and
+// range of tiles) work items from an atomic counter, costly classes first, and
 // one reduction kernel.  The three launches and the upload of the per-call
 // table are captured once into a CUDA graph and replayed; sizes and pointers
 // travel in the table, so a replay serves any call that fits the capacity.
@@ -33,8 +33,7 @@ struct esp_batch {
     DevBuf table, counter;
     void *host_table = nullptr;
     size_t table_bytes = 0;
-    std::vector<DevBuf> scratch;      // per system: staged positions, then partial sums
-    std::vector<size_t> scratch_cap;
+    DevBuf scratch;                   // per system: staged positions, partial sums, spatial order
     cudaGraphExec_t exec = nullptr;
     bool graph_valid = false;
     cudaEvent_t ev_copied = nullptr, ev_start = nullptr, ev_end = nullptr;
@@ -46,10 +45,30 @@ namespace {
 
 bool valid_batch(const esp_batch *b) { return b && b->magic == 0x45535042u; }
 
-int base_splits(const esp_ctx *c)
+// Estimated cost of a tile group's entry.  Low classes count for more than their
+// far form's operations: their diffuse tiles take the general form (Boys values
+// per position) and come last, where long items would leave SMs idle.
+double group_cost(int cls)
 {
-    // work items of about 24 tiles each for every position block
-    return std::max(1, (c->n_tiles + 23) / 24);
+    static const double kCost[kMaxL + 1] = {30.0, 60.0, 90.0, 120.0, 180.0};
+    return cls == kClassPoint ? 54.0 : cls == kClassPoint32 ? 10.0 : kCost[cls & 7];
+}
+
+constexpr int kMaxBatchSplits = 96;
+
+// Ranges of a system's tile groups for items of about `target` cost; returns
+// their number (partial sums).
+int plan_ranges(const esp_ctx *c, double target, int *ranges)
+{
+    const TileView &v = c->full;
+    int sum = 0;
+    for (int g = 0; g < v.n_groups; ++g) {
+        const int tiles = v.grp_tile[g + 1] - v.grp_tile[g];
+        const double cost = tiles > 0 ? tiles * c->env.tile_size * group_cost(c->env.tiles[size_t(v.grp_tile[g])].cls) : 0.0;
+        ranges[g] = std::max(1, std::min(tiles, int(std::ceil(cost / target))));
+        sum += ranges[g];
+    }
+    return sum;
 }
 
 void release_batch(esp_batch *b)
@@ -60,8 +79,7 @@ void release_batch(esp_batch *b)
     b->graph_valid = false;
     b->table.release();
     b->counter.release();
-    for (DevBuf &d : b->scratch)
-        d.release();
+    b->scratch.release();
     if (b->host_table)
         cudaFreeHost(b->host_table);
     b->host_table = nullptr;
@@ -73,6 +91,13 @@ void release_batch(esp_batch *b)
     if (b->gstream)
         cudaStreamDestroy(b->gstream);
     b->gstream = nullptr;
+}
+
+// the groups' place in the table (device or host)
+BatchGroup *groups_of(const esp_batch *b, void *table)
+{
+    return reinterpret_cast<BatchGroup *>(static_cast<char *>(table) + sizeof(BatchHeader) +
+                                          b->ctxs.size() * sizeof(SysDesc));
 }
 
 esp_status capture_graph(esp_batch *b)
@@ -98,7 +123,7 @@ esp_status capture_graph(esp_batch *b)
         if (!boysdd)
             boysdd = static_cast<const float *>(c->boysdd.p);
     cudaError_t e4 = e3 == cudaSuccess
-                         ? launch_batch(b->precision, hdr, sys, int(b->ctxs.size()), static_cast<int *>(b->counter.p),
+                         ? launch_batch(b->precision, hdr, sys, groups_of(b, b->table.p), int(b->ctxs.size()), static_cast<int *>(b->counter.p),
                                         1 << 30,
                                         static_cast<const float *>(c0->boys32.p),
                                         static_cast<const double *>(c0->boys64.p),
@@ -141,27 +166,40 @@ esp_status batch_eval(esp_batch *b, const double *const *positions, const int64_
     }
     if (total > (int64_t(1) << 30))
         return fail(ESP_ERR_INVALID, "too many positions in one batch");
-    // per-system split counts and work items; largest item cost first
-    std::vector<int> order(ns), splits(ns), blocks(ns);
-    std::vector<double> item_cost(ns);
+    // Items of about equal cost, eight for each resident CTA (four per SM): a
+    // range of tiles of one class against one block of positions.  (Items of 24
+    // tiles strided over the classes: 900 for 608 CTAs in a batch of 12 systems
+    // of 4,096 positions x 12,000 distributions, and a third of the issue slots
+    // waiting for instructions.)
+    std::vector<int> splits(ns), blocks(ns), ranges(size_t(ns) * kMaxTileGroups);
     const int per_cta = b->threads * b->ppt;
+    double work = 0.0;
     for (int k = 0; k < ns; ++k) {
-        order[size_t(k)] = k;
         const esp_ctx *c = b->ctxs[size_t(k)];
-        int sp = int(std::lround(base_splits(c) * b->split_scale));
-        splits[size_t(k)] = std::max(1, std::min({sp, 64, std::max(c->n_tiles, 1)}));
         blocks[size_t(k)] = int((n[k] + per_cta - 1) / per_cta);
-        item_cost[size_t(k)] = double(c->n_tiles) / splits[size_t(k)];
+        for (int g = 0; g < c->full.n_groups; ++g) {
+            const int t0 = c->full.grp_tile[g], t1 = c->full.grp_tile[g + 1];
+            if (t1 > t0)
+                work += double(blocks[size_t(k)]) * (t1 - t0) * c->env.tile_size * group_cost(c->env.tiles[size_t(t0)].cls);
+        }
     }
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return item_cost[size_t(x)] > item_cost[size_t(y)]; });
-    // scratch capacity (staged positions + partial sums) per system
-    cudaError_t e;
+    const double target = std::max(1.0, work / (8.0 * 4.0 * b->num_sms * b->split_scale));
     for (int k = 0; k < ns; ++k) {
-        size_t need = size_t(n[k]) * kStagedBytes + 256 +
-                      size_t(n[k]) * size_t(splits[size_t(k)]) * sizeof(double) + 2 * size_t(n[k]) * sizeof(int);
-        if ((e = b->scratch[size_t(k)].ensure(std::max<size_t>(need, 256))) != cudaSuccess)
-            return cuda_fail(e, "allocating batched scratch");
+        double t = target;
+        int *r = ranges.data() + size_t(k) * kMaxTileGroups;
+        while ((splits[size_t(k)] = plan_ranges(b->ctxs[size_t(k)], t, r)) > kMaxBatchSplits)
+            t *= 1.5;
     }
+    // scratch of all systems in one allocation
+    cudaError_t e;
+    std::vector<size_t> place(size_t(ns) + 1, 0);
+    for (int k = 0; k < ns; ++k) {
+        const size_t need = size_t(n[k]) * kStagedBytes + 256 + size_t(n[k]) * size_t(splits[size_t(k)]) * sizeof(double) +
+                            2 * size_t(n[k]) * sizeof(int);
+        place[size_t(k) + 1] = place[size_t(k)] + (need + 255) / 256 * 256;
+    }
+    if ((e = b->scratch.ensure(place[size_t(ns)])) != cudaSuccess)
+        return cuda_fail(e, "allocating batched scratch");
     // wait until the previous replay has read the pinned table
     if (b->copied_pending) {
         if ((e = cudaEventSynchronize(b->ev_copied)) != cudaSuccess)
@@ -170,11 +208,10 @@ esp_status batch_eval(esp_batch *b, const double *const *positions, const int64_
     }
     BatchHeader *hdr = static_cast<BatchHeader *>(b->host_table);
     SysDesc *sys = reinterpret_cast<SysDesc *>(static_cast<char *>(b->host_table) + sizeof(BatchHeader));
-    int item = 0, pos = 0;
-    for (int r = 0; r < ns; ++r) {
-        const int k = order[size_t(r)];
+    int pos = 0;
+    for (int k = 0; k < ns; ++k) {
         const esp_ctx *c = b->ctxs[size_t(k)];
-        SysDesc &d = sys[r];
+        SysDesc &d = sys[k];
         std::memset(&d, 0, sizeof(d));
         d.tiles = static_cast<const TileMeta *>(c->tiles.p);
         d.rec32 = static_cast<const float *>(c->rec32.p);
@@ -184,7 +221,7 @@ esp_status batch_eval(esp_batch *b, const double *const *positions, const int64_
         d.pos_in = positions[k];
         d.V_out = V_out[k];
         const int nk = int(n[k]);
-        char *base = static_cast<char *>(b->scratch[size_t(k)].p);
+        char *base = static_cast<char *>(b->scratch.p) + place[size_t(k)];
         d.st = staged_at(base, size_t(nk));
         size_t off = (size_t(nk) * kStagedBytes + 255) / 256 * 256;
         d.partial = reinterpret_cast<double *>(base + off);
@@ -200,16 +237,33 @@ esp_status batch_eval(esp_batch *b, const double *const *positions, const int64_
         d.n_pos = nk;
         d.splits = splits[size_t(k)];
         d.blocks = blocks[size_t(k)];
-        d.item_begin = item;
         d.pos_begin = pos;
         d.near_r = near_radius(c);
-        item += d.blocks * d.splits;
         pos += nk;
     }
+    // the items, costly classes first
+    int item = 0, n_groups = 0;
+    BatchGroup *groups = groups_of(b, b->host_table);
+    static const int order[] = {kClassPoint, 4, 3, 2, 1, 0, kClassPoint32};
+    for (int cls : order)
+        for (int k = 0; k < ns; ++k) {
+            const TileView &v = b->ctxs[size_t(k)]->full;
+            const int *r = ranges.data() + size_t(k) * kMaxTileGroups;
+            for (int g = 0, split = 0; g < v.n_groups; split += r[g++]) {
+                const int tiles = v.grp_tile[g + 1] - v.grp_tile[g];
+                if (tiles <= 0)
+                    continue;
+                const int tc = b->ctxs[size_t(k)]->env.tiles[size_t(v.grp_tile[g])].cls;
+                if (blocks[size_t(k)] == 0 || (is_point_class(tc) ? tc : tc & 7) != cls)
+                    continue;
+                groups[n_groups++] = {item, k, v.grp_tile[g], tiles, r[g], split};
+                item += blocks[size_t(k)] * r[g];
+            }
+        }
     hdr->n_sys = ns;
     hdr->n_items = item;
     hdr->n_pos_total = pos;
-    hdr->pad = 0;
+    hdr->n_groups = n_groups;
     if (!b->graph_valid) {
         esp_status st = capture_graph(b);
         if (st != ESP_OK)
@@ -272,10 +326,8 @@ esp_status esp_batch_create(esp_ctx *const *ctxs, int32_t n_sys, void *cuda_stre
         b->tile_cap = std::max(b->tile_cap, c->env.tile_size);
     b->threads = b->precision == 1 ? 128 : 128;
     b->ppt = b->precision == 1 ? 4 : 2;
-    b->scratch.resize(size_t(n_sys));
-    b->scratch_cap.assign(size_t(n_sys), 0);
     DeviceGuard dg(b->device);
-    b->table_bytes = sizeof(BatchHeader) + size_t(n_sys) * sizeof(SysDesc);
+    b->table_bytes = sizeof(BatchHeader) + size_t(n_sys) * (sizeof(SysDesc) + kMaxTileGroups * sizeof(BatchGroup));
     cudaError_t e;
     if ((e = b->table.ensure(b->table_bytes)) != cudaSuccess || (e = b->counter.ensure(sizeof(int))) != cudaSuccess ||
         (e = cudaMallocHost(&b->host_table, b->table_bytes)) != cudaSuccess ||

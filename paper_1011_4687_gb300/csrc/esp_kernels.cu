@@ -189,7 +189,7 @@ __global__ void batch_key_kernel(const BatchHeader *__restrict__ hdr, const SysD
 {
     const int total = hdr->n_pos_total, n_sys = hdr->n_sys;
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < total; g += gridDim.x * blockDim.x) {
-        const SysDesc &d = sys[find_sys(sys, n_sys, g, false)];
+        const SysDesc &d = sys[find_sys(sys, n_sys, g)];
         const int i = g - d.pos_begin;
         if (d.sorted)
             d.slot_of[i] = sort_cell(d.pos_in, i, d.qm[0], d.qm[1], d.qm[2]);
@@ -200,7 +200,7 @@ __global__ void batch_stage_kernel(const BatchHeader *__restrict__ hdr, const Sy
 {
     const int total = hdr->n_pos_total, n_sys = hdr->n_sys;
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < total; g += gridDim.x * blockDim.x) {
-        const SysDesc &d = sys[find_sys(sys, n_sys, g, false)];
+        const SysDesc &d = sys[find_sys(sys, n_sys, g)];
         const int i = g - d.pos_begin;
         double x = d.pos_in[3 * i] - d.qm[0], y = d.pos_in[3 * i + 1] - d.qm[1], z = d.pos_in[3 * i + 2] - d.qm[2];
         const int j = d.sorted ? d.slot_of[i] : i;
@@ -212,7 +212,7 @@ __global__ void batch_reduce_kernel(const BatchHeader *__restrict__ hdr, const S
 {
     const int total = hdr->n_pos_total, n_sys = hdr->n_sys;
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < total; g += gridDim.x * blockDim.x) {
-        const SysDesc &d = sys[find_sys(sys, n_sys, g, false)];
+        const SysDesc &d = sys[find_sys(sys, n_sys, g)];
         const int i = g - d.pos_begin;
         double s = 0.0, c = 0.0;
         if (d.n_tiles > 0)
@@ -846,7 +846,8 @@ cudaError_t launch_potential(int precision, const EvalArgs &a, int threads, int 
     return cudaErrorInvalidConfiguration;
 }
 
-cudaError_t launch_batch(int precision, const BatchHeader *hdr, const SysDesc *sys, int max_sys, int *counter,
+cudaError_t launch_batch(int precision, const BatchHeader *hdr, const SysDesc *sys, const BatchGroup *groups,
+                         int max_sys, int *counter,
                          int max_items, const float *boys32, const double *boys64, const float *boysdd, int tile_cap,
                          int threads, int ppt,
                          int num_sms, int max_pos_total, cudaStream_t s)
@@ -867,7 +868,7 @@ cudaError_t launch_batch(int precision, const BatchHeader *hdr, const SysDesc *s
     bool launched = false;
 #define ESP_BLAUNCH(NT, PPT, PR)                                                                                \
     if (!launched && threads == NT && ppt == PPT && precision == PR) {                                        \
-        e = launch_batch_shape<NT, PPT, PR>(hdr, sys, counter, max_items, boys32, boys64, boysdd, tile_cap, num_sms, smem, \
+        e = launch_batch_shape<NT, PPT, PR>(hdr, sys, groups, counter, max_items, boys32, boys64, boysdd, tile_cap, num_sms, smem, \
                                             s); \
         launched = true;                                                                                      \
     }

@@ -86,21 +86,30 @@ struct SysDesc {
     Staged st;
     double qm[3];
     double quantum;
-    int n_tiles, tile_size, n_pos, splits, blocks, item_begin, pos_begin;
+    int n_tiles, tile_size, n_pos, splits, blocks, pos_begin;
     float near_r;
     int sorted;           // stage in spatial order (slot_of / perm below are [n_pos] scratch)
     int *slot_of, *perm;
 };
 
+// The work items of one tile group of one system: items item_begin + range *
+// blocks + block, each range a contiguous part of the group's tiles with its own
+// partial sums (split split0 + range).  Entries are ordered by class first, so
+// that the CTAs of an SM run one class's code at a time.
+struct BatchGroup {
+    int item_begin, sys, tile0, n_tiles, ranges, split0;
+};
+
 struct BatchHeader {
-    int n_sys, n_items, n_pos_total, pad;
+    int n_sys, n_items, n_pos_total, n_groups;
 };
 
 // Batched pipeline on stream s: staging, persistent potential kernel over all
-// (system, block, split) items, reduction into each system's V_out.  The
+// (system, block, range of tiles) items, reduction into each system's V_out.  The
 // counter must be zero when the potential kernel starts.
 // max_sys: the number of systems (one spatial-order CTA each, for systems marked sorted)
-cudaError_t launch_batch(int precision, const BatchHeader *hdr, const SysDesc *sys, int max_sys, int *counter,
+cudaError_t launch_batch(int precision, const BatchHeader *hdr, const SysDesc *sys, const BatchGroup *groups,
+                         int max_sys, int *counter,
                          int max_items,
                          const float *boys32, const double *boys64, const float *boysdd, int tile_cap, int threads,
                          int ppt,

@@ -421,13 +421,25 @@ __global__ void __launch_bounds__(NT) potential_f64_kernel(EvalArgs a)
 // the device-side table (BatchHeader + SysDesc[]), so one captured CUDA graph
 // serves every call whose work fits the allocated capacity.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int find_sys(const SysDesc *__restrict__ sys, int n_sys, int key, bool by_item)
+__device__ __forceinline__ int find_sys(const SysDesc *__restrict__ sys, int n_sys, int pos)
 {
     int lo = 0, hi = n_sys - 1;
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
-        int v = by_item ? sys[mid].item_begin : sys[mid].pos_begin;
-        if (v <= key)
+        if (sys[mid].pos_begin <= pos)
+            lo = mid;
+        else
+            hi = mid - 1;
+    }
+    return lo;
+}
+
+__device__ __forceinline__ int find_group(const BatchGroup *__restrict__ groups, int n, int item)
+{
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        int mid = (lo + hi + 1) >> 1;
+        if (groups[mid].item_begin <= item)
             lo = mid;
         else
             hi = mid - 1;
@@ -440,8 +452,7 @@ __device__ __forceinline__ EvalArgs args_of(const SysDesc &d, const float *boys3
 {
     EvalArgs a;
     a.n_pos = d.n_pos;
-    a.n_splits = d.splits;
-    a.n_tiles = d.n_tiles;
+    a.n_splits = 1;
     a.tile_size = d.tile_size;
     a.pos = d.st;
     a.tiles = d.tiles;
@@ -453,15 +464,14 @@ __device__ __forceinline__ EvalArgs args_of(const SysDesc &d, const float *boys3
     a.boysdd = boysdd;
     a.dd_lim = d.dd_lim;
     a.pairs = 0;
-    a.partial = d.partial;
     a.near_r = d.near_r;
-    single_group(a);
     return a;
 }
 
 template <int NT, int PPT, int PREC>
 __global__ void __launch_bounds__(NT, PREC == 1 ? 512 / NT : 1) batch_potential_kernel(const BatchHeader *__restrict__ hdr,
-                                                             const SysDesc *__restrict__ sys, int *counter,
+                                                             const SysDesc *__restrict__ sys,
+                                                             const BatchGroup *__restrict__ groups, int *counter,
                                                              const float *boys32, const double *boys64,
                                                              const float *boysdd, int tile_cap)
 {
@@ -472,7 +482,7 @@ __global__ void __launch_bounds__(NT, PREC == 1 ? 512 / NT : 1) batch_potential_
     if (PREC == 1)
         for (int i = threadIdx.x; i < kBoys32Rows * kBoys32Row; i += NT)
             s_boys[i] = boys32[i];
-    const int n_items = hdr->n_items, n_sys = hdr->n_sys;
+    const int n_items = hdr->n_items, n_groups = hdr->n_groups;
     for (;;) {
         __syncthreads(); // s_item and the tile buffer are free again
         if (threadIdx.x == 0)
@@ -481,14 +491,19 @@ __global__ void __launch_bounds__(NT, PREC == 1 ? 512 / NT : 1) batch_potential_
         const int item = s_item;
         if (item >= n_items)
             break;
-        const int k = find_sys(sys, n_sys, item, true);
-        const SysDesc &d = sys[k];
-        const int local = item - d.item_begin;
-        const EvalArgs a = args_of(d, boys32, boys64, boysdd);
+        const BatchGroup g = groups[find_group(groups, n_groups, item)];
+        const SysDesc &d = sys[g.sys];
+        const int local = item - g.item_begin, range = local / d.blocks, bx = local % d.blocks;
+        EvalArgs a = args_of(d, boys32, boys64, boysdd);
+        const int t0 = int((long long)g.n_tiles * range / g.ranges), t1 = int((long long)g.n_tiles * (range + 1) / g.ranges);
+        a.tiles = d.tiles + g.tile0 + t0;
+        a.n_tiles = t1 - t0;
+        a.partial = d.partial + (size_t)(g.split0 + range) * d.n_pos;
+        single_group(a);
         if (PREC == 1)
-            cta_f32c<NT, PPT, true>(a, local / d.splits, local % d.splits, smem4, s_boys, s_acc);
+            cta_f32c<NT, PPT, true>(a, bx, 0, smem4, s_boys, s_acc);
         else
-            cta_f64<NT, PPT>(a, local / d.splits, local % d.splits, smem4);
+            cta_f64<NT, PPT>(a, bx, 0, smem4);
     }
 }
 

@@ -40,7 +40,7 @@ template cudaError_t launch_f64_shape<ESP_NT, ESP_PPT>(const EvalArgs &, dim3, s
 
 #elif defined(ESP_SHAPE_BATCH)
 template <int NT, int PPT, int PREC>
-cudaError_t launch_batch_shape(const BatchHeader *hdr, const SysDesc *sys, int *counter, int max_items,
+cudaError_t launch_batch_shape(const BatchHeader *hdr, const SysDesc *sys, const BatchGroup *groups, int *counter, int max_items,
                                const float *boys32, const double *boys64, const float *boysdd, int tile_cap, int num_sms, size_t smem,
                                cudaStream_t s)
 {
@@ -52,10 +52,11 @@ cudaError_t launch_batch_shape(const BatchHeader *hdr, const SysDesc *sys, int *
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NT, smem)) != cudaSuccess)
         return e;
     const int grid = std::max(1, std::min(per_sm * num_sms, max_items));
-    k<<<grid, NT, smem, s>>>(hdr, sys, counter, boys32, boys64, boysdd, tile_cap);
+    k<<<grid, NT, smem, s>>>(hdr, sys, groups, counter, boys32, boys64, boysdd, tile_cap);
     return cudaGetLastError();
 }
-template cudaError_t launch_batch_shape<ESP_NT, ESP_PPT, ESP_PREC>(const BatchHeader *, const SysDesc *, int *, int,
+template cudaError_t launch_batch_shape<ESP_NT, ESP_PPT, ESP_PREC>(const BatchHeader *, const SysDesc *, const BatchGroup *,
+                                                                   int *, int,
                                                                    const float *, const double *, const float *, int, int, size_t,
                                                                    cudaStream_t);
 #else

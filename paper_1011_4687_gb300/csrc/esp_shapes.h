@@ -25,7 +25,7 @@ cudaError_t launch_f64_shape(const EvalArgs &a, dim3 grid, size_t smem, cudaStre
 // The persistent batched kernel with as many CTAs as fit on the GPU (capped
 // at max_items work items).
 template <int NT, int PPT, int PREC>
-cudaError_t launch_batch_shape(const BatchHeader *hdr, const SysDesc *sys, int *counter, int max_items,
+cudaError_t launch_batch_shape(const BatchHeader *hdr, const SysDesc *sys, const BatchGroup *groups, int *counter, int max_items,
                                const float *boys32, const double *boys64, const float *boysdd, int tile_cap, int num_sms, size_t smem,
                                cudaStream_t s);
 
