@@ -366,7 +366,7 @@ def batch_leg(args, esp, torch, stream, flush, wls, oracle_mod=None):
            "value": evals / (ms_b * 1e-3), "unit": "evals/s", "ms_per_step": ms_b,
            "evals_per_step": evals, "separate_evals_ms": ms_s, "speedup_vs_separate": ms_s / ms_b,
            "tuned_shape": {k2: tune[k2] for k2 in ("threads_per_block", "positions_per_thread", "split_scale")},
-           "gpu_launches_per_step": 3}
+           "gpu_launches_per_step": 5}
     if acc is not None:
         res["accuracy"] = acc
     b.close()
@@ -519,7 +519,7 @@ def latency_leg(args, esp, torch, stream, oracle_mod=None):
             env.eval(hp, out=hv)
         us_host = (time.perf_counter() - t0) * 1e6 / reps
         leg = {"us_per_call": us, "us_per_call_graph_replay": us_graph, "us_per_call_host_buffers": us_host,
-               "evals_per_s": units * npos / (us * 1e-6), "launches_per_call": 2}
+               "evals_per_s": units * npos / (us * 1e-6), "launches_per_call": 1}
         if ref is not None:
             leg["max_point_err_ha"] = float(np.abs(Vg.cpu().numpy() - ref[:npos]).max())
         out["positions_%d" % npos] = leg
@@ -766,7 +766,7 @@ def fp32c_step_leg(args, wl, kind, env, esp, torch, stream, flush, world, local,
            "e2e": {"value": evals * world / statistics.mean(e2e_t), "unit": "evals/s",
                    "h2d_bytes_per_step": int(n_pos * 24), "d2h_bytes_per_step": int(n_pos * 8 + wl.n_walkers * 8),
                    "steps": len(e2e_t)},
-           "gpu_launches_per_step": 7 if n_pos >= 4096 else 4, "info": info}
+           "gpu_launches_per_step": 7 if n_pos >= 4096 else 5, "info": info}
     return res, pos, V, E
 
 
@@ -795,7 +795,9 @@ def fp64_leg(args, wl, env, torch, stream, flush, peaks):
             "sample": "%d whole walkers x %d electrons of the workload" % (nw, wl.n_elec), "ms_per_step": ms,
             "roofline": {"bound": "fp64", "achieved": achieved / 1e12, "peak": peaks["fp64_fma_per_s"] / 1e12,
                          "unit": "Tops/s (FP64 lane ops)", "frac": achieved / peaks["fp64_fma_per_s"],
-                         "kernel": "potential_f64_kernel", "kernel_ms": kms,
+                         "kernel": "potential_td_kernel", "kernel_ms": kms,
+                         "note": "far entries run on the FP32 pipe in exact FP32 words, so the plain FP64 "
+                                 "operation count can exceed the FP64 pipe's rate",
                          "ops_per_distribution_term": ops / max(terms, 1.0),
                          "peak_source": "measured DFMA lane-op rate (esp_measure_peaks) of measured"}}
 
@@ -876,9 +878,10 @@ def main(argv=None):
            "warmup": args.warmup, "ms_per_step": head["ms_per_step"], "higher_is_better": True, "scaling": "weak",
            "vs_baseline": None, "dtype": "f32", "data": "synthetic",
            "config": workload_config(wl, args.config, head["info"], world, reduced),
-           "path": {"precision": "FP32C (FP32 pair sum, compensated; nuclei and near blocks FP64)",
+           "path": {"precision": "FP32C (FP32 pair sum, compensated; nuclei and near blocks in FP32 pairs of 48 bits)",
                     "distributions_by_L": head["info"]["n_by_L"],
-                    "step": "esp_eval_walkers: spatial order (3 launches), stage, potential, reduce, walker energies"},
+                    "step": "esp_eval_walkers: spatial order (2 launches), stage, point charges and near blocks, "
+                            "potential, reduce, walker energies"},
            "gpu_launches": head["gpu_launches_per_step"] * args.steps,
            "clocks": head["clocks"], "roofline": head["roofline"], "e2e": head["e2e"], "fp64": f64,
            "peaks_measured": peaks}
