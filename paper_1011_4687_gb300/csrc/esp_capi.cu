@@ -44,12 +44,13 @@ int esp::choose_splits(const esp_ctx *c, const TileView &v, int n, int prec)
     int target = 48 * c->num_sms;
     int s = (target + blocks - 1) / blocks;
     // at most 64 partial sums per position where the blocks alone fill the GPU;
-    // with few blocks as many as give every SM eight CTAs (1,001 positions
+    // with few blocks as many as give every SM twelve CTAs (1,001 positions
     // against 894 tiles: 128 CTAs of 64 splits left 24 SMs idle and the others
-    // with one CTA)
-    const int fill = (8 * c->num_sms + blocks - 1) / blocks;
-    s = std::min(s, v.labels ? 64 : std::max(64, fill));
-    s = std::min(s, std::max(v.n_tiles, 1));
+    // with one CTA; 3,000 positions, 4 / 8 / 12 / 16 per SM: 444 / 355 / 343 /
+    // 340 us; 200 positions: 105 / 86 / 88 / 89)
+    const int fill = v.labels ? 64 : std::max(1, 12 * c->num_sms / blocks);
+    s = std::min(s, std::max(64, fill));
+    s = std::min(s, std::max(v.n_tiles, 1) << (prec == 1 && !v.labels ? kMaxPartShift : 0));
     return std::max(s, 1);
 }
 
@@ -64,6 +65,27 @@ bool esp::use_td(const esp_ctx *c, const TileView &v, int prec)
            c->opt.pair_splits == 0 && v.n_entries >= kTdMinEntries;
 }
 
+namespace {
+
+// Parts (log2) in which the tiles of group g are dealt: until one is at most
+// half of a split's load.  A tile of L = 4 takes seventeen times one of L = 0,
+// and with few position blocks a split's share is less than that: a call of
+// 1,001 positions x 889 tiles took 195 us in whole tiles and takes 155 in parts,
+// 200 positions 110 and 88, 400 positions x 4,000 s-charges 81 and 52.
+int part_shift(const esp_ctx *c, const TileView &v, int g, double load)
+{
+    const int tiles = v.grp_tile[g + 1] - v.grp_tile[g];
+    if (v.labels || c->opt.pair_splits > 0 || tiles <= 0)
+        return 0;
+    const double cost = v.grp_work[g] / tiles;
+    int s = 0;
+    while (s < kMaxPartShift && cost / (1 << s) > 0.5 * load)
+        ++s;
+    return s;
+}
+
+} // namespace
+
 int esp::plan_splits(const esp_ctx *c, const TileView &v, int n, int prec, int max_splits, EvalArgs &a, int &dd_splits)
 {
     a.n_tiles = v.n_tiles;
@@ -71,8 +93,10 @@ int esp::plan_splits(const esp_ctx *c, const TileView &v, int n, int prec, int m
     dd_splits = 0;
     a.pairs = prec == 1 && !v.labels && v.n_tiles > 0;
     if (use_td(c, v, prec)) {
-        a.n_splits = std::min(td_splits(n, v.n_tiles, c->num_sms), max_splits);
+        int shift;
+        a.n_splits = std::min(td_splits(n, v.n_tiles, c->num_sms, shift), max_splits);
         single_group(a);
+        a.grp_shift[0] = shift;
         return a.n_splits;
     }
     if (prec == 1 && v.n_dd > 0 && !v.labels) // (with few partial sums allowed, at most a quarter of them)
@@ -87,16 +111,19 @@ int esp::plan_splits(const esp_ctx *c, const TileView &v, int n, int prec, int m
     const int ng = v.n_groups - g0;
     if (prec == 1 && v.labels && v.n_dd > 0)
         dd_splits = 1;
-    if (prec == 0 || c->opt.pair_splits > 0 || v.n_groups <= 1 || ng > total)
-        return dd_splits + total;
     double work = 0.0;
     for (int g = g0; g < v.n_groups; ++g)
         work += v.grp_work[g];
-    int S[kMaxTileGroups], sum = 0;
+    if (prec == 1 && v.n_groups == 1)
+        a.grp_shift[0] = part_shift(c, v, 0, work / total);
+    if (prec == 0 || c->opt.pair_splits > 0 || v.n_groups <= 1 || ng > total)
+        return dd_splits + total;
+    int S[kMaxTileGroups], shift[kMaxTileGroups], sum = 0;
     for (int g = g0; g < v.n_groups; ++g) {
         const int tiles = v.grp_tile[g + 1] - v.grp_tile[g];
         const int want = int(std::lround(total * v.grp_work[g] / std::max(work, 1e-300)));
-        S[g] = std::max(1, std::min(want, tiles));
+        shift[g] = part_shift(c, v, g, work / total);
+        S[g] = std::max(1, std::min(want, tiles << shift[g]));
         sum += S[g];
     }
     while (sum > total) { // give back from the group with the most splits
@@ -115,6 +142,7 @@ int esp::plan_splits(const esp_ctx *c, const TileView &v, int n, int prec, int m
     a.grp_split[0] = 0;
     for (int g = 0; g < a.n_groups; ++g) {
         a.grp_tile[g] = v.grp_tile[gp + g];
+        a.grp_shift[g] = shift[gp + g];
         a.grp_split[g + 1] = a.grp_split[g] + S[gp + g];
     }
     a.grp_tile[a.n_groups] = v.grp_tile[v.n_groups];

@@ -142,19 +142,24 @@ __global__ void __launch_bounds__(kDdThreads, 4) potential_td_kernel(EvalArgs a)
     const double x = a.pos.x64[ic], y = a.pos.y64[ic], z = a.pos.z64[ic];
     const bool in_range = dd_in_range(c.h, a.dd_lim);
     double S = 0.0, Cc = 0.0;
-    for (int k = blockIdx.y; k < a.n_tiles; k += gridDim.y) {
-        const TileMeta m = a.tiles[k];
+    const int shift = a.grp_shift[0], part = a.tile_size >> shift;
+    for (int k = blockIdx.y; k < a.n_tiles << shift; k += gridDim.y) {
+        const TileMeta m = a.tiles[k >> shift];
         const bool pts = is_point_class(m.cls);
-        const double *rec64 = a.rec64 + m.off64;
+        // this part's records [p0, p0 + n)
+        const int p0 = (k & ((1 << shift) - 1)) * part, n = min(m.n - p0, part);
+        if (n <= 0)
+            continue;
+        const double *rec64 = a.rec64 + m.off64 + (size_t)p0 * (pts ? kPointStride64 : rec64_stride(m.cls & 7));
         if (m.offdd < 0) {
-            two_sum_acc(S, Cc, pts ? point_tile_f64(rec64, m.n, x, y, z)
-                                   : tile_f64_one_any(m.cls, rec64, m.n, x, y, z, a.boys64));
+            two_sum_acc(S, Cc, pts ? point_tile_f64(rec64, n, x, y, z)
+                                   : tile_f64_one_any(m.cls, rec64, n, x, y, z, a.boys64));
             continue;
         }
-        const int n4 = dd_pad(m.n), L = m.cls & 7;
+        const int n4 = dd_pad(n), L = m.cls & 7;
         __syncthreads(); // the previous tile is fully consumed
-        copy_tile(smem4, reinterpret_cast<const float4 *>(a.recdd) + m.offdd,
-                  (pts ? kDdPointWords : dd_far_words(L)) * n4 / 4);
+        copy_part(smem4, reinterpret_cast<const float4 *>(a.recdd) + m.offdd, pts ? kDdPointWords : dd_far_words(L),
+                  dd_pad(m.n), p0, n4);
         __syncthreads();
         float r2min = 1.0f;
         double v = 0.0;
@@ -186,14 +191,14 @@ __global__ void __launch_bounds__(kDdThreads, 4) potential_td_kernel(EvalArgs a)
                 }
                 for (unsigned long long b = near; b; b &= b - 1) {
                     const int j = j0 + __ffsll((long long)b) - 1;
-                    if (j < m.n) // (padding repeats the last record)
+                    if (j < n) // (padding repeats the last record)
                         v += near_entry(m.cls, rec64 + (size_t)j * rec64_stride(L), x, y, z, a.boys64);
                 }
             }
         }
         // closer than the words resolve, or out of their range
         if (!(r2min >= kDdMinR2) || !in_range)
-            v = pts ? point_tile_f64(rec64, m.n, x, y, z) : tile_f64_one_any(m.cls, rec64, m.n, x, y, z, a.boys64);
+            v = pts ? point_tile_f64(rec64, n, x, y, z) : tile_f64_one_any(m.cls, rec64, n, x, y, z, a.boys64);
         two_sum_acc(S, Cc, v);
     }
     if (i < a.n_pos)
@@ -241,13 +246,20 @@ cudaError_t launch_dd_sum(const EvalArgs &a, const int *list, int n_list, int n_
     return cudaGetLastError();
 }
 
-int td_splits(int n, int n_tiles, int num_sms)
+int td_splits(int n, int n_tiles, int num_sms, int &shift)
 {
     const int blocks = (n + kDdThreads - 1) / kDdThreads;
-    // 16 CTAs per SM where the tiles allow it; not more partial sums than 64
-    // where the blocks alone give every SM several
-    const int fill = (16 * num_sms + blocks - 1) / blocks;
-    return std::max(1, std::min(n_tiles, std::min(fill, std::max(64, (8 * num_sms + blocks - 1) / blocks))));
+    // One wave of the four CTAs an SM holds, two where that would leave fewer
+    // than 16 splits: a partial second wave costs a whole one (2,048 positions x
+    // 889 tiles: 38 splits, one wave, 1.56 ms; 47: 2.20; 57: 1.74; 76: 1.71).
+    const int wave = 4 * num_sms / blocks;
+    const int want = std::max(1, wave >= 16 ? wave : 8 * num_sms / blocks);
+    // parts of tiles until a split has eight of them (1,999 positions x 39 tiles:
+    // 188 us in whole tiles, 151 in quarters, 160 in eighths)
+    shift = 0;
+    while (shift < kMaxPartShift && n_tiles << shift < 8 * want)
+        ++shift;
+    return std::max(1, std::min(n_tiles << shift, want));
 }
 
 cudaError_t launch_td(const EvalArgs &a, cudaStream_t s)

@@ -17,6 +17,20 @@ __device__ __forceinline__ void copy_tile(float4 *__restrict__ dst, const float4
         dst[i] = __ldg(src + i);
 }
 
+// words [0, words) of records [j0, j0 + n4p) of a dd tile of n4 records (j0 and
+// n4p multiples of 4), as a tile of n4p records
+__device__ __forceinline__ void copy_part(float4 *__restrict__ dst, const float4 *__restrict__ src, int words, int n4,
+                                          int j0, int n4p)
+{
+    if (n4p == n4)
+        return copy_tile(dst, src, words * n4 / 4);
+    const int q = n4p / 4;
+    for (int i = threadIdx.x; i < words * q; i += blockDim.x) {
+        const int w = i / q;
+        dst[i] = __ldg(src + w * (n4 / 4) + j0 / 4 + (i - w * q));
+    }
+}
+
 __device__ __forceinline__ DdPos dd_position(const Staged &p, int i)
 {
     return {{p.xh[i], p.yh[i], p.zh[i]}, {p.xm[i], p.ym[i], p.zm[i]}, {p.xr[i], p.yr[i], p.zr[i]}};

@@ -36,6 +36,7 @@ inline Staged staged_at(void *b, size_t n)
 // FP32C tile groups: FP64 point charges, FP32 point charges, then one group
 // per L (long- and short-range tiles of that L together).
 constexpr int kMaxTileGroups = 7;
+constexpr int kMaxPartShift = 2; // tiles are dealt in up to four parts
 
 struct EvalArgs {
     int n_pos;
@@ -61,6 +62,8 @@ struct EvalArgs {
     int n_groups;
     int grp_tile[kMaxTileGroups + 1];
     int grp_split[kMaxTileGroups + 1];
+    // A group's tiles are dealt in 2^grp_shift parts of tile_size >> grp_shift records.
+    int grp_shift[kMaxTileGroups];
 };
 
 // the plain deal: every tile in one group over n_splits splits
@@ -71,6 +74,7 @@ ESP_HD void single_group(EvalArgs &a)
     a.grp_tile[1] = a.n_tiles;
     a.grp_split[0] = 0;
     a.grp_split[1] = a.n_splits;
+    a.grp_shift[0] = 0;
 }
 
 // One system of a batched evaluation (device-side table entry).
@@ -123,7 +127,7 @@ int dd_sum_splits(int n, int n_list, int num_sms);
 cudaError_t launch_dd_sum(const EvalArgs &a, const int *list, int n_list, int n_splits, cudaStream_t s);
 // All tiles at FP64 accuracy into a.n_splits partial sums (esp_ddsum.cu): far
 // entries in FP32 words, the others in FP64.
-int td_splits(int n, int n_tiles, int num_sms);
+int td_splits(int n, int n_tiles, int num_sms, int &shift);
 cudaError_t launch_td(const EvalArgs &a, cudaStream_t s);
 // dd records (esp_dd.h) of the tiles with offdd >= 0, on the coordinate grid q
 cudaError_t launch_dd_build(const TileMeta *tiles, int n_tiles, const double *rec64, double q, float *recdd,

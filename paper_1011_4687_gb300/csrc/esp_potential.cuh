@@ -80,9 +80,15 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
     while (g + 1 < a.n_groups && split >= a.grp_split[g + 1])
         ++g;
     const int g_stride = a.grp_split[g + 1] - a.grp_split[g];
-    const int g_end = a.grp_tile[g + 1];
-    for (int t = a.grp_tile[g] + (split - a.grp_split[g]); t < g_end; t += g_stride) {
-        const TileMeta m = a.tiles[t];
+    const int shift = ALL ? 0 : a.grp_shift[g];
+    const int g_units = (a.grp_tile[g + 1] - a.grp_tile[g]) << shift;
+    for (int u = split - a.grp_split[g]; u < g_units; u += g_stride) {
+        const TileMeta m = a.tiles[a.grp_tile[g] + (u >> shift)];
+        // this part's records [j0, j0 + n)
+        const int j0 = ALL ? 0 : (u & ((1 << shift) - 1)) * (a.tile_size >> shift);
+        const int n = ALL ? m.n : min(m.n - j0, a.tile_size >> shift);
+        if (!ALL && n <= 0)
+            continue;
         if (!ALL && m.cls == kClassPoint)
             continue;
         __syncthreads(); // previous tile fully consumed
@@ -91,9 +97,9 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
         const int n4 = dd_pad(m.n);
         const float4 *s_dd = reinterpret_cast<const float4 *>(a.recdd) + (ddt ? m.offdd : 0);
         const float4 *src = pts ? (ddt ? s_dd : reinterpret_cast<const float4 *>(a.rec64 + m.off64))
-                                : reinterpret_cast<const float4 *>(a.rec32 + m.off32);
+                                : reinterpret_cast<const float4 *>(a.rec32 + m.off32 + j0 * rec32_stride_cls(m.cls));
         const int nvec = pts ? (ddt ? kDdPointWords * n4 / 4 : m.n * 2)
-                             : (m.n * rec32_stride_cls(m.cls)) / 4;
+                             : (n * rec32_stride_cls(m.cls)) / 4;
         copy_tile(s_tile4, src, nvec);
         if (!ALL)
             asm volatile("cp.async.wait_all;" ::: "memory"); // the Boys table, once
@@ -131,7 +137,7 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
 #pragma unroll
                     for (int d = 0; d < 3; ++d)
                         th2[q][d] = f2(0.0f) - ch2[q][d];
-                tile_f32c2<0, NP, true, false, false>(s_rec, m.n, th2, cl2, cl2, wq, S2, C2, s_boys);
+                tile_f32c2<0, NP, true, false, false>(s_rec, n, th2, cl2, cl2, wq, S2, C2, s_boys);
             } else {
                 bool none[PPT];
                 float th[PPT][3];
@@ -142,7 +148,7 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
                     for (int d = 0; d < 3; ++d)
                         th[q][d] = 0.0f - ch[q][d];
                 }
-                tile_f32c<0, PPT, true, false, false>(s_rec, m.n, th, cl, cl, none, S, Cc, s_boys);
+                tile_f32c<0, PPT, true, false, false>(s_rec, n, th, cl, cl, none, S, Cc, s_boys);
             }
             continue;
         }
@@ -206,13 +212,13 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
 #define ESP_TILE(CLS, LL, SH)                                                                         \
     case CLS:                                                                                         \
         if (rel && !sel)                                                                              \
-            tile_f32c2<LL, NP, true, SH, false, true>(s_rec, m.n, th2, cl2, dq2, wq, S2, C2, s_boys); \
+            tile_f32c2<LL, NP, true, SH, false, true>(s_rec, n, th2, cl2, dq2, wq, S2, C2, s_boys); \
         else if (far && !sel)                                                                         \
-            tile_f32c2<LL, NP, true, SH, false>(s_rec, m.n, th2, cl2, dq2, wq, S2, C2, s_boys);       \
+            tile_f32c2<LL, NP, true, SH, false>(s_rec, n, th2, cl2, dq2, wq, S2, C2, s_boys);       \
         else if (far)                                                                                 \
-            tile_f32c2<LL, NP, true, SH, true>(s_rec, m.n, th2, cl2, dq2, wq, S2, C2, s_boys);        \
+            tile_f32c2<LL, NP, true, SH, true>(s_rec, n, th2, cl2, dq2, wq, S2, C2, s_boys);        \
         else                                                                                          \
-            tile_f32c2<LL, NP, false, SH, true>(s_rec, m.n, th2, cl2, dq2, wq, S2, C2, s_boys);       \
+            tile_f32c2<LL, NP, false, SH, true>(s_rec, n, th2, cl2, dq2, wq, S2, C2, s_boys);       \
         break;
             switch (m.cls) {
                 ESP_TILE(0, 0, false)
@@ -240,13 +246,13 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
 #define ESP_TILE(CLS, LL, SH)                                                                         \
     case CLS:                                                                                         \
         if (rel && !sel)                                                                              \
-            tile_f32c<LL, PPT, true, SH, false, true>(s_rec, m.n, th, cl, dq, nearq, S, Cc, s_boys);  \
+            tile_f32c<LL, PPT, true, SH, false, true>(s_rec, n, th, cl, dq, nearq, S, Cc, s_boys);  \
         else if (far && !sel)                                                                         \
-            tile_f32c<LL, PPT, true, SH, false>(s_rec, m.n, th, cl, dq, nearq, S, Cc, s_boys);        \
+            tile_f32c<LL, PPT, true, SH, false>(s_rec, n, th, cl, dq, nearq, S, Cc, s_boys);        \
         else if (far)                                                                                 \
-            tile_f32c<LL, PPT, true, SH, true>(s_rec, m.n, th, cl, dq, nearq, S, Cc, s_boys);         \
+            tile_f32c<LL, PPT, true, SH, true>(s_rec, n, th, cl, dq, nearq, S, Cc, s_boys);         \
         else                                                                                          \
-            tile_f32c<LL, PPT, false, SH, true>(s_rec, m.n, th, cl, dq, nearq, S, Cc, s_boys);        \
+            tile_f32c<LL, PPT, false, SH, true>(s_rec, n, th, cl, dq, nearq, S, Cc, s_boys);        \
         break;
             switch (m.cls) {
                 ESP_TILE(0, 0, false)
@@ -297,6 +303,8 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
             }
         }
     }
+    if (!ALL) // (a split without a part)
+        asm volatile("cp.async.wait_all;" ::: "memory");
     if constexpr (PPT % 2 == 0) {
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
