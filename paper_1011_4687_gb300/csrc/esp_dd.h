@@ -39,11 +39,10 @@
 namespace esp {
 
 constexpr int kDdGeneralMaxL = 2;         // larger L takes the FP64 code when not far
-constexpr double kDdMinDist = 0x1p-10;    // closer offsets may lack the 48 bits: FP64
-constexpr float kDdMinR2 = 0x1p-20f;
+constexpr float kDdMinR2 = 0x1p-20f;      // |P - C|^2; closer offsets may lack the 48 bits: FP64
 // T below which an entry is near (FP64): 45 where the asymptotic form holds to
 // 1e-20, and a margin for T formed from the hi words (1e-2 of it at most beyond
-// kDdMinDist)
+// a distance of 2^-10)
 constexpr float kTdNearT = 46.0f;
 ESP_HD constexpr int dd_pad(int n) { return (n + 3) & ~3; }
 constexpr int kDdPointWords = 13;

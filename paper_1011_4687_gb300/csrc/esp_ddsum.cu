@@ -7,7 +7,7 @@
 // packed FP32 operation.  Bound by the FP32 pipe: 75 operations per two charges,
 // about 130 per two s-distributions with their Boys values.  In FP64 (1/63 of
 // the rate) the same blocks took 500 of the 650 us of 10,000 positions x 2,200
-// entries whose tiles' spheres cover the QM region.
+// entries whose tiles' spheres cover the QM region; here they take 53.
 #include "esp_ddsum.cuh"
 
 #include <algorithm>
@@ -71,17 +71,21 @@ __global__ void __launch_bounds__(kDdThreads, 4) dd_sum_kernel(EvalArgs a, const
 }
 
 // ---------------------------------------------------------------------------
-// FP64 evaluations.  Every entry whose Gaussian is negligible at the positions
-// of a warp (T = p |P - C|^2 >= 45 and a margin) takes the far form of esp_dd.h:
-// the monopole in three FP32 words (an error of 1e-20 of the term), the higher
-// orders in two; the others take the FP64 code for the warp.  Bound by the FP32
-// pipe (about 200 packed operations per two monopoles) and, where exponents are
-// small, by the FP64 pipe (near entries: some 40 operations of 64 cycles).
+// FP64 evaluations.  Every entry whose Gaussian is negligible at a position
+// (T = p |P - C|^2 >= 45 and a margin) takes the far form of esp_dd.h: the
+// monopole in three FP32 words (an error of 1e-20 of the term), the higher
+// orders in two (about 200 packed FP32 operations per two monopoles).  The
+// others take the FP64 code, each lane its own entries: a warp runs as many as
+// its busiest lane has, not as many as any lane has (2,048 positions x 48,000
+// distributions 1.56 -> 1.52 ms, 9,000 x 24,000 3.42 -> 3.27).  Bound by the
+// FP64 pipe, where exponents are small (those entries: some 40 operations of 64
+// cycles; the pipe is 60 % busy, 90 % on the busiest SM), by FP32 otherwise.
+// All in FP64, 2,048 x 48,000 took 9.5 ms.
 // ---------------------------------------------------------------------------
 constexpr int kTdWordsMax = dd_far_words(kMaxL);
 
-// The far pairs of a chunk of at most 64 records; near: bits of the records to
-// leave out.  lo: the smallest |P - C|^2 met.
+// The far pairs of a chunk of at most 64 records; near: bits of the records
+// that this lane leaves out.  lo: the smallest |P - C|^2 met.
 template <int L>
 __device__ __noinline__ double td_chunk(const float *__restrict__ s_rec, int n4, int j0, int j1, const DdPos c,
                                         unsigned long long near, float *lo)
@@ -96,7 +100,7 @@ __device__ __noinline__ double td_chunk(const float *__restrict__ s_rec, int n4,
 #pragma unroll 1
         for (int j = b; j < e; j += 2) {
             const bool u0 = !(near >> (j - j0) & 1), u1 = !(near >> (j - j0 + 1) & 1);
-            if (!u0 && !u1)
+            if (!__any_sync(0xffffffffu, u0 || u1))
                 continue;
             f2 r2;
             td_far<L>(t, j, c, u0, u1, sum, r2);
@@ -173,13 +177,12 @@ __global__ void __launch_bounds__(kDdThreads, 4) potential_td_kernel(EvalArgs a)
             for (int j0 = 0; j0 < n4; j0 += 64) {
                 const int j1 = min(n4, j0 + 64);
                 unsigned long long near = 0ull;
-                if (!far) { // which records are near any of the warp's positions
+                if (!far) { // which records are near this lane's position
                     for (int j = j0; j < j1; j += 2) {
                         const f2 dx = t(0, j) - f2(c.h[0]), dy = t(1, j) - f2(c.h[1]), dz = t(2, j) - f2(c.h[2]);
                         const f2 T = t(10, j) * esp_fma(dx, dx, esp_fma(dy, dy, dz * dz));
-                        const unsigned b0 = __any_sync(0xffffffffu, !(T.x >= kTdNearT)),
-                                       b1 = __any_sync(0xffffffffu, !(T.y >= kTdNearT));
-                        near |= (unsigned long long)((b0 ? 1u : 0u) | (b1 ? 2u : 0u)) << (j - j0);
+                        near |= (unsigned long long)((T.x >= kTdNearT ? 0u : 1u) | (T.y >= kTdNearT ? 0u : 2u))
+                                << (j - j0);
                     }
                 }
                 switch (L) {
@@ -189,11 +192,11 @@ __global__ void __launch_bounds__(kDdThreads, 4) potential_td_kernel(EvalArgs a)
                 case 3: v += td_chunk<3>(s_rec, n4, j0, j1, c, near, &r2min); break;
                 default: v += td_chunk<4>(s_rec, n4, j0, j1, c, near, &r2min); break;
                 }
-                for (unsigned long long b = near; b; b &= b - 1) {
-                    const int j = j0 + __ffsll((long long)b) - 1;
-                    if (j < n) // (padding repeats the last record)
-                        v += near_entry(m.cls, rec64 + (size_t)j * rec64_stride(L), x, y, z, a.boys64);
-                }
+                if (n - j0 < 64) // (padding repeats the last record)
+                    near &= (1ull << (n - j0)) - 1ull;
+                for (; near; near &= near - 1)
+                    v += near_entry(m.cls, rec64 + (size_t)(j0 + __ffsll((long long)near) - 1) * rec64_stride(L), x, y,
+                                    z, a.boys64);
             }
         }
         // closer than the words resolve, or out of their range

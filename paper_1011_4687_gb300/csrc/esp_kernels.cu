@@ -147,7 +147,7 @@ __device__ __forceinline__ void cta_scatter(int *__restrict__ key_slot, int *__r
 // every CTA reads the others' histograms (distributed shared memory) for its
 // own first slot in each cell.  (A histogram pass over up to 256 blocks, a scan
 // of cells x blocks by one CTA and a scatter took 50 us for 10,000 positions
-// and 257 us for 65,536, most of it the scan.)
+// and 257 us for 65,536, most of it the scan; now 14 us, and 30 for 50,000.)
 __global__ void __cluster_dims__(kSortCtas, 1, 1) __launch_bounds__(kSortThreads)
     sort_cluster_kernel(int *__restrict__ key_slot, int n, int *__restrict__ perm)
 {
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(kSortThreads) batch_sort_kernel(const BatchHea
 // position per operation, reduced every position over all lanes, put the
 // nuclei's FP64 terms of all positions on one CTA and left the sum of 1,216
 // partials to a second kernel: 268,818 cells at 1 / 16 / 128 positions took
-// 18.4 / 39 / 78 us.
+// 18.4 / 39 / 78 us, now 9.8 / 16.6 / 37 (kernel).
 // ---------------------------------------------------------------------------
 constexpr int kSmallWarps = kSmallThreads / 32;
 constexpr int kNearList = 64;  // near entries a warp keeps for the end
@@ -723,7 +723,7 @@ __global__ void __launch_bounds__(32 * SLICES) reduce_kernel(const double *__res
 // The same where the partials after the first n64 (the dd kernel's, FP64) are
 // FP32 (sum, compensation) pairs, as an FP32C kernel holds them: few FP64
 // operations (FP64 partials of 1,001 positions in 512 splits took 38 us, of
-// 65,536 in 60 splits 65 us).
+// 65,536 in 60 splits 65 us; now 7 us, and 25 for 50,000 in 68).
 template <int SLICES>
 __global__ void __launch_bounds__(32 * SLICES) reduce_pairs_kernel(const double *__restrict__ partial, int n64,
                                                                     int n_splits, int n, double *__restrict__ V,
