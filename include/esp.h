@@ -114,13 +114,15 @@ typedef struct {
     int32_t flags;                 /* ESP_FLAG_* bits; 0 for normal use */
     double near_radius;            /* FP32C: a (position, tile) block whose distance to the
                                       tile's bounding sphere is below this is evaluated in
+                                      pairs of FP32 numbers (48 bits) or
                                       FP64, for tiles holding a distribution whose potential
                                       can exceed 2 Ha (a compact charge not merged into a
                                       point charge); < 0 = default (1.5 bohr), 0 = off */
     double point32_max_charge;     /* FP32C: point charges with |Z| at or below this (the paper's
                                       density cells) are summed in compensated FP32 like the
                                       distributions, larger ones (nuclei, merged monopoles) in
-                                      FP64; < 0 = default (0.25), 0 = every point charge FP64 */
+                                      pairs of FP32 numbers (48 bits) or FP64; < 0 = default
+                                      (0.25), 0 = every point charge so */
 } esp_options;
 
 /* Per-context facts, for reporting and for counting evaluations. */
@@ -163,7 +165,8 @@ esp_status esp_create(const esp_point_charge *charges, int64_t n_charges,
  *   V_out     [n]    same space as positions, float64
  * Calls with at most 16 positions (the paper's one r_new per Metropolis move,
  * Sec. III) spread the environment's entries over the GPU's threads instead
- * of the positions and evaluate in FP64 whatever the precision setting.
+ * of the positions and evaluate to FP64 accuracy (small point charges in
+ * compensated FP32) whatever the precision setting.
  * n == 0 is a no-op.  Errors: ESP_ERR_INVALID, ESP_ERR_STATE, ESP_ERR_CUDA,
  * ESP_ERR_TIMEOUT, ESP_ERR_OOM. */
 esp_status esp_eval(esp_ctx *ctx, const double *positions, int64_t n, double *V_out);
@@ -215,7 +218,7 @@ esp_status esp_eval_noalloc(esp_ctx *ctx, const double *positions, int64_t n, do
  * stream, so the caller writes the next positions into the same buffer (on
  * that stream, or before the launch) and reads V after it.  The precision is
  * the context's at creation (ESP_FP32C: small point charges in compensated
- * FP32, everything else FP64; ESP_FP64: all FP64).
+ * FP32, everything else to FP64 accuracy; ESP_FP64: all to FP64 accuracy).
  * ------------------------------------------------------------------------ */
 #define ESP_GRAPH_MAX_POSITIONS 128
 typedef struct esp_graph esp_graph;
