@@ -514,9 +514,16 @@ __global__ void __launch_bounds__(kSmallThreads, NQ <= 4 ? 2 : 1) small_n_kernel
             const int o = u / a.tile_parts;
             const int tile = o < a.skip_begin ? o : o + a.n_skip;
             const TileMeta m = a.tiles[tile];
-            const int j = (u % a.tile_parts) * 64 + 2 * lane;
+            const int j = a.direct ? (u % a.tile_parts) * 32 + lane : (u % a.tile_parts) * 64 + 2 * lane;
             const bool words = m.offdd >= 0 && dd_in_range(s_dd[q].h, a.dd_lim);
-            if (m.cls == kClassPoint && a.points_dd) {
+            if (a.direct) { // (FP64 throughout)
+                double v = j < m.n ? entry_f64(a, m, j, s_pos[q]) : 0.0;
+#pragma unroll
+                for (int w = 16; w > 0; w >>= 1)
+                    v += __shfl_xor_sync(0xffffffffu, v, w);
+                if (lane == 0)
+                    s_red64[warp][q] += v;
+            } else if (m.cls == kClassPoint && a.points_dd) {
                 // beside FP32 sums: dd sums
                 float s = 0.0f, c = 0.0f;
                 if (j < m.n) {
@@ -917,7 +924,8 @@ int small_grid(int g_threads, int num_sms, int chunks, bool fp32)
 size_t small_n_bytes(int n_tiles, int num_sms, int n)
 {
     const int chunks = std::max(1, (n + kSmallChunk - 1) / kSmallChunk);
-    return (size_t)small_grid(small_n_threads(n_tiles, num_sms, n), num_sms, chunks, true) * chunks * small_nq(n) * (sizeof(float2) + sizeof(double));
+    const int grid = std::max(small_grid(small_n_threads(n_tiles, num_sms, n), num_sms, chunks, true), num_sms / chunks);
+    return (size_t)grid * chunks * small_nq(n) * (sizeof(float2) + sizeof(double));
 }
 
 cudaError_t launch_small_n(SmallArgs a, void *scratch, int num_sms, double *V, cudaStream_t s)
@@ -927,7 +935,9 @@ cudaError_t launch_small_n(SmallArgs a, void *scratch, int num_sms, double *V, c
     a.g_threads = small_n_threads(a.n_tiles, num_sms, a.n_pos);
     const int nq = small_nq(a.n_pos);
     const int chunks = (a.n_pos + kSmallChunk - 1) / kSmallChunk;
-    const dim3 grid(small_grid(a.g_threads, num_sms, chunks, a.n_p32 > 0), chunks);
+    dim3 grid(small_grid(a.g_threads, num_sms, chunks, a.n_p32 > 0), chunks);
+    if (a.direct) // latency counts: a part per CTA
+        grid.x = std::max(int(grid.x), std::min(a.n_other * a.tile_parts, num_sms / chunks));
     a.part64 = static_cast<double *>(scratch);
     a.part32 = reinterpret_cast<float2 *>(a.part64 + (size_t)grid.x * grid.y * nq);
     switch (nq) {
