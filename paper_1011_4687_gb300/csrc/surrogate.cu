@@ -329,7 +329,9 @@ esp_status upload_split(esp_surrogate *s)
 {
     cudaError_t e;
     const bool near = near_radius(s->ctx) > 0.0f;
-    const std::vector<int> nd = dd_tile_list(s->near_tiles, near), fd = dd_tile_list(s->far_tiles, false);
+    // ("near" there is close to the QM sphere; here, within near_radius of a
+    // position, which far tiles can be too: the dd kernel sums those blocks)
+    const std::vector<int> nd = dd_tile_list(s->near_tiles, near), fd = dd_tile_list(s->far_tiles, near);
     if ((e = upload_vec(s->d_near_tiles, s->near_tiles)) != cudaSuccess ||
         (e = upload_vec(s->d_far_tiles, s->far_tiles)) != cudaSuccess ||
         (e = upload_vec(s->d_near_dd, nd)) != cudaSuccess || (e = upload_vec(s->d_far_dd, fd)) != cudaSuccess)
