@@ -39,11 +39,24 @@
 namespace esp {
 
 constexpr int kDdGeneralMaxL = 2;         // larger L takes the FP64 code when not far
-constexpr float kDdMinR2 = 0x1p-20f;      // |P - C|^2; closer offsets may lack the 48 bits: FP64
+// The words of an offset hold it to 2^-48 q, and its hi word alone (the
+// difference of two roundings to the grid q) is off by up to sqrt(3) q.  So the
+// words are used where offsets are at least 256 q long, which the coordinates of
+// the environment decide (q = 2^-24 times a power of two above 4 max |P|):
+//  - distributions: tiles with q sqrt(p) above kDdMaxQs keep the FP64 code, so
+//    that T = p |P - C|^2 >= 46 (kTdNearT) implies |P - C| >= 6.78 / sqrt(p) >= 271 q;
+//  - point charges: closer positions take the FP64 code (dd_min_r2), as do all
+//    closer than 2^-10 bohr;
+//  - environments with q above kDdMaxQuantum (beyond 16,384 bohr) have no dd
+//    records at all.  (That also keeps d^4 below 2^64: FP32's range.)
+constexpr double kDdMaxQuantum = 0x1p-8;
+constexpr double kDdMaxQs = 0.025;
 // T below which an entry is near (FP64): 45 where the asymptotic form holds to
-// 1e-20, and a margin for T formed from the hi words (1e-2 of it at most beyond
-// a distance of 2^-10)
+// 1e-20, and 2.2 % for T formed from the hi words (1.3 % at most from 256 q on)
 constexpr float kTdNearT = 46.0f;
+constexpr float kDdMinR2 = 0x1p-20f;
+// Smallest |P - C|^2 of a point charge in words; lim = 2^23 q (dd_limit).  At most 1.
+ESP_HD float dd_min_r2(float lim) { return fmaxf(kDdMinR2, (lim * 0x1p-15f) * (lim * 0x1p-15f)); }
 ESP_HD constexpr int dd_pad(int n) { return (n + 3) & ~3; }
 constexpr int kDdPointWords = 13;
 ESP_HD constexpr int dd_far_words(int L) { return 11 + 2 * num_hermite(L); }
@@ -466,7 +479,7 @@ ESP_HD void dd_offsets(const DdTile &t, int j, const DdPos &c, dd (&d)[3])
 }
 
 // Point charges j, j + 1: Z / |P - C|; r2 receives |P - C|^2 (the caller
-// re-evaluates in FP64 below kDdMinR2).
+// re-evaluates in FP64 below dd_min_r2).
 ESP_HD dd dd_point(const DdTile &t, int j, const DdPos &c, f2 &r2)
 {
     dd d[3];

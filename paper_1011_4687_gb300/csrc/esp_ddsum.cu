@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(kDdThreads, 4) dd_sum_kernel(EvalArgs a, const
             float r2min;
             double v = dd_sum_points(s_rec, n4, c, &r2min);
             // closer than the dd words resolve, or out of their range
-            if (!(r2min >= kDdMinR2) || !in_range)
+            if (!(r2min >= dd_min_r2(a.dd_lim)) || !in_range)
                 v = point_tile_f64(a.rec64 + m.off64, m.n, a.pos.x64[ic], a.pos.y64[ic], a.pos.z64[ic]);
             acc += v;
         } else if (__any_sync(0xffffffffu, mine)) {
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(kDdThreads, 4) potential_td_kernel(EvalArgs a)
             }
         }
         // closer than the words resolve, or out of their range
-        if (!(r2min >= kDdMinR2) || !in_range)
+        if (!(r2min >= dd_min_r2(a.dd_lim)) || !in_range)
             v = pts ? point_tile_f64(rec64, n, x, y, z) : tile_f64_one_any(m.cls, rec64, n, x, y, z, a.boys64);
         two_sum_acc(S, Cc, v);
     }

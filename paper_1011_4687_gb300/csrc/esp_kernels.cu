@@ -386,7 +386,7 @@ __device__ __forceinline__ double entries_words(const SmallArgs &a, const TileMe
         default: v = far_pair<4>(t, j, c, !n0, !n1, &r2min); break;
         }
     }
-    if (!(r2min >= kDdMinR2)) { // closer than the words resolve
+    if (!(r2min >= dd_min_r2(a.dd_lim))) { // closer than the words resolve
         v = 0.0;
         n0 = n1 = true;
     }
@@ -532,7 +532,7 @@ __global__ void __launch_bounds__(kSmallThreads, NQ <= 4 ? 2 : 1) small_n_kernel
                     const dd v = dd_point(tile, j, s_dd[q], r2);
                     s = v.h.x, c = v.l.x;
                     two_sum_pair(s, c, v.h.y, v.l.y); // (a padding charge is zero)
-                    if (!(fminf(r2.x, r2.y) >= kDdMinR2) || !words) {
+                    if (!(fminf(r2.x, r2.y) >= dd_min_r2(a.dd_lim)) || !words) {
                         const double x = entries_f64(a, m, j, s_pos[q]);
                         s = float(x);
                         c = float(x - double(s));

@@ -176,7 +176,7 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
                 float r2min;
                 double v = dd_points_call(reinterpret_cast<const float *>(s_tile4), n4, c, &r2min);
                 // closer than the dd words resolve, or out of their range
-                if (!(r2min >= kDdMinR2) || !dd_in_range(c.h, a.dd_lim))
+                if (!(r2min >= dd_min_r2(a.dd_lim)) || !dd_in_range(c.h, a.dd_lim))
                     v = point_tile_f64(a.rec64 + m.off64, m.n, a.pos.x64[ic], a.pos.y64[ic], a.pos.z64[ic]);
                 acc64[q * NT] += v;
             }
