@@ -775,7 +775,8 @@ __global__ void __launch_bounds__(32 * SLICES) reduce_pairs_kernel(const double 
 // one warp per walker: its lanes' electrons by TwoSum, then the lanes in a fixed order
 __global__ void walker_kernel(const double *__restrict__ V, int n_walkers, int n_elec, double *__restrict__ E)
 {
-    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    // (blocks first: 32 n_walkers threads pass 2^32 from 2^27 walkers on)
+    const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (w >= n_walkers)
         return;
     double s = 0.0, c = 0.0;

@@ -1,0 +1,24 @@
+"""GPU: walker energies where a walker's thread index passes 32 bits (one warp per
+walker: from 2^27 walkers on)."""
+import numpy as np
+import pytest
+
+from paper_1011_4687_gb300 import build_lib, esp
+from workloads import PairList
+
+pytestmark = pytest.mark.gpu
+
+
+def test_walkers_beyond_2_27():
+    torch = pytest.importorskip("torch")
+    build_lib.build()
+    n = (1 << 27) + 5
+    with esp.Environment(np.array([[9.0, 0.0, 0.0]]), np.array([2.0]), PairList.empty(), precision="fp64") as env:
+        pos = torch.zeros((n, 3), dtype=torch.float64, device="cuda")
+        pos[:, 0] = torch.arange(n, device="cuda") % 1000 * 1e-3
+        E = torch.full((n,), float("nan"), dtype=torch.float64, device="cuda")
+        V = torch.empty(n, dtype=torch.float64, device="cuda")
+        env.eval_walkers(pos, n, 1, V_out=V, E_out=E)
+        torch.cuda.synchronize()
+        assert torch.equal(E, -V)
+        assert (V * (9.0 - pos[:, 0]) - 2.0).abs().max().item() <= 1e-14
