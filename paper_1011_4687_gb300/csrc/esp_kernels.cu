@@ -46,7 +46,8 @@ __global__ void stage_kernel(const double *__restrict__ pos, int n, double cx, d
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n)
         return;
-    double x = pos[3 * i] - cx, y = pos[3 * i + 1] - cy, z = pos[3 * i + 2] - cz;
+    const double *p = pos + 3 * (size_t)i; // (3 i passes 32 bits within the 2^30 positions of a call)
+    double x = p[0] - cx, y = p[1] - cy, z = p[2] - cz;
     const int j = slot_of ? slot_of[i] : i;
     stage_position(st, j, x, y, z, q);
 }
@@ -61,7 +62,8 @@ __global__ void stage_kernel(const double *__restrict__ pos, int n, double cx, d
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int sort_cell(const double *__restrict__ pos, int i, double cx, double cy, double cz)
 {
-    const double r[3] = {pos[3 * i] - cx, pos[3 * i + 1] - cy, pos[3 * i + 2] - cz};
+    const double *p = pos + 3 * (size_t)i;
+    const double r[3] = {p[0] - cx, p[1] - cy, p[2] - cz};
     int key = 0;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -202,7 +204,8 @@ __global__ void batch_stage_kernel(const BatchHeader *__restrict__ hdr, const Sy
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < total; g += gridDim.x * blockDim.x) {
         const SysDesc &d = sys[find_sys(sys, n_sys, g)];
         const int i = g - d.pos_begin;
-        double x = d.pos_in[3 * i] - d.qm[0], y = d.pos_in[3 * i + 1] - d.qm[1], z = d.pos_in[3 * i + 2] - d.qm[2];
+        const double *p = d.pos_in + 3 * (size_t)i;
+        double x = p[0] - d.qm[0], y = p[1] - d.qm[1], z = p[2] - d.qm[2];
         const int j = d.sorted ? d.slot_of[i] : i;
         stage_position(d.st, j, x, y, z, d.quantum);
     }
