@@ -241,7 +241,7 @@ cudaError_t launch_dd_sum(const EvalArgs &a, const int *list, int n_list, int n_
     if (a.n_pos <= 0 || n_list <= 0)
         return cudaSuccess;
     const size_t smem = (size_t)a.tile_size * kDdWordsMax * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(dd_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(dd_sum_kernel, (size_t)kMaxTileSize * kDdWordsMax * sizeof(float));
     if (e != cudaSuccess)
         return e;
     const dim3 grid((a.n_pos + kDdThreads - 1) / kDdThreads, n_splits);
@@ -270,7 +270,7 @@ cudaError_t launch_td(const EvalArgs &a, cudaStream_t s)
     if (a.n_pos <= 0)
         return cudaSuccess;
     const size_t smem = (size_t)a.tile_size * kTdWordsMax * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(potential_td_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(potential_td_kernel, (size_t)kMaxTileSize * kTdWordsMax * sizeof(float));
     if (e != cudaSuccess)
         return e;
     const dim3 grid((a.n_pos + kDdThreads - 1) / kDdThreads, a.n_splits);

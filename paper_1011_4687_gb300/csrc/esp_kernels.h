@@ -153,6 +153,15 @@ cudaError_t launch_sort(const double *pos_in, int n, const double center[3], int
 // precision: 0 = FP64, 1 = FP32C.  threads in {64, 128, 256}, ppt in {1, 2, 4}.
 cudaError_t launch_potential(int precision, const EvalArgs &a, int threads, int ppt, cudaStream_t s);
 size_t potential_smem_bytes(int precision, int tile_size);
+// A kernel's limit of dynamic shared memory belongs to the function, not to a
+// launch: set to what kMaxTileSize takes, the same from every thread.  (Set to
+// the calling context's own size, a thread with smaller tiles could lower it
+// between another thread's set and launch, which then failed.)
+constexpr int kMaxTileSize = 256;
+template <typename K> inline cudaError_t allow_smem(K kernel, size_t bytes)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
 // Launch shapes compiled into the library: FP64 threads {64,128,256} x ppt {1,2};
 // FP32C (64,{2,4}), (128,{1,2,4}), (256,{1,2}).
 bool potential_shape_supported(int precision, int threads, int ppt);

@@ -17,7 +17,7 @@ template <int NT, int PPT>
 cudaError_t launch_f32c_shape(const EvalArgs &a, dim3 grid, size_t smem, cudaStream_t s)
 {
     auto k = potential_f32c_kernel<NT, PPT>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, potential_smem_bytes(1, kMaxTileSize));
     if (e != cudaSuccess)
         return e;
     k<<<grid, NT, smem, s>>>(a);
@@ -30,7 +30,7 @@ template <int NT, int PPT>
 cudaError_t launch_f64_shape(const EvalArgs &a, dim3 grid, size_t smem, cudaStream_t s)
 {
     auto k = potential_f64_kernel<NT, PPT>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, potential_smem_bytes(0, kMaxTileSize));
     if (e != cudaSuccess)
         return e;
     k<<<grid, NT, smem, s>>>(a);
@@ -45,7 +45,7 @@ cudaError_t launch_batch_shape(const BatchHeader *hdr, const SysDesc *sys, const
                                cudaStream_t s)
 {
     auto k = batch_potential_kernel<NT, PPT, PREC>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, potential_smem_bytes(PREC, kMaxTileSize));
     if (e != cudaSuccess)
         return e;
     int per_sm = 0;
