@@ -90,8 +90,10 @@ typedef struct {
 } esp_gauss_pair;
 
 typedef enum {
-    ESP_FP64 = 0,  /* FP64 accuracy throughout: reference path (far entries of calls
-                      above 16 positions in exact FP32 words, the rest in FP64) */
+    ESP_FP64 = 0,  /* FP64 accuracy throughout: reference path.  Entries whose
+                      Gaussian is negligible at a position may be summed in three FP32
+                      numbers each (72 bits; in calls of few positions too), the rest
+                      in FP64 */
     ESP_FP32C = 1  /* bulk of the pair sum in FP32 with compensated accumulation;
                       point charges and near (position, tile) blocks in pairs of
                       FP32 numbers (48 bits) or FP64 */

@@ -28,8 +28,9 @@
 // padding repeats the last record's coordinates with zero coefficients):
 //   0..2 h(x, y, z)   3..5 m   6..8 l
 //   points:        9..11 Z (three words), 12 (Z - word 9) / word 9
-//   distributions: far block [9, 11 + 2 nh): the monopole's third word, p, then
-//                  the coefficients h, then l (nh = number of Hermite coefficients);
+//   distributions: far block [9, 10 + 3 nh): the monopole's third word, p, then the
+//                  coefficients h, then l, then the third words of those after the
+//                  monopole (nh = number of Hermite coefficients);
 //                  L <= 2, near-capable tiles: general block of 2 + 2 nh words: sqrt(p) h, l,
 //                  sqrt(pi)/2 G h, then l.
 #pragma once
@@ -59,7 +60,7 @@ constexpr float kDdMinR2 = 0x1p-20f;
 ESP_HD float dd_min_r2(float lim) { return fmaxf(kDdMinR2, (lim * 0x1p-15f) * (lim * 0x1p-15f)); }
 ESP_HD constexpr int dd_pad(int n) { return (n + 3) & ~3; }
 constexpr int kDdPointWords = 13;
-ESP_HD constexpr int dd_far_words(int L) { return 11 + 2 * num_hermite(L); }
+ESP_HD constexpr int dd_far_words(int L) { return 10 + 3 * num_hermite(L); }
 ESP_HD constexpr int dd_gen_words(int L) { return L <= kDdGeneralMaxL ? 2 + 2 * num_hermite(L) : 0; }
 // does a tile hold the general block (it can be near a position of an FP32C call)?
 ESP_HD bool dd_has_general(const TileMeta &m)
@@ -306,9 +307,11 @@ ESP_HD void dd_convert_dist(const double *r, bool shortr, bool general, float *o
         dd_project<3>(M + 10);
     if constexpr (L >= 4)
         dd_project<4>(M + 20);
-    for (int k = 0; k < nh; ++k)
-        dd_split2(M[k], out[(11 + k) * n4], out[(11 + nh + k) * n4]);
-    out[9 * n4] = float(M[0] - double(out[11 * n4]) - double(out[(11 + nh) * n4]));
+    for (int k = 0; k < nh; ++k) {
+        float &h = out[(11 + k) * n4], &l = out[(11 + nh + k) * n4];
+        dd_split2(M[k], h, l);
+        out[(k == 0 ? 9 : 10 + 2 * nh + k) * n4] = float(M[k] - double(h) - double(l));
+    }
     out[10 * n4] = float(r[3] * r[3]);
     if (L <= kDdGeneralMaxL && general) {
         constexpr int go = dd_far_words(L);
@@ -345,7 +348,7 @@ ESP_HD void dd_convert(const TileMeta &m, const double *r, double q, float *out,
 }
 
 // ---------------------------------------------------------------------------
-// The leading term at FP64 accuracy.  One rounding of a low word costs up to
+// The far form at FP64 accuracy.  One rounding of a low word costs up to
 // 2^-49 of the result, and the dd form above makes about fifteen of them
 // (3e-15 rms per term, against 1e-16 of FP64 arithmetic, which many-term sums
 // average but small ones show).  Here r^2 = a + b + c has a third word and the
@@ -355,6 +358,51 @@ ESP_HD void dd_convert(const TileMeta &m, const double *r, double q, float *out,
 struct Td {
     f2 a, b, c;
 };
+// Three words a + b + c that need not be normalised: |b| up to a few 2^-23 |a|,
+// c the rest in FP32.  A product or sum keeps every rounding of the first two
+// words, so its error is that of c: below 2^-60 of the operands' size.
+ESP_HD Td td_mul(const Td &x, const Td &y)
+{
+    f2 e, f, g, e1, e2;
+    const f2 p = two_prod(x.a, y.a, e), q = two_prod(x.a, y.b, f), r = two_prod(x.b, y.a, g);
+    f2 b = two_sum(q, r, e1);
+    b = two_sum(b, e, e2);
+    return {p, b, esp_fma(x.b, y.b, esp_fma(x.a, y.c, esp_fma(x.c, y.a, f + g))) + (e1 + e2)};
+}
+ESP_HD Td td_sqr(const Td &x)
+{
+    f2 e, f, e1;
+    const f2 p = two_prod(x.a, x.a, e), q = two_prod(x.a + x.a, x.b, f);
+    const f2 b = two_sum(q, e, e1);
+    return {p, b, esp_fma(x.b, x.b, esp_fma(x.a + x.a, x.c, f + e1))};
+}
+ESP_HD Td td_add(const Td &x, const Td &y)
+{
+    f2 e, e1, e2;
+    const f2 a = two_sum(x.a, y.a, e);
+    f2 b = two_sum(x.b, y.b, e1);
+    b = two_sum(b, e, e2);
+    return {a, b, (x.c + y.c) + (e1 + e2)};
+}
+// dd_form in three words
+template <int N, typename C>
+ESP_HD Td td_form(const Td &x, const Td &y, const Td &z, C c)
+{
+    if constexpr (N == 1) {
+        return td_add(td_add(td_mul(c(0), x), td_mul(c(1), y)), td_mul(c(2), z));
+    } else {
+        const Td v = td_mul(x, td_form<N - 1>(x, y, z, c));
+        constexpr int k0 = N * (N + 1) / 2;
+        Td w = td_add(td_mul(c(k0), y), td_mul(c(k0 + 1), z));
+        Td zk = z;
+#pragma unroll
+        for (int k = 2; k <= N; ++k) {
+            zk = k == 2 ? td_sqr(z) : td_mul(zk, z);
+            w = td_add(td_mul(w, y), td_mul(c(k0 + k), zk));
+        }
+        return td_add(v, w);
+    }
+}
 // offset in three words: s + e exactly h + m, l the rest
 struct TdOff {
     f2 s, e, l;
@@ -400,8 +448,8 @@ struct TdSum {
     f2 a, b, c;
     ESP_HD void clear() { a = b = c = f2(0.0f); }
     ESP_HD void mid(f2 x) { td_acc(b, c, x); }
-    // add z / sqrt(r2) for z = zh + zl + zm; returns 1 / sqrt(r2) to 48 bits
-    ESP_HD dd div_sqrt(f2 zh, f2 zl, f2 zm, const Td &r2)
+    // add z / sqrt(r2) for z = zh + zl + zm; returns 1 / sqrt(r2)
+    ESP_HD Td div_sqrt(f2 zh, f2 zl, f2 zm, const Td &r2)
     {
         const f2 y = esp_rsqrt(r2.a);
         f2 pe, qe, fe, ge, he, ze, ke, le, e;
@@ -427,14 +475,17 @@ struct TdSum {
         mid(ze);
         const f2 u = u1 + u2;
         c += esp_fma(v, u3, esp_fma(l + ze, u, esp_fma(zm, y, (he + ke) + le)));
-        return {y, y * (u + u3)};
+        f2 e1, e2, ye;
+        const f2 y1 = two_prod(y, u1, e1), y2 = two_prod(y, u2, e2), yb = two_sum(y1, y2, ye);
+        return {y, yb, esp_fma(y, u3, (e1 + e2) + ye)};
     }
-    ESP_HD void add(const dd &x)
+    ESP_HD void add(const Td &x)
     {
         f2 e;
-        a = two_sum(a, x.h, e);
+        a = two_sum(a, x.a, e);
         mid(e);
-        mid(x.l);
+        mid(x.b);
+        c += x.c;
     }
     ESP_HD double total() const
     {
@@ -489,9 +540,11 @@ ESP_HD dd dd_point(const DdTile &t, int j, const DdPos &c, f2 &r2)
     return dd_div_sqrt(t(9, j), t(12, j), s);
 }
 
-// Far form of distributions j, j + 1, the monopole at FP64 accuracy and the
-// higher orders (which fall off as (size / distance)^N) in 48 bits, added to
-// sum.  Lanes with use = 0 add nothing, whatever their offset; r2 receives
+// Far form of distributions j, j + 1 at FP64 accuracy, added to sum: every
+// order in three words.  (The orders above the monopole in 48 bits, as they
+// were, erred by up to 7e-15 of the terms, against 6e-16 of the FP64 code: they
+// fall off as (size / distance)^N, but a product of s and p on one centre, say,
+// has no monopole beside them.)  Lanes with use = 0 add nothing, whatever their offset; r2 receives
 // |P - C|^2 (1 for those).
 template <int L>
 ESP_HD void td_far(const DdTile &t, int j, const DdPos &c, bool use0, bool use1, TdSum &sum, f2 &r2)
@@ -507,35 +560,21 @@ ESP_HD void td_far(const DdTile &t, int j, const DdPos &c, bool use0, bool use1,
     s.c = f2(use0 ? s.c.x : 0.0f, use1 ? s.c.y : 0.0f);
     r2 = s.a;
     const f2 w(use0 ? 1.0f : 0.0f, use1 ? 1.0f : 0.0f);
-    const dd y = sum.div_sqrt(w * t(11, j), w * t(11 + nh, j), w * t(9, j), s);
+    const Td y = sum.div_sqrt(w * t(11, j), w * t(11 + nh, j), w * t(9, j), s);
     if constexpr (L > 0) {
-        auto coef = [&](int k) { return dd{t(11 + k, j), t(11 + nh + k, j)}; };
-        dd d[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-            d[k] = {o[k].s, o[k].e + o[k].l};
-        const dd i2 = dd_sqr(y);
-        dd a;
-        if constexpr (L == 1) {
-            a = dd_form<1>(d[0], d[1], d[2], [&](int k) { return coef(1 + k); });
-        } else {
-            dd b;
-            if constexpr (L == 2) {
-                b = dd_form<2>(d[0], d[1], d[2], [&](int k) { return coef(4 + k); });
-            } else {
-                dd g;
-                if constexpr (L == 3) {
-                    g = dd_form<3>(d[0], d[1], d[2], [&](int k) { return coef(10 + k); });
-                } else {
-                    const dd h = dd_form<4>(d[0], d[1], d[2], [&](int k) { return coef(20 + k); });
-                    g = dd_add(dd_form<3>(d[0], d[1], d[2], [&](int k) { return coef(10 + k); }), dd_mul(i2, h));
-                }
-                b = dd_add(dd_form<2>(d[0], d[1], d[2], [&](int k) { return coef(4 + k); }), dd_mul(i2, g));
-            }
-            a = dd_add(dd_form<1>(d[0], d[1], d[2], [&](int k) { return coef(1 + k); }), dd_mul(i2, b));
-        }
-        const dd v = dd_mul(dd_mul(i2, a), y);
-        sum.add(dd{w * v.h, w * v.l});
+        auto coef = [&](int k) { return Td{t(11 + k, j), t(11 + nh + k, j), t(10 + 2 * nh + k, j)}; };
+        const Td x = {o[0].s, o[0].e, o[0].l}, yy = {o[1].s, o[1].e, o[1].l}, z = {o[2].s, o[2].e, o[2].l};
+        const Td i2 = td_sqr(y);
+        // Horner's scheme in 1 / r^2 from the highest order down
+        Td v = td_form<L>(x, yy, z, [&](int k) { return coef(L * (L + 1) * (L + 2) / 6 + k); });
+        if constexpr (L >= 4)
+            v = td_add(td_form<3>(x, yy, z, [&](int k) { return coef(10 + k); }), td_mul(i2, v));
+        if constexpr (L >= 3)
+            v = td_add(td_form<2>(x, yy, z, [&](int k) { return coef(4 + k); }), td_mul(i2, v));
+        if constexpr (L >= 2)
+            v = td_add(td_form<1>(x, yy, z, [&](int k) { return coef(1 + k); }), td_mul(i2, v));
+        v = td_mul(td_mul(i2, y), v);
+        sum.add(Td{w * v.a, w * v.b, w * v.c});
     }
 }
 // Point charges j, j + 1 at FP64 accuracy.

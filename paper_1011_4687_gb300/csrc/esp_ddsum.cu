@@ -72,15 +72,15 @@ __global__ void __launch_bounds__(kDdThreads, 4) dd_sum_kernel(EvalArgs a, const
 
 // ---------------------------------------------------------------------------
 // FP64 evaluations.  Every entry whose Gaussian is negligible at a position
-// (T = p |P - C|^2 >= 45 and a margin) takes the far form of esp_dd.h: the
-// monopole in three FP32 words (an error of 1e-20 of the term), the higher
-// orders in two (about 200 packed FP32 operations per two monopoles).  The
-// others take the FP64 code, each lane its own entries: a warp runs as many as
-// its busiest lane has, not as many as any lane has (2,048 positions x 48,000
-// distributions 1.56 -> 1.52 ms, 9,000 x 24,000 3.42 -> 3.27).  Bound by the
-// FP64 pipe, where exponents are small (those entries: some 40 operations of 64
-// cycles; the pipe is 60 % busy, 90 % on the busiest SM), by FP32 otherwise.
-// All in FP64, 2,048 x 48,000 took 9.5 ms.
+// (T = p |P - C|^2 >= 45 and a margin) takes the far form of esp_dd.h in three
+// FP32 words: about 170 packed FP32 operations per two monopoles, 400 with L = 1
+// and 750 with L = 2.  (The orders above the monopole in two words were faster,
+// 2,048 positions x 48,000 distributions in 1.5 ms, but erred by 7e-15 and more
+// of an order that stands alone; in three 2.0 ms and 1e-16.)  The others take the
+// FP64 code, each lane its own entries: a warp runs as many as its busiest lane
+// has, not as many as any lane has (with two words 1.56 -> 1.52 ms).  Bound by the
+// FP64 pipe where exponents are small (those entries: some 40 operations of 64
+// cycles), by FP32 otherwise.  All in FP64, 2,048 x 48,000 took 9.5 ms.
 // ---------------------------------------------------------------------------
 constexpr int kTdWordsMax = dd_far_words(kMaxL);
 
