@@ -216,7 +216,7 @@ esp_status batch_eval(esp_batch *b, const double *const *positions, const int64_
         d.tiles = static_cast<const TileMeta *>(c->tiles.p);
         d.rec32 = static_cast<const float *>(c->rec32.p);
         d.rec64 = static_cast<const double *>(c->rec64.p);
-        d.recdd = static_cast<const float *>(c->recdd.p);
+        d.recdd = points_alone(c->full) ? nullptr : static_cast<const float *>(c->recdd.p);
         d.dd_lim = dd_limit(c);
         d.pos_in = positions[k];
         d.V_out = V_out[k];

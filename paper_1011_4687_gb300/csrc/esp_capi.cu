@@ -29,10 +29,6 @@ std::string &esp::last_error()
     return msg;
 }
 
-namespace {
-
-} // namespace
-
 int esp::choose_splits(const esp_ctx *c, const TileView &v, int n, int prec)
 {
     if (c->opt.pair_splits > 0)
@@ -56,7 +52,7 @@ int esp::choose_splits(const esp_ctx *c, const TileView &v, int n, int prec)
 
 int esp::view_precision(const esp_ctx *c, const TileView &v)
 {
-    return c->opt.precision == ESP_FP64 || (v.n_tiles > 0 && v.n_tiles == v.n_point_tiles) ? 0 : 1;
+    return c->opt.precision == ESP_FP64 || points_alone(v) ? 0 : 1;
 }
 
 bool esp::use_td(const esp_ctx *c, const TileView &v, int prec)

@@ -206,8 +206,10 @@ inline float near_radius(const esp_ctx *c)
 inline float dd_limit(const esp_ctx *c) { return float(0x1p23 * c->env.coord_quantum); }
 // per-split count for n positions in precision prec (0 FP64, 1 FP32C)
 int choose_splits(const esp_ctx *c, const TileView &v, int n, int prec);
-// Precision of an evaluation of the view (0 FP64, 1 FP32C): FP64 point charges
-// alone stay FP64 under FP32C, where no FP32 sum hides the 48 bits of a dd term.
+// FP64 point charges alone: they stay FP64 under FP32C, where no FP32 sum hides
+// the 48 bits of a dd term.
+inline bool points_alone(const TileView &v) { return v.n_tiles > 0 && v.n_tiles == v.n_point_tiles; }
+// Precision of an evaluation of the view (0 FP64, 1 FP32C).
 int view_precision(const esp_ctx *c, const TileView &v);
 // FP64 evaluations by launch_td: default launch shape, dd records, and enough
 // entries (kTdMinEntries) that its order of summation is no worse than FP64's.

@@ -82,7 +82,7 @@ struct SysDesc {
     const TileMeta *tiles;
     const float *rec32;
     const double *rec64;
-    const float *recdd;
+    const float *recdd;   // null: FP64 code in place of the dd sums
     float dd_lim;
     const double *pos_in; // [n_pos][3] device
     double *V_out;        // [n_pos] device

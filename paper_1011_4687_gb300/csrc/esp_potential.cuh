@@ -93,7 +93,7 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
             continue;
         __syncthreads(); // previous tile fully consumed
         const bool pts = ALL && m.cls == kClassPoint;
-        const bool ddt = m.offdd >= 0;
+        const bool ddt = a.recdd && m.offdd >= 0;
         const int n4 = dd_pad(m.n);
         const float4 *s_dd = reinterpret_cast<const float4 *>(a.recdd) + (ddt ? m.offdd : 0);
         const float4 *src = pts ? (ddt ? s_dd : reinterpret_cast<const float4 *>(a.rec64 + m.off64))

@@ -529,7 +529,7 @@ esp_status predict(esp_surrogate *s, const double *pos, int n, double *V, cudaSt
         cudaError_t e = cudaMemsetAsync(V, 0, size_t(n) * sizeof(double), st);
         if (e != cudaSuccess)
             return cuda_fail(e, "clearing surrogate values");
-    } else if ((r = eval_view(s->ctx, s->near_view, 1, pos, n, V)) != ESP_OK) {
+    } else if ((r = eval_view(s->ctx, s->near_view, points_alone(s->near_view) ? 0 : 1, pos, n, V)) != ESP_OK) {
         return r;
     }
     return far_approx(s, pos, n, V, true, st);
@@ -880,7 +880,7 @@ esp_status fallback_pass(esp_surrogate *s, const double *pos, int n, double *V, 
     *count_out = count;
     if (count == 0)
         return ESP_OK;
-    esp_status r = eval_view(s->ctx, s->ctx->full, 1, static_cast<const double *>(s->d_cpos.p), count,
+    esp_status r = eval_view(s->ctx, s->ctx->full, points_alone(s->ctx->full) ? 0 : 1, static_cast<const double *>(s->d_cpos.p), count,
                              static_cast<double *>(s->d_cV.p));
     if (r != ESP_OK)
         return r;
