@@ -65,7 +65,8 @@ int plan_ranges(const esp_ctx *c, double target, int *ranges)
     for (int g = 0; g < v.n_groups; ++g) {
         const int tiles = v.grp_tile[g + 1] - v.grp_tile[g];
         const double cost = tiles > 0 ? tiles * c->env.tile_size * group_cost(c->env.tiles[size_t(v.grp_tile[g])].cls) : 0.0;
-        ranges[g] = std::max(1, std::min(tiles, int(std::ceil(cost / target))));
+        // (in double: a system without positions has no part in the target)
+        ranges[g] = std::max(1, int(std::min(double(tiles), std::ceil(cost / target))));
         sum += ranges[g];
     }
     return sum;
