@@ -52,10 +52,12 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
                                          const float *s_boys, double *s_acc)
 {
     const int base = bx * NT * PPT + threadIdx.x;
-    // Only the FP32 sums live in registers from tile to tile.  The positions'
-    // words come from L1 again for each tile (24 loads beside the thousands of
-    // operations of a tile) and the FP64 sums, which few tiles add to, stay in
-    // shared memory: the far form's inner loop has those 30 registers more.
+    // The FP32 sums and the positions' words live in registers from tile to
+    // tile; the FP64 sums, which few tiles add to, stay in shared memory.  (The
+    // words from L1 again for each tile gave the far form's loops 24 registers
+    // and no spills, but cost more than they gave: the records stream through
+    // the same L1.  65,536 positions x 19.7 million distributions 1,297 ms
+    // against 1,274, 131,072 x 1.1 million 160.9 against 158.6.)
     auto pos_of = [&](int q) { return min(base + q * NT, a.n_pos - 1); };
     double *acc64 = s_acc + threadIdx.x; // [q * NT]
     float S[PPT], Cc[PPT];
@@ -73,6 +75,28 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
     for (int q = 0; q < NP; ++q) {
         S2[q] = f2(0.0f);
         C2[q] = f2(0.0f);
+    }
+    float ch[PPT][3], cl[PPT][3];
+#pragma unroll
+    for (int q = 0; q < PPT; ++q) {
+        const int ic = pos_of(q);
+        ch[q][0] = a.pos.xh[ic];
+        ch[q][1] = a.pos.yh[ic];
+        ch[q][2] = a.pos.zh[ic];
+        cl[q][0] = a.pos.xl[ic];
+        cl[q][1] = a.pos.yl[ic];
+        cl[q][2] = a.pos.zl[ic];
+    }
+    // the same positions as lane pairs
+    f2 ch2[NP][3], cl2[NP][3];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+        const int q0 = 2 * q < PPT ? 2 * q : 0, q1 = 2 * q + 1 < PPT ? 2 * q + 1 : 0;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            ch2[q][d] = f2(ch[q0][d], ch[q1][d]);
+            cl2[q][d] = f2(cl[q0][d], cl[q1][d]);
+        }
     }
     const float near_r = a.near_r;
     // this split's group and its place among the group's splits
@@ -104,28 +128,6 @@ __device__ __forceinline__ void cta_f32c(const EvalArgs &a, int bx, int split, f
         if (!ALL)
             asm volatile("cp.async.wait_all;" ::: "memory"); // the Boys table, once
         __syncthreads();
-        float ch[PPT][3], cl[PPT][3];
-#pragma unroll
-        for (int q = 0; q < PPT; ++q) {
-            const int ic = pos_of(q);
-            ch[q][0] = a.pos.xh[ic];
-            ch[q][1] = a.pos.yh[ic];
-            ch[q][2] = a.pos.zh[ic];
-            cl[q][0] = a.pos.xl[ic];
-            cl[q][1] = a.pos.yl[ic];
-            cl[q][2] = a.pos.zl[ic];
-        }
-        // the same positions as lane pairs
-        f2 ch2[NP][3], cl2[NP][3];
-#pragma unroll
-        for (int q = 0; q < NP; ++q) {
-            const int q0 = 2 * q < PPT ? 2 * q : 0, q1 = 2 * q + 1 < PPT ? 2 * q + 1 : 0;
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                ch2[q][d] = f2(ch[q0][d], ch[q1][d]);
-                cl2[q][d] = f2(cl[q0][d], cl[q1][d]);
-            }
-        }
         if (m.cls == kClassPoint32) {
             // small point charges: the far form of an L = 0 record, no near path
             const float *s_rec = reinterpret_cast<const float *>(s_tile4);
