@@ -498,7 +498,8 @@ esp_status esp_debug_solid_harmonics(int32_t L, const double *u, double *out);
 /* Test hook, not part of the evaluation path: evaluate a built context's
  * tiles on the host with the kernels' own per-tile code, in the context's
  * precision (ESP_FP64: FP64; ESP_FP32C: the FP32-compensated arithmetic of
- * the kernel, emulated in IEEE single precision), so CPU tests can check the
+ * the kernel, emulated in IEEE single precision, with point charges and near
+ * blocks in FP64), so CPU tests can check the
  * pair builder and the error budget of the FP32 path without a GPU.
  * positions and V_out are host arrays.  esp_eval never calls this. */
 esp_status esp_debug_host_eval(const esp_ctx *ctx, const double *positions, int64_t n,

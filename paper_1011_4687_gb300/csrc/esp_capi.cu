@@ -500,8 +500,9 @@ void release_all(esp_ctx *c)
         b->release();
 }
 
-// Host emulation of the FP32C kernel for one position (one split): the same
-// per-tile core, the same staging, near test and accumulation.
+// Host emulation of the FP32C evaluation for one position (one split): the
+// kernel's per-tile core, staging, near test and accumulation.  Point charges and
+// near blocks are FP64 here; the device sums them in 48 bits where it can.
 double host_eval_f32c(const esp_ctx *c, const double *C)
 {
     const float *boys32 = boys_table32().data();

@@ -39,7 +39,7 @@ constexpr double kDefaultPoint32Max = 0.25;
 ESP_HD constexpr bool is_point_class(int cls) { return cls == kClassPoint || cls == kClassPoint32; }
 // FP32 record stride of a tile class (point charges use the L = 0 layout)
 ESP_HD constexpr int rec32_stride_cls(int cls);
-// FP64 re-evaluation radius of the FP32C kernel when the caller leaves it unset.
+// Radius of the blocks that the FP32C kernel leaves to FP64 or 48-bit sums, when the caller leaves it unset.
 // It applies only to tiles holding a distribution whose potential can exceed
 // kNearVmax (|Q| 2 sqrt(p/pi) bounds the potential of a charge Q spread with
 // exponent p); nuclei and on-site monopoles are FP64 point charges already.

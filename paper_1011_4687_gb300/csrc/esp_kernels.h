@@ -52,9 +52,9 @@ struct EvalArgs {
     const float *recdd;   // dd records (TileMeta::offdd)
     const float *boysdd;  // Boys table of the dd general form
     float dd_lim;         // |coordinate| up to which the dd words of a position are exact
-    double *partial;  // [n_splits][n_pos], FP64
+    double *partial;  // [n_splits][n_pos], 8 bytes each
     int pairs;        // FP32C kernel: its partials as float2 (sum, compensation), in the same places
-    float near_r;     // FP32C: FP64 re-evaluation radius around a tile's bounding sphere
+    float near_r;     // FP32C: blocks closer than this to a tile's bounding sphere are left to the dd kernel
     // FP32C deal by tile group: group g holds tiles [grp_tile[g], grp_tile[g+1])
     // and takes the splits [grp_split[g], grp_split[g+1]) (grp_split[n_groups] =
     // n_splits), so each CTA runs the code of one class.  One group over all
@@ -145,7 +145,7 @@ constexpr int kSortCells = kSortSide * kSortSide * kSortSide;
 constexpr int kSortThreads = 1024;
 constexpr int kSortCtas = 8; // the cluster that orders one call's positions
 constexpr double kSortHalf = 8.0;
-constexpr int kSortMinPositions = 4096; // fewer: the order is not worth its three launches
+constexpr int kSortMinPositions = 4096; // fewer: the order is not worth its two launches
 constexpr int kSortMinTd = 512;        // FP64: compact warps have fewer near entries
 size_t sort_scratch_ints(int n);
 cudaError_t launch_sort(const double *pos_in, int n, const double center[3], int *scratch, int **slot_of, int **perm,

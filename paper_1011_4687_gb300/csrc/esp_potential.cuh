@@ -9,7 +9,7 @@
 // of distributions at a time in shared memory with coalesced 16-byte loads,
 // and every warp reads the tile's records as same-address broadcasts.  Tiles
 // are dealt round-robin to `n_splits` CTAs per position block; each split
-// writes its own FP64 partial, and a separate kernel sums the partials in a
+// writes its own partial, and a separate kernel sums the partials in a
 // fixed order (deterministic, no atomics on the result).
 //
 // Only esp_shape.cu instantiates these templates, once per launch shape and
