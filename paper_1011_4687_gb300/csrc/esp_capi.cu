@@ -18,6 +18,7 @@
 
 #include "../../include/esp.h"
 #include "esp_ctx.h"
+#include "esp_dd.h"
 #include "esp_eval_core.h"
 #include "esp_harmonics.h"
 
@@ -63,8 +64,8 @@ int esp::view_precision(const esp_ctx *c, const TileView &v)
 
 bool esp::use_td(const esp_ctx *c, const TileView &v, int prec)
 {
-    return prec == 0 && !v.labels && c->recdd.p && c->opt.threads_per_block == 0 && c->opt.positions_per_thread == 0 &&
-           c->opt.pair_splits == 0 && v.n_entries >= kTdMinEntries;
+    return prec == 0 && !v.labels && c->recdd.p && td_resolves(dd_limit(c)) && c->opt.threads_per_block == 0 &&
+           c->opt.positions_per_thread == 0 && c->opt.pair_splits == 0 && v.n_entries >= kTdMinEntries;
 }
 
 namespace {

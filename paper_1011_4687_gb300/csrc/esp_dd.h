@@ -41,23 +41,28 @@ namespace esp {
 
 constexpr int kDdGeneralMaxL = 2;         // larger L takes the FP64 code when not far
 // The words of an offset hold it to 2^-48 q, and its hi word alone (the
-// difference of two roundings to the grid q) is off by up to sqrt(3) q.  So the
-// words are used where offsets are at least 256 q long, which the coordinates of
-// the environment decide (q = 2^-24 times a power of two above 4 max |P|):
-//  - distributions: tiles with q sqrt(p) above kDdMaxQs keep the FP64 code, so
-//    that T = p |P - C|^2 >= 46 (kTdNearT) implies |P - C| >= 6.78 / sqrt(p) >= 271 q;
-//  - point charges: closer positions take the FP64 code (dd_min_r2), as do all
-//    closer than 2^-10 bohr;
-//  - environments with q above kDdMaxQuantum (beyond 16,384 bohr) have no dd
-//    records at all.  (That also keeps d^4 below 2^64: FP32's range.)
-constexpr double kDdMaxQuantum = 0x1p-8;
-constexpr double kDdMaxQs = 0.025;
+// difference of two roundings to the grid q) is off by up to sqrt(3) q; q, 2^-24
+// times a power of two above 4 max |P|, follows the farthest centre.  So words
+// are used where offsets are long enough, which distant charges decide:
+//  - at FP64 accuracy (three words): from 256 q on, so that the offset's error
+//    is below 2^-56 of it and T = p |P - C|^2 from hi words within 1.4 %; in
+//    environments with q up to kTdMaxQuantum (16,384 bohr), which also keeps d^4
+//    below 2^64 (FP32's range);
+//  - in 48 bits (beside FP32 sums): point charges from 4 q on, distributions of
+//    q sqrt(p) <= 1; with q up to kDdMaxQuantum (a million bohr).
+// The rest takes the FP64 code, as do point charges closer than 2^-10 bohr.
+constexpr double kDdMaxQuantum = 0x1p-2, kTdMaxQuantum = 0x1p-8;
 // T below which an entry is near (FP64): 45 where the asymptotic form holds to
-// 1e-20, and 2.2 % for T formed from the hi words (1.3 % at most from 256 q on)
+// 1e-20, and a margin for T from the hi words
 constexpr float kTdNearT = 46.0f;
 constexpr float kDdMinR2 = 0x1p-20f;
-// Smallest |P - C|^2 of a point charge in words; lim = 2^23 q (dd_limit).  At most 1.
-ESP_HD float dd_min_r2(float lim) { return fmaxf(kDdMinR2, (lim * 0x1p-15f) * (lim * 0x1p-15f)); }
+// Smallest |P - C|^2 in words; lim = 2^23 q (dd_limit).  At most 1.
+ESP_HD float dd_min_r2(float lim) { return fmaxf(kDdMinR2, (lim * 0x1p-21f) * (lim * 0x1p-21f)); }
+ESP_HD float td_min_r2(float lim) { return fmaxf(kDdMinR2, (lim * 0x1p-15f) * (lim * 0x1p-15f)); }
+// three words at all (by 2^23 q)
+ESP_HD bool td_resolves(float lim) { return lim <= float(0x1p23 * kTdMaxQuantum); }
+// Is an entry far, by T and |P - C|^2 from hi words?
+ESP_HD bool td_is_far(float T, float r2, float min_r2) { return T >= kTdNearT && r2 >= 1.03f * min_r2; }
 ESP_HD constexpr int dd_pad(int n) { return (n + 3) & ~3; }
 constexpr int kDdPointWords = 13;
 ESP_HD constexpr int dd_far_words(int L) { return 10 + 3 * num_hermite(L); }

@@ -145,6 +145,7 @@ __global__ void __launch_bounds__(kDdThreads, 4) potential_td_kernel(EvalArgs a)
     const DdPos c = dd_position(a.pos, ic);
     const double x = a.pos.x64[ic], y = a.pos.y64[ic], z = a.pos.z64[ic];
     const bool in_range = dd_in_range(c.h, a.dd_lim);
+    const float min_r2 = td_min_r2(a.dd_lim);
     double S = 0.0, Cc = 0.0;
     const int shift = a.grp_shift[0], part = a.tile_size >> shift;
     for (int k = blockIdx.y; k < a.n_tiles << shift; k += gridDim.y) {
@@ -172,7 +173,7 @@ __global__ void __launch_bounds__(kDdThreads, 4) potential_td_kernel(EvalArgs a)
         } else {
             const float ex = c.h[0] - m.cx, ey = c.h[1] - m.cy, ez = c.h[2] - m.cz;
             const float d = sqrtf(ex * ex + ey * ey + ez * ez) - m.rad;
-            const bool far = __all_sync(0xffffffffu, d > 0.0f && m.pmin * d * d >= kTdNearT);
+            const bool far = __all_sync(0xffffffffu, d > 0.0f && td_is_far(m.pmin * d * d, d * d, min_r2));
             const DdTile t = {s_rec, n4};
             for (int j0 = 0; j0 < n4; j0 += 64) {
                 const int j1 = min(n4, j0 + 64);
@@ -180,8 +181,9 @@ __global__ void __launch_bounds__(kDdThreads, 4) potential_td_kernel(EvalArgs a)
                 if (!far) { // which records are near this lane's position
                     for (int j = j0; j < j1; j += 2) {
                         const f2 dx = t(0, j) - f2(c.h[0]), dy = t(1, j) - f2(c.h[1]), dz = t(2, j) - f2(c.h[2]);
-                        const f2 T = t(10, j) * esp_fma(dx, dx, esp_fma(dy, dy, dz * dz));
-                        near |= (unsigned long long)((T.x >= kTdNearT ? 0u : 1u) | (T.y >= kTdNearT ? 0u : 2u))
+                        const f2 r2 = esp_fma(dx, dx, esp_fma(dy, dy, dz * dz)), T = t(10, j) * r2;
+                        near |= (unsigned long long)((td_is_far(T.x, r2.x, min_r2) ? 0u : 1u) |
+                                                     (td_is_far(T.y, r2.y, min_r2) ? 0u : 2u))
                                 << (j - j0);
                     }
                 }
@@ -200,7 +202,7 @@ __global__ void __launch_bounds__(kDdThreads, 4) potential_td_kernel(EvalArgs a)
             }
         }
         // closer than the words resolve, or out of their range
-        if (!(r2min >= dd_min_r2(a.dd_lim)) || !in_range)
+        if (!(r2min >= min_r2) || !in_range)
             v = pts ? point_tile_f64(rec64, n, x, y, z) : tile_f64_one_any(m.cls, rec64, n, x, y, z, a.boys64);
         two_sum_acc(S, Cc, v);
     }

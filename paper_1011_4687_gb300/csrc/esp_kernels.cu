@@ -370,6 +370,7 @@ __device__ __forceinline__ double entries_words(const SmallArgs &a, const TileMe
     const int n4 = dd_pad(m.n);
     const DdTile t = {a.recdd + (size_t)m.offdd * 4, n4};
     const bool mine = j < m.n;
+    const float min_r2 = td_min_r2(a.dd_lim);
     double v = 0.0;
     float r2min = 1.0f;
     n0 = n1 = false;
@@ -378,9 +379,9 @@ __device__ __forceinline__ double entries_words(const SmallArgs &a, const TileMe
             v = point_pair(t, j, c, &r2min);
     } else if (mine) {
         const f2 dx = t(0, j) - f2(c.h[0]), dy = t(1, j) - f2(c.h[1]), dz = t(2, j) - f2(c.h[2]);
-        const f2 T = t(10, j) * esp_fma(dx, dx, esp_fma(dy, dy, dz * dz));
-        n0 = !(T.x >= kTdNearT);
-        n1 = !(T.y >= kTdNearT);
+        const f2 s = esp_fma(dx, dx, esp_fma(dy, dy, dz * dz)), T = t(10, j) * s;
+        n0 = !td_is_far(T.x, s.x, min_r2);
+        n1 = !td_is_far(T.y, s.y, min_r2);
         switch (m.cls & 7) {
         case 0: v = far_pair<0>(t, j, c, !n0, !n1, &r2min); break;
         case 1: v = far_pair<1>(t, j, c, !n0, !n1, &r2min); break;
@@ -389,7 +390,7 @@ __device__ __forceinline__ double entries_words(const SmallArgs &a, const TileMe
         default: v = far_pair<4>(t, j, c, !n0, !n1, &r2min); break;
         }
     }
-    if (!(r2min >= dd_min_r2(a.dd_lim))) { // closer than the words resolve
+    if (!(r2min >= min_r2)) { // closer than the words resolve
         v = 0.0;
         n0 = n1 = true;
     }
@@ -552,7 +553,7 @@ __global__ void __launch_bounds__(kSmallThreads, NQ <= 4 ? 2 : 1) small_n_kernel
             } else {
                 double v = 0.0;
                 bool n0 = j < m.n, n1 = j + 1 < m.n;
-                if (words)
+                if (words && td_resolves(a.dd_lim))
                     v = entries_words(a, m, j, s_dd[q], n0, n1);
                 // near entries: an FP64 operation takes its 64 cycles whatever
                 // the number of lanes, so few of them wait in the warp's list

@@ -308,7 +308,7 @@ namespace {
 void plan_dd(HostEnv &env)
 {
     const double small = 0x1p-60;
-    const bool ok_coord = env.coord_quantum <= kDdMaxQuantum; // offsets below 2^16, fourth powers below 2^64
+    const bool ok_coord = env.coord_quantum <= kDdMaxQuantum;
     for (TileMeta &m : env.tiles) {
         m.offdd = -1;
         const bool pts = is_point_class(m.cls);
@@ -324,7 +324,7 @@ void plan_dd(HostEnv &env)
         if (!pts) // far-field moments: G sqrt(pi)/2 p^{-(N + 1)/2}
             cmax *= std::max(1.0, std::pow(double(m.pmin), -0.5 * ((m.cls & 7) + 1)));
         if (!ok_coord || !(cmax > small) || !(cmax < (pts ? 0x1p+60 : 0x1p+50)) ||
-            (!pts && !(m.pmin > float(small * small) && smax < 0x1p+30 && smax * env.coord_quantum <= kDdMaxQs)))
+            (!pts && !(m.pmin > float(small * small) && smax < 0x1p+30 && smax * env.coord_quantum <= 1.0)))
             continue;
         m.offdd = int32_t(env.dd_floats / 4);
         env.dd_floats += int64_t(dd_words(m)) * dd_pad(m.n);

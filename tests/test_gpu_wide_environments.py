@@ -73,3 +73,21 @@ def test_close_to_point_charges(far, n):
     d = rng.normal(size=(n, 3))
     d *= (np.exp(rng.uniform(np.log(2e-4), 0.0, size=n)) / np.linalg.norm(d, axis=1))[:, None]
     check(xyz, Z, PairList.empty(), xyz[rng.integers(0, 7000, size=n)] + d, "fp64")
+
+
+@pytest.mark.parametrize("far", [1e3, 3e4, 1e5, 5e5, 1e7])
+def test_points_and_near_blocks_beside_fp32_sums(far):
+    """FP32C: charges and near blocks (every tile: near_radius beyond the environment)
+    keep 48 bits, 1e-11 of the absolute terms with three digits to spare."""
+    rng = np.random.default_rng(34)
+    C = rng.uniform(-6.0, 6.0, size=(700, 3))
+    p = np.linspace(6.0, 80.0, 700)
+    pairs = s_charge_pairs(C, p, np.full(700, -1.5))
+    xyz, Z = with_field(rng.uniform(-6.0, 6.0, size=(70, 3)), rng.choice([1.0, 6.0, -7.0], size=70), far)
+    d = rng.normal(size=(200, 3))
+    d *= (np.exp(rng.uniform(np.log(2e-4), 0.0, size=200)) / np.linalg.norm(d, axis=1))[:, None]
+    pos = np.concatenate([xyz[rng.integers(0, 70, size=200)] + d, at_T(rng, C, p, 100)])
+    ref = oracle.potential(xyz, Z, pairs, pos)
+    kappa = oracle.abs_terms(xyz, Z, pairs, pos)
+    with esp.Environment(xyz, Z, pairs, near_radius=1e3) as env:
+        assert np.all(np.abs(env.eval(pos) - ref) <= 1e-11 * kappa)
