@@ -477,7 +477,7 @@ def latency_leg(args, esp, torch, stream, oracle_mod=None):
     move is one position): microseconds per call on the device (CUDA events,
     device buffers), replayed as a captured graph, and through host buffers
     (wall clock, copies included).  Cells are summed in compensated FP32,
-    nuclei in FP64."""
+    nuclei in pairs of FP32 numbers (48 bits)."""
     from workloads import point_cells_environment
     wl = point_cells_environment(seed=1011 * 100 + 6, n_cells=268782, n_nuclei=36, n_positions=128)
     env = esp.Environment(wl.nuclei_xyz, wl.nuclei_Z, wl.pairs, precision="fp32c", stream=stream.cuda_stream)
