@@ -176,6 +176,7 @@ SmallArgs esp::small_args(const esp_ctx *c, const TileView &v, int prec, const d
     a.n_skip = a.n_p32 > 0 ? v.n_p32_tiles : 0;
     a.skip_begin = v.p32_tile;
     a.n_other = v.n_tiles - a.n_skip;
+    a.dist = v.n_tiles > v.n_point_tiles + v.n_p32_tiles;
     a.tile_parts = (c->env.tile_size + 63) / 64;
     a.points_dd = a.n_p32 > 0 && v.points_have_dd;
     a.any64 = v.n_tiles > a.n_skip + (a.points_dd ? v.n_point_tiles : 0);

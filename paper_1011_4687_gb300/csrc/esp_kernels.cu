@@ -320,9 +320,10 @@ __device__ __forceinline__ int small_owner(int lane)
 
 // one entry of a tile at one position, FP64
 // (a call: its registers would spill those of the FP32 pass)
+template <bool DIST>
 __device__ __noinline__ double entry_f64(const SmallArgs &a, const TileMeta &m, int j, const double *p)
 {
-    if (is_point_class(m.cls)) {
+    if (!DIST || is_point_class(m.cls)) {
         const double *r = a.rec64 + m.off64 + (size_t)j * kPointStride64;
         const double dx = r[0] - p[0], dy = r[1] - p[1], dz = r[2] - p[2];
         return r[3] * esp_rsqrt(dx * dx + dy * dy + dz * dz);
@@ -331,13 +332,14 @@ __device__ __noinline__ double entry_f64(const SmallArgs &a, const TileMeta &m, 
                             a.boys64);
 }
 // entries j, j + 1 where they exist
+template <bool DIST>
 __device__ __forceinline__ double entries_f64(const SmallArgs &a, const TileMeta &m, int j, const double *p)
 {
     double v = 0.0;
     if (j < m.n)
-        v = entry_f64(a, m, j, p);
+        v = entry_f64<DIST>(a, m, j, p);
     if (j + 1 < m.n)
-        v += entry_f64(a, m, j + 1, p);
+        v += entry_f64<DIST>(a, m, j + 1, p);
     return v;
 }
 
@@ -364,6 +366,7 @@ __device__ __noinline__ double point_pair(const DdTile t, int j, const DdPos &c,
     return sum.total();
 }
 // n0, n1: entries left to FP64.
+template <bool DIST>
 __device__ __forceinline__ double entries_words(const SmallArgs &a, const TileMeta &m, int j, const DdPos &c,
                                                 bool &n0, bool &n1)
 {
@@ -374,20 +377,22 @@ __device__ __forceinline__ double entries_words(const SmallArgs &a, const TileMe
     double v = 0.0;
     float r2min = 1.0f;
     n0 = n1 = false;
-    if (is_point_class(m.cls)) {
+    if (!DIST || is_point_class(m.cls)) {
         if (mine)
             v = point_pair(t, j, c, &r2min);
-    } else if (mine) {
-        const f2 dx = t(0, j) - f2(c.h[0]), dy = t(1, j) - f2(c.h[1]), dz = t(2, j) - f2(c.h[2]);
-        const f2 s = esp_fma(dx, dx, esp_fma(dy, dy, dz * dz)), T = t(10, j) * s;
-        n0 = !td_is_far(T.x, s.x, min_r2);
-        n1 = !td_is_far(T.y, s.y, min_r2);
-        switch (m.cls & 7) {
-        case 0: v = far_pair<0>(t, j, c, !n0, !n1, &r2min); break;
-        case 1: v = far_pair<1>(t, j, c, !n0, !n1, &r2min); break;
-        case 2: v = far_pair<2>(t, j, c, !n0, !n1, &r2min); break;
-        case 3: v = far_pair<3>(t, j, c, !n0, !n1, &r2min); break;
-        default: v = far_pair<4>(t, j, c, !n0, !n1, &r2min); break;
+    } else if constexpr (DIST) {
+        if (mine) {
+            const f2 dx = t(0, j) - f2(c.h[0]), dy = t(1, j) - f2(c.h[1]), dz = t(2, j) - f2(c.h[2]);
+            const f2 s = esp_fma(dx, dx, esp_fma(dy, dy, dz * dz)), T = t(10, j) * s;
+            n0 = !td_is_far(T.x, s.x, min_r2);
+            n1 = !td_is_far(T.y, s.y, min_r2);
+            switch (m.cls & 7) {
+            case 0: v = far_pair<0>(t, j, c, !n0, !n1, &r2min); break;
+            case 1: v = far_pair<1>(t, j, c, !n0, !n1, &r2min); break;
+            case 2: v = far_pair<2>(t, j, c, !n0, !n1, &r2min); break;
+            case 3: v = far_pair<3>(t, j, c, !n0, !n1, &r2min); break;
+            default: v = far_pair<4>(t, j, c, !n0, !n1, &r2min); break;
+            }
         }
     }
     if (!(r2min >= min_r2)) { // closer than the words resolve
@@ -428,8 +433,12 @@ struct P32Entry {
     }
 };
 
-template <int NQ>
-__global__ void __launch_bounds__(kSmallThreads, NQ <= 4 ? 2 : 1) small_n_kernel(SmallArgs a, double *__restrict__ V)
+// DIST: the view holds distributions.  Kernels for point charges alone go without
+// their code: in 64 registers (two CTAs per SM at up to four positions) its calls
+// made every thread spill (60,000 cells at two positions 8.2 us without, 10.1 with).
+template <int NQ, bool DIST>
+__global__ void __launch_bounds__(kSmallThreads, NQ <= 4 && !DIST ? 2 : 1)
+    small_n_kernel(SmallArgs a, double *__restrict__ V)
 {
     // grid: x = slice of the environment's entries, y = chunk of positions
     __shared__ double s_pos[NQ][3];
@@ -521,7 +530,7 @@ __global__ void __launch_bounds__(kSmallThreads, NQ <= 4 ? 2 : 1) small_n_kernel
             const int j = a.direct ? (u % a.tile_parts) * 32 + lane : (u % a.tile_parts) * 64 + 2 * lane;
             const bool words = m.offdd >= 0 && dd_in_range(s_dd[q].h, a.dd_lim);
             if (a.direct) { // (FP64 throughout)
-                double v = j < m.n ? entry_f64(a, m, j, s_pos[q]) : 0.0;
+                double v = j < m.n ? entry_f64<DIST>(a, m, j, s_pos[q]) : 0.0;
 #pragma unroll
                 for (int w = 16; w > 0; w >>= 1)
                     v += __shfl_xor_sync(0xffffffffu, v, w);
@@ -537,7 +546,7 @@ __global__ void __launch_bounds__(kSmallThreads, NQ <= 4 ? 2 : 1) small_n_kernel
                     s = v.h.x, c = v.l.x;
                     two_sum_pair(s, c, v.h.y, v.l.y); // (a padding charge is zero)
                     if (!(fminf(r2.x, r2.y) >= dd_min_r2(a.dd_lim)) || !words) {
-                        const double x = entries_f64(a, m, j, s_pos[q]);
+                        const double x = entries_f64<DIST>(a, m, j, s_pos[q]);
                         s = float(x);
                         c = float(x - double(s));
                     }
@@ -554,7 +563,7 @@ __global__ void __launch_bounds__(kSmallThreads, NQ <= 4 ? 2 : 1) small_n_kernel
                 double v = 0.0;
                 bool n0 = j < m.n, n1 = j + 1 < m.n;
                 if (words && td_resolves(a.dd_lim))
-                    v = entries_words(a, m, j, s_dd[q], n0, n1);
+                    v = entries_words<DIST>(a, m, j, s_dd[q], n0, n1);
                 // near entries: an FP64 operation takes its 64 cycles whatever
                 // the number of lanes, so few of them wait in the warp's list
                 const unsigned b0 = __ballot_sync(0xffffffffu, n0), b1 = __ballot_sync(0xffffffffu, n1);
@@ -568,9 +577,9 @@ __global__ void __launch_bounds__(kSmallThreads, NQ <= 4 ? 2 : 1) small_n_kernel
                     listed += cnt;
                 } else {
                     if (n0)
-                        v += entry_f64(a, m, j, s_pos[q]);
+                        v += entry_f64<DIST>(a, m, j, s_pos[q]);
                     if (n1)
-                        v += entry_f64(a, m, j + 1, s_pos[q]);
+                        v += entry_f64<DIST>(a, m, j + 1, s_pos[q]);
                 }
 #pragma unroll
                 for (int w = 16; w > 0; w >>= 1)
@@ -593,7 +602,7 @@ __global__ void __launch_bounds__(kSmallThreads, NQ <= 4 ? 2 : 1) small_n_kernel
                 i -= s_listed[w++];
             const int2 x = s_list[w][i];
             const TileMeta m = a.tiles[x.x];
-            s_val[k] = entry_f64(a, m, x.y / kSmallChunk, s_pos[x.y % kSmallChunk]);
+            s_val[k] = entry_f64<DIST>(a, m, x.y / kSmallChunk, s_pos[x.y % kSmallChunk]);
             s_own[k] = (unsigned char)(x.y % kSmallChunk);
         }
         __syncthreads();
@@ -945,12 +954,18 @@ cudaError_t launch_small_n(SmallArgs a, void *scratch, int num_sms, double *V, c
         grid.x = std::max(int(grid.x), std::min(a.n_other * a.tile_parts, num_sms / chunks));
     a.part64 = static_cast<double *>(scratch);
     a.part32 = reinterpret_cast<float2 *>(a.part64 + (size_t)grid.x * grid.y * nq);
+#define ESP_SMALL(NQ)                                                  \
+    if (a.dist)                                                        \
+        small_n_kernel<NQ, true><<<grid, kSmallThreads, 0, s>>>(a, V); \
+    else                                                               \
+        small_n_kernel<NQ, false><<<grid, kSmallThreads, 0, s>>>(a, V)
     switch (nq) {
-    case 2: small_n_kernel<2><<<grid, kSmallThreads, 0, s>>>(a, V); break;
-    case 4: small_n_kernel<4><<<grid, kSmallThreads, 0, s>>>(a, V); break;
-    case 8: small_n_kernel<8><<<grid, kSmallThreads, 0, s>>>(a, V); break;
-    default: small_n_kernel<16><<<grid, kSmallThreads, 0, s>>>(a, V); break;
+    case 2: ESP_SMALL(2); break;
+    case 4: ESP_SMALL(4); break;
+    case 8: ESP_SMALL(8); break;
+    default: ESP_SMALL(16); break;
     }
+#undef ESP_SMALL
     return cudaGetLastError();
 }
 

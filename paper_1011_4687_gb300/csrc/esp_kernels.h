@@ -198,6 +198,7 @@ struct SmallArgs {
     // skip_begin on, o + n_skip, in tile_parts parts of 64 entries each
     int n_other, skip_begin, n_skip, tile_parts;
     int direct; // all of them in FP64, in parts of 32 entries
+    int dist;   // some of them are distributions
     int *counters;         // [kSmallMaxChunks], zero before and after every launch
     // set by launch_small_n
     int g_threads;
