@@ -183,10 +183,10 @@ SmallArgs esp::small_args(const esp_ctx *c, const TileView &v, int prec, const d
     a.counters = counters;
     // Few (entry, position) pairs: latency counts, and the words of the far
     // entries with the list of the near ones are two chains where FP64 is one.
-    // us with words / direct, positions x primitive products: 1 x 2,400 35 / 23,
-    // 1 x 96,000 31 / 25, 8 x 9,600 39 / 35, 8 x 24,000 39 / 41, 2 x 96,000
-    // 33 / 33, 16 x 96,000 74 / 155.
-    if (a.any64 && int64_t(a.n_other) * c->env.tile_size * n <= 100000) {
+    // us with words / direct, positions x primitive products: 1 x 2,400 35 / 21,
+    // 1 x 96,000 31 / 25, 2 x 96,000 (113,800 by this count) 36 / 29, 16 x 96,000
+    // 81 / 155; 4 x 96,000 in words 37.
+    if (a.any64 && int64_t(a.n_other) * c->env.tile_size * n <= 150000) {
         a.direct = 1;
         a.tile_parts = c->env.tile_size / 32;
     }

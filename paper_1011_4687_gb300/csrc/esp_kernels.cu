@@ -433,14 +433,19 @@ struct P32Entry {
     }
 };
 
-// DIST: the view holds distributions.  Kernels for point charges alone go without
-// their code: in 64 registers (two CTAs per SM at up to four positions) its calls
-// made every thread spill (60,000 cells at two positions 8.2 us without, 10.1 with).
-template <int NQ, bool DIST>
-__global__ void __launch_bounds__(kSmallThreads, NQ <= 4 && !DIST ? 2 : 1)
+// What a kernel holds besides the FP32 point charges: point charges alone;
+// distributions, all of them in FP64 (direct); distributions in words.  Up to four
+// positions take 64 registers and two CTAs per SM; the words' code, whose calls made
+// every thread spill there (a stack of 424 bytes), takes 128 and one (1 x 96,000
+// products and their FP32 points: 31 us with the words' code aboard, 27 direct).
+enum SmallMode { kSmallPoints, kSmallDirect, kSmallWords };
+constexpr int small_ctas(int nq, int mode) { return nq <= 4 && mode != kSmallWords ? 2 : 1; }
+template <int NQ, int MODE>
+__global__ void __launch_bounds__(kSmallThreads, small_ctas(NQ, MODE))
     small_n_kernel(SmallArgs a, double *__restrict__ V)
 {
     // grid: x = slice of the environment's entries, y = chunk of positions
+    constexpr bool DIST = MODE != kSmallPoints;
     __shared__ double s_pos[NQ][3];
     __shared__ DdPos s_dd[NQ];
     __shared__ __align__(16) float s_pair[NQ / 2 > 0 ? NQ / 2 : 1][12]; // lanes' hi x y z, lo x y z of position pairs
@@ -529,7 +534,7 @@ __global__ void __launch_bounds__(kSmallThreads, NQ <= 4 && !DIST ? 2 : 1)
             const TileMeta m = a.tiles[tile];
             const int j = a.direct ? (u % a.tile_parts) * 32 + lane : (u % a.tile_parts) * 64 + 2 * lane;
             const bool words = m.offdd >= 0 && dd_in_range(s_dd[q].h, a.dd_lim);
-            if (a.direct) { // (FP64 throughout)
+            if (MODE == kSmallDirect || (MODE == kSmallPoints && a.direct)) { // (FP64 throughout)
                 double v = j < m.n ? entry_f64<DIST>(a, m, j, s_pos[q]) : 0.0;
 #pragma unroll
                 for (int w = 16; w > 0; w >>= 1)
@@ -562,8 +567,9 @@ __global__ void __launch_bounds__(kSmallThreads, NQ <= 4 && !DIST ? 2 : 1)
             } else {
                 double v = 0.0;
                 bool n0 = j < m.n, n1 = j + 1 < m.n;
-                if (words && td_resolves(a.dd_lim))
-                    v = entries_words<DIST>(a, m, j, s_dd[q], n0, n1);
+                if constexpr (MODE != kSmallDirect)
+                    if (words && td_resolves(a.dd_lim))
+                        v = entries_words<DIST>(a, m, j, s_dd[q], n0, n1);
                 // near entries: an FP64 operation takes its 64 cycles whatever
                 // the number of lanes, so few of them wait in the warp's list
                 const unsigned b0 = __ballot_sync(0xffffffffu, n0), b1 = __ballot_sync(0xffffffffu, n1);
@@ -949,16 +955,23 @@ cudaError_t launch_small_n(SmallArgs a, void *scratch, int num_sms, double *V, c
     a.g_threads = small_n_threads(a.n_tiles, num_sms, a.n_pos);
     const int nq = small_nq(a.n_pos);
     const int chunks = (a.n_pos + kSmallChunk - 1) / kSmallChunk;
+    const int mode = !a.dist ? kSmallPoints : a.direct ? kSmallDirect : kSmallWords;
+    // one CTA per SM, where each thread has one FP32 entry at most all the same
+    const int per_wave = num_sms / chunks * kSmallThreads;
+    if (mode == kSmallWords && a.n_p32 <= per_wave)
+        a.g_threads = std::min(a.g_threads, per_wave);
     dim3 grid(small_grid(a.g_threads, num_sms, chunks, a.n_p32 > 0), chunks);
     if (a.direct) // latency counts: a part per CTA
         grid.x = std::max(int(grid.x), std::min(a.n_other * a.tile_parts, num_sms / chunks));
     a.part64 = static_cast<double *>(scratch);
     a.part32 = reinterpret_cast<float2 *>(a.part64 + (size_t)grid.x * grid.y * nq);
-#define ESP_SMALL(NQ)                                                  \
-    if (a.dist)                                                        \
-        small_n_kernel<NQ, true><<<grid, kSmallThreads, 0, s>>>(a, V); \
-    else                                                               \
-        small_n_kernel<NQ, false><<<grid, kSmallThreads, 0, s>>>(a, V)
+#define ESP_SMALL(NQ)                                                           \
+    if (mode == kSmallWords)                                                    \
+        small_n_kernel<NQ, kSmallWords><<<grid, kSmallThreads, 0, s>>>(a, V);   \
+    else if (mode == kSmallDirect)                                              \
+        small_n_kernel<NQ, kSmallDirect><<<grid, kSmallThreads, 0, s>>>(a, V);  \
+    else                                                                        \
+        small_n_kernel<NQ, kSmallPoints><<<grid, kSmallThreads, 0, s>>>(a, V)
     switch (nq) {
     case 2: ESP_SMALL(2); break;
     case 4: ESP_SMALL(4); break;
